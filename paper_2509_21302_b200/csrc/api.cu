@@ -407,8 +407,7 @@ int qvggt_calibrate_smooth(const void *X_calib_bf16, int Mc, const void *W_bf16,
     if (!device_is_sm100()) return QVGGT_ERR_UNSUPPORTED;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     cudaError_t e = cudaMemsetAsync(colmax_scratch, 0, sizeof(float) * 2 * K, st);
-    if (e == cudaSuccess) e = qvggt_launch_colmax(X_calib_bf16, Mc, K, colmax_scratch, st);
-    if (e == cudaSuccess) e = qvggt_launch_colmax(W_bf16, N, K, colmax_scratch + K, st);
+    if (e == cudaSuccess) e = qvggt_launch_colmax(X_calib_bf16, Mc, W_bf16, N, K, colmax_scratch, colmax_scratch + K, st);
     if (e == cudaSuccess) e = qvggt_launch_smooth_finalize(colmax_scratch, colmax_scratch + K, K, alpha, lo, hi, smooth_c, st);
     return e == cudaSuccess ? QVGGT_OK : QVGGT_ERR_CUDA;
 }

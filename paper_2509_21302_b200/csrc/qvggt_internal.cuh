@@ -43,7 +43,8 @@ cudaError_t qvggt_launch_ln_rsq_c8(const void *X, long long ldx, int M, int K, c
 cudaError_t qvggt_launch_gelu_rsq_c8(const void *X, long long ldx, int M, int K, const float *mul, int bits, signed char *Xq8,
                                      float *scales, void *gelu_out, cudaStream_t st);
 cudaError_t qvggt_launch_max_reduce(const float *in, int n, float *out, cudaStream_t st);
-cudaError_t qvggt_launch_colmax(const void *X, int M, int K, float *colmax, cudaStream_t st);
+// column maxima of the rotated rows of A and of B (rows >= 1 each), into zeroed max_a, max_b [K]
+cudaError_t qvggt_launch_colmax(const void *A, int rows_a, const void *B, int rows_b, int K, float *max_a, float *max_b, cudaStream_t st);
 cudaError_t qvggt_launch_smooth_finalize(const float *ax, const float *aw, int K, float alpha, float lo, float hi,
                                          float *c, cudaStream_t st);
 
