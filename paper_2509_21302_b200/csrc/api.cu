@@ -2,6 +2,7 @@
 #include <new>
 
 #include "qvggt_internal.cuh"
+#include "tensor_map.cuh"
 
 namespace {
 
@@ -17,15 +18,12 @@ int device_is_sm100()
     return major == 10;
 }
 
+// The handle's device work is complete and its device is current.
 void release(qvggt_weights *w)
 {
     if (!w) return;
-    cudaFree(w->Wq);
-    cudaFree(w->Wq8);
-    cudaFree(w->w_scale);
-    cudaFree(w->amul);
-    cudaFree(w->bias);
-    cudaFree(w->status);
+    qvggt_block_release(w->device, w->codes, w->codes_bytes);
+    qvggt_block_release(w->device, w->small, w->small_bytes);
     delete w;
 }
 
@@ -56,26 +54,34 @@ int qvggt_prepare_weights(const void *W_bf16, const void *bias_bf16, const float
     w->N = N;
     w->K = K;
     w->bits = w8 ? 8 : 4;
-    w->Wq = nullptr; w->Wq8 = nullptr; w->w_scale = nullptr; w->amul = nullptr; w->bias = nullptr; w->status = nullptr;
-    cudaGetDevice(&w->device);
-    float *wmul = nullptr;                                   // [K] multipliers, followed by one float for the tensor-wise step size
-    bool ok = (!packed || cudaMalloc(&w->Wq, (size_t)N * K / 2) == cudaSuccess) &&
-              cudaMalloc(&w->w_scale, sizeof(float) * N) == cudaSuccess &&
-              cudaMalloc(&w->amul, sizeof(float) * K) == cudaSuccess &&
-              cudaMalloc(&w->status, sizeof(int)) == cudaSuccess &&
-              cudaMallocAsync(&wmul, sizeof(float) * (K + 4), st) == cudaSuccess &&
-              (!bias_bf16 || cudaMalloc(&w->bias, sizeof(uint16_t) * N) == cudaSuccess) &&
-              (!c8 || cudaMalloc(&w->Wq8, (size_t)N * K) == cudaSuccess);
-    if (!ok) {
+    w->device = qvggt_current_device();
+    w->codes = w->small = nullptr;
+    // each array on a 256-byte boundary of its block
+    auto place = [](size_t &total, size_t bytes) {
+        const size_t at = total;
+        total += (bytes + 255) / 256 * 256;
+        return at;
+    };
+    size_t codes = 0, small = 0;
+    const size_t at_wq = place(codes, packed ? (size_t)N * K / 2 : 0), at_wq8 = place(codes, c8 ? (size_t)N * K : 0);
+    const size_t at_scale = place(small, sizeof(float) * N), at_amul = place(small, sizeof(float) * K),
+                 at_bias = place(small, bias_bf16 ? sizeof(uint16_t) * N : 0), at_status = place(small, sizeof(int)),
+                 at_wmul = place(small, sizeof(float) * (K + 4));    // scratch: [K] multipliers, then one float for the tensor-wise step size
+    if (qvggt_block_acquire(w->device, codes, &w->codes, &w->codes_bytes) != cudaSuccess ||
+        qvggt_block_acquire(w->device, small, &w->small, &w->small_bytes) != cudaSuccess) {
         cudaGetLastError();
-        if (wmul) cudaFreeAsync(wmul, st);
         release(w);
         return QVGGT_ERR_NOMEM;
     }
-    cudaError_t e = cudaMemsetAsync(w->status, 0, sizeof(int), st);
-    if (e == cudaSuccess && bias_bf16)
-        e = cudaMemcpyAsync(w->bias, bias_bf16, sizeof(uint16_t) * N, cudaMemcpyDeviceToDevice, st);
-    if (e == cudaSuccess) e = qvggt_launch_multipliers(smooth_c, sign_v, K, w->amul, wmul, st);
+    unsigned char *wide = static_cast<unsigned char *>(w->codes), *base = static_cast<unsigned char *>(w->small);
+    w->Wq = packed ? wide + at_wq : nullptr;
+    w->Wq8 = c8 ? reinterpret_cast<signed char *>(wide + at_wq8) : nullptr;
+    w->w_scale = reinterpret_cast<float *>(base + at_scale);
+    w->amul = reinterpret_cast<float *>(base + at_amul);
+    w->bias = bias_bf16 ? reinterpret_cast<uint16_t *>(base + at_bias) : nullptr;
+    w->status = reinterpret_cast<int *>(base + at_status);
+    float *wmul = reinterpret_cast<float *>(base + at_wmul);
+    cudaError_t e = qvggt_launch_multipliers(smooth_c, sign_v, K, w->amul, wmul, st, static_cast<const uint16_t *>(bias_bf16), N, w->bias, w->status);
     if (e == cudaSuccess && w->Wq) e = qvggt_launch_rsq(W_bf16, K, N, K, wmul, 0, w->Wq, w->w_scale, st);
     if (e == cudaSuccess && w->Wq8) e = qvggt_launch_rsq_c8(W_bf16, K, N, K, wmul, w->bits, w->Wq8, w->w_scale, st);
     if (e == cudaSuccess && tensorwise) {
@@ -84,8 +90,6 @@ int qvggt_prepare_weights(const void *W_bf16, const void *bias_bf16, const float
         e = qvggt_launch_max_reduce(w->w_scale, N, wmul + K, st);
         if (e == cudaSuccess) e = qvggt_launch_rsq_static_c8(W_bf16, K, N, K, wmul, w->bits, wmul + K, w->Wq8, w->w_scale, st);
     }
-    // wmul is scratch: stream-ordered release so that the call stays asynchronous
-    if (cudaFreeAsync(wmul, st) != cudaSuccess) cudaGetLastError();
     if (e != cudaSuccess) {
         cudaStreamSynchronize(st);
         release(w);

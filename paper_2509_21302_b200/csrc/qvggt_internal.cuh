@@ -15,6 +15,8 @@ struct qvggt_weights {
     float *amul;         // [K]
     uint16_t *bias;      // [N] bf16 bits, or nullptr
     int *status;         // device status word (0 = ok)
+    void *codes, *small; // the two device blocks that these lie in: Wq and Wq8; the rest
+    size_t codes_bytes, small_bytes;   // their sizes as allocated
 };
 
 // Device status codes written by kernels whose bounded waits expire.
@@ -28,9 +30,15 @@ enum : int {
     QVGGT_DEV_TIMEOUT_PACKED_FREE = 6 // TMA producer gave up waiting for a packed stage to be released
 };
 
+// device_blocks.cu: device memory of the handles, kept for the next handle within a bound.  A block that is released must have
+// no work in flight that uses it.
+cudaError_t qvggt_block_acquire(int device, size_t bytes, void **block, size_t *block_bytes);
+void qvggt_block_release(int device, void *block, size_t block_bytes);
+
 // rsq.cu
-cudaError_t qvggt_launch_multipliers(const float *c, const signed char *v, int K, float *amul, float *wmul,
-                                     cudaStream_t st);
+// multipliers; also copies the bias and clears the status word, if given
+cudaError_t qvggt_launch_multipliers(const float *c, const signed char *v, int K, float *amul, float *wmul, cudaStream_t st,
+                                     const uint16_t *bias = nullptr, int N = 0, uint16_t *bias_out = nullptr, int *status = nullptr);
 cudaError_t qvggt_launch_rsq(const void *X, long long ldx, int M, int K, const float *mul, int group,
                              unsigned char *Xq, float *scales, cudaStream_t st);
 cudaError_t qvggt_launch_rsq_c8(const void *X, long long ldx, int M, int K, const float *mul, int bits, signed char *Xq8,

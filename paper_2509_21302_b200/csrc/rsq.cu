@@ -596,10 +596,14 @@ colmax_kernel(const uint16_t *__restrict__ A, int rows_a, int grid_a, const uint
     }
 }
 
-__global__ void multipliers_kernel(const float *__restrict__ c, const signed char *__restrict__ v, int K,
-                                   float *__restrict__ amul, float *__restrict__ wmul)
+// The small arrays of a handle in one launch: multipliers, a copy of the bias, the cleared status word (any may be absent).
+__global__ void multipliers_kernel(const float *__restrict__ c, const signed char *__restrict__ v, int K, float *__restrict__ amul,
+                                   float *__restrict__ wmul, const uint16_t *__restrict__ bias, int N, uint16_t *__restrict__ bias_out,
+                                   int *__restrict__ status)
 {
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (status && k == 0) *status = 0;
+    if (bias_out && k < N) bias_out[k] = bias[k];
     if (k >= K) return;
     const float nrm = (K == 1024) ? 0.03125f : 0.015625f;   // K^{-1/2}, exact
     const float sgn = (v != nullptr && v[k] < 0) ? -nrm : nrm;
@@ -649,10 +653,11 @@ int rsq_grid(int M, int rows_per_cta, int ctas_per_sm = 6)
 
 }  // namespace
 
-cudaError_t qvggt_launch_multipliers(const float *c, const signed char *v, int K, float *amul, float *wmul,
-                                     cudaStream_t st)
+cudaError_t qvggt_launch_multipliers(const float *c, const signed char *v, int K, float *amul, float *wmul, cudaStream_t st,
+                                     const uint16_t *bias, int N, uint16_t *bias_out, int *status)
 {
-    multipliers_kernel<<<(K + 255) / 256, 256, 0, st>>>(c, v, K, amul, wmul);
+    const int n = (bias_out && N > K) ? N : K;
+    multipliers_kernel<<<(n + 255) / 256, 256, 0, st>>>(c, v, K, amul, wmul, bias, N, bias_out, status);
     return cudaGetLastError();
 }
 

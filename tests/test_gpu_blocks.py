@@ -1,0 +1,81 @@
+"""Device memory of the weight handles: a freed handle's blocks may serve the next one.  Contents never leak from one handle into the
+next, threads and streams do not disturb each other, and what is kept is bounded."""
+import threading
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2509_21302_b200 as q
+import workload
+from _util import dev_bf16
+
+pytestmark = pytest.mark.gpu
+
+
+def _layer(K, N, seed):
+    spec = workload.LinearSpec("b", K, N, workload.DIST_NORMAL, seed, 0)
+    W, b = spec.weight(), spec.bias()
+    c = oracle.smooth_factors(spec.x_calib(16), W)
+    return dev_bf16(W), dev_bf16(b), torch.from_numpy(c).cuda(), oracle.prepare_weights(W, c), b
+
+
+def _check(h, ref, bias, flags):
+    v = h.view()
+    assert np.array_equal(v["w_scale"].cpu().numpy(), ref["w_scale"]) and np.array_equal(v["amul"].cpu().numpy(), ref["amul"])
+    assert (v["bias"] is None) == (bias is None)
+    if bias is not None:
+        assert np.array_equal(v["bias"].view(torch.int16).cpu().numpy().view(np.uint16), bias)
+    if flags in (False, True):
+        assert np.array_equal(v["wq"].cpu().numpy(), ref["wq_packed"])
+    if flags:
+        assert np.array_equal(h.view_c8().cpu().numpy(), ref["wq"])
+    assert h.device_status() == 0
+
+
+@pytest.mark.parametrize("flags", [False, True, "only"])
+def test_handles_of_changing_size_one_after_the_other(flags):
+    layers = [_layer(K, N, 40 + i) for i, (K, N) in enumerate([(1024, 384), (4096, 128), (1024, 384), (1024, 512), (4096, 128)])]
+    for i in range(3):
+        for W, b, c, ref, bias in layers:
+            with_bias = i != 1
+            h = q.prepare_weights(W, b if with_bias else None, c, None, c8=flags)
+            _check(h, ref, bias if with_bias else None, flags)
+            h.free()
+
+
+def test_threads_and_streams_prepare_and_free_at_the_same_time():
+    layers = [_layer(K, N, 60 + i) for i, (K, N) in enumerate([(1024, 384), (1024, 384), (4096, 128), (1024, 256)])]
+    torch.cuda.synchronize()
+    failed = []
+
+    def work(i):
+        try:
+            W, b, c, ref, bias = layers[i]
+            with torch.cuda.stream(torch.cuda.Stream()):
+                for _ in range(12):
+                    h = q.prepare_weights(W, b, c, None, c8=True)
+                    _check(h, ref, bias, True)
+                    h.free()
+        except BaseException as e:      # reported by the main thread
+            failed.append(e)
+
+    ts = [threading.Thread(target=work, args=(i,)) for i in range(len(layers))]
+    for t in ts:
+        t.start()
+    for t in ts:
+        t.join()
+    assert not failed, failed
+
+
+def test_what_is_kept_is_bounded():
+    W, b, c, _, _ = _layer(4096, 1024, 80)
+    q.prepare_weights(W, b, c, None, c8="only").free()
+    torch.cuda.synchronize()
+    free0 = torch.cuda.mem_get_info()[0]
+    hs = [q.prepare_weights(W, b, c, None, c8="only") for _ in range(48)]       # 200 MB of codes
+    for h in hs:
+        h.free()
+    # at most 64 MB of freed blocks stay with the library (and the allocator's own granules)
+    assert free0 - torch.cuda.mem_get_info()[0] <= (64 << 20) + (4 << 20)
