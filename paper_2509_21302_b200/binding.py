@@ -1,4 +1,6 @@
-"""Thin Python binding of libqvggt (ctypes): argument marshalling only.
+"""Thin Python binding of libqvggt: argument marshalling only.  The calls made per layer and forward pass go through a small
+extension module (csrc/fastcall.cpp, 3 us a call instead of 8.5); everything else, and every call that is not plainly
+well-formed, through ctypes.
 
 Every step of the path runs in the CUDA kernels behind the C ABI declared in include/qvggt.h;
 PyTorch is used for device memory and streams.  There is no CPU fallback: if the shared library
@@ -7,6 +9,8 @@ is missing or a call fails, an exception is raised.
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
 
 import torch
@@ -41,16 +45,18 @@ class QvggtError(RuntimeError):
 
 
 _lib = None
+_fast = None       # the extension module, once lib() has loaded it
 
 
 def lib() -> ctypes.CDLL:
     """Loads libqvggt.so (built in-tree by `build.build()`); raises if it is not there."""
-    global _lib
+    global _lib, _fast
     if _lib is None:
         path = _build.LIB
-        if not os.path.exists(path):
-            raise RuntimeError(f"{path} is missing: run __graft_entry__.build() (nvcc, sm_100a) first; "
-                               "there is no fallback path")
+        for p in (path, _build.FASTCALL):
+            if not os.path.exists(p):
+                raise RuntimeError(f"{p} is missing: run __graft_entry__.build() (nvcc, sm_100a) first; "
+                                   "there is no fallback path")
         L = ctypes.CDLL(path)
         vp, i32, i64, f32 = ctypes.c_void_p, ctypes.c_int, ctypes.c_longlong, ctypes.c_float
         L.qvggt_prepare_weights.argtypes = [vp, vp, vp, vp, i32, i32, i32, vp, ctypes.POINTER(vp)]
@@ -83,6 +89,10 @@ def lib() -> ctypes.CDLL:
         for name in EXPORTS:
             if name not in ("qvggt_free_weights", "qvggt_status_string"):
                 getattr(L, name).restype = i32
+        loader = importlib.machinery.ExtensionFileLoader("_qvggt_fastcall", _build.FASTCALL)
+        fast = importlib.util.module_from_spec(importlib.util.spec_from_loader("_qvggt_fastcall", loader))
+        loader.exec_module(fast)
+        _fast = fast
         _lib = L
     return _lib
 
@@ -124,15 +134,10 @@ class Weights:
                "qvggt_weights_view")
         N, K = n.value, k.value
 
-        def wrap(p, nbytes, dtype, shape):
-            if not p.value:
-                return None
-            return _from_device_ptr(p.value, nbytes, dtype, shape)
+        def copy(p, kind, d0, d1=-1):
+            return _fast.copy_array(p.value, kind, d0, d1) if p.value else None
 
-        return dict(wq=wrap(ptrs[0], N * K // 2, torch.uint8, (N, K // 2)),
-                    w_scale=wrap(ptrs[1], 4 * N, torch.float32, (N,)),
-                    amul=wrap(ptrs[2], 4 * K, torch.float32, (K,)),
-                    bias=wrap(ptrs[3], 2 * N, torch.bfloat16, (N,)))
+        return dict(wq=copy(ptrs[0], 0, N, K // 2), w_scale=copy(ptrs[1], 2, N), amul=copy(ptrs[2], 2, K), bias=copy(ptrs[3], 3, N))
 
     def view_c8(self) -> torch.Tensor | None:
         """Copy of the int8 [N, K] codes (None if prepared without c8=True)."""
@@ -141,7 +146,7 @@ class Weights:
         self.bits = bits.value
         if not p.value:
             return None
-        return _from_device_ptr(p.value, self.N * self.K, torch.uint8, (self.N, self.K)).view(torch.int8)
+        return _fast.copy_array(p.value, 1, self.N, self.K)
 
     def device_status(self) -> int:
         code = ctypes.c_int(0)
@@ -160,22 +165,6 @@ class Weights:
             self.free()
         except Exception:
             pass
-
-
-class _DeviceArray:
-    """Minimal __cuda_array_interface__ carrier so torch can wrap a raw device pointer."""
-
-    def __init__(self, ptr: int, shape, typestr: str):
-        self.__cuda_array_interface__ = {"shape": tuple(shape), "typestr": typestr, "data": (ptr, False), "version": 2}
-
-
-def _from_device_ptr(ptr: int, nbytes: int, dtype: torch.dtype, shape) -> torch.Tensor:
-    """Copy of the device array at `ptr` as a fresh torch tensor (so it outlives the handle)."""
-    typestr = {torch.uint8: "|u1", torch.float32: "<f4", torch.bfloat16: "<i2"}[dtype]
-    t = torch.as_tensor(_DeviceArray(ptr, shape, typestr), device="cuda")
-    assert t.numel() * t.element_size() == nbytes
-    t = t.clone()
-    return t.view(torch.bfloat16) if dtype == torch.bfloat16 else t
 
 
 def prepare_weights(W: torch.Tensor, bias: torch.Tensor | None, smooth_c: torch.Tensor,
@@ -203,6 +192,10 @@ def prepare_weights(W: torch.Tensor, bias: torch.Tensor | None, smooth_c: torch.
 def rotate_smooth_quantize(w: Weights, X: torch.Tensor, group: int = 0, Xq: torch.Tensor | None = None,
                            a_scale: torch.Tensor | None = None):
     """X [M,K] bf16 (row stride may exceed K) -> (Xq [M,K/2] uint8, a_scale fp32 [M] or [M,K/128])."""
+    if _fast is not None:
+        r = _fast.rotate_smooth_quantize(w._h, w.K, X, group, Xq, a_scale)
+        if r is not None:
+            return r
     assert X.dim() == 2 and X.element_size() == 2 and X.stride(1) == 1 and X.shape[1] == w.K
     M = X.shape[0]
     if Xq is None:
@@ -218,6 +211,10 @@ def rotate_smooth_quantize(w: Weights, X: torch.Tensor, group: int = 0, Xq: torc
 def w4a4_linear(w: Weights, Xq: torch.Tensor, a_scale: torch.Tensor, group: int = 0, Y: torch.Tensor | None = None,
                 acc_debug: torch.Tensor | None = None) -> torch.Tensor:
     """-> Y [M,N] bf16.  acc_debug: optional int32 [M,N] (group 0) or [K/128,M,N] receiving the integer sums."""
+    if _fast is not None and acc_debug is None:
+        r = _fast.w4a4_linear(w._h, w.N, w.K, Xq, a_scale, group, Y)
+        if r is not None:
+            return r
     M = Xq.shape[0]
     assert Xq.dtype == torch.uint8 and Xq.is_contiguous() and Xq.shape[1] == w.K // 2
     assert a_scale.dtype == torch.float32 and a_scale.is_contiguous()
@@ -235,6 +232,10 @@ def w4a4_linear(w: Weights, Xq: torch.Tensor, a_scale: torch.Tensor, group: int 
 def rotate_smooth_quantize_c8(w: Weights, X: torch.Tensor, Xq8: torch.Tensor | None = None,
                               a_scale: torch.Tensor | None = None):
     """X [M,K] bf16 (row stride may exceed K) -> (Xq8 [M,K] int8, one code per byte; a_scale fp32 [M])."""
+    if _fast is not None:
+        r = _fast.rotate_smooth_quantize_c8(w._h, w.K, X, Xq8, a_scale)
+        if r is not None:
+            return r
     assert X.dim() == 2 and X.element_size() == 2 and X.stride(1) == 1 and X.shape[1] == w.K
     M = X.shape[0]
     if Xq8 is None:
@@ -252,6 +253,10 @@ def rotate_smooth_quantize_tc(w: Weights, X: torch.Tensor, c8: bool = False, Xq:
                               a_scale: torch.Tensor | None = None, y_debug: torch.Tensor | None = None):
     """Tensor-core Hadamard mode (tolerance contract, see include/qvggt.h): X [M,K] bf16 ->
     (Xq [M,K/2] uint8, or [M,K] int8 with c8=True; a_scale fp32 [M]).  y_debug: optional fp32 [M,K] receiving the rotated rows."""
+    if _fast is not None and y_debug is None:
+        r = _fast.rotate_smooth_quantize_tc(w._h, w.K, X, c8, Xq, a_scale)
+        if r is not None:
+            return r
     assert X.dim() == 2 and X.element_size() == 2 and X.stride(1) == 1 and X.shape[1] == w.K
     M = X.shape[0]
     if Xq is None:
@@ -270,6 +275,10 @@ def rotate_smooth_quantize_tc(w: Weights, X: torch.Tensor, c8: bool = False, Xq:
 def rotate_smooth_quantize_static_c8(w: Weights, X: torch.Tensor, delta: torch.Tensor, Xq8: torch.Tensor | None = None,
                                      a_scale: torch.Tensor | None = None):
     """Static tensor-wise quantizer: delta = one fp32 step size on the device -> (Xq8 [M,K] int8, a_scale [M] = delta)."""
+    if _fast is not None:
+        r = _fast.rotate_smooth_quantize_static_c8(w._h, w.K, X, delta, Xq8, a_scale)
+        if r is not None:
+            return r
     assert X.dim() == 2 and X.element_size() == 2 and X.stride(1) == 1 and X.shape[1] == w.K
     assert delta.dtype == torch.float32 and delta.numel() == 1 and delta.is_cuda
     M = X.shape[0]
@@ -286,6 +295,10 @@ def rotate_smooth_quantize_static_c8(w: Weights, X: torch.Tensor, delta: torch.T
 def layernorm_rotate_smooth_quantize_c8(w: Weights, X: torch.Tensor, gamma: torch.Tensor, beta: torch.Tensor, eps: float = 1e-5,
                                         Xq8: torch.Tensor | None = None, a_scale: torch.Tensor | None = None):
     """LayerNorm (gamma, beta fp32 [K]) fused in front of rotate_smooth_quantize_c8 -> (Xq8 [M,K] int8, a_scale [M])."""
+    if _fast is not None:
+        r = _fast.layernorm_rotate_smooth_quantize_c8(w._h, w.K, X, gamma, beta, eps, Xq8, a_scale)
+        if r is not None:
+            return r
     assert X.dim() == 2 and X.element_size() == 2 and X.stride(1) == 1 and X.shape[1] == w.K
     assert gamma.dtype == torch.float32 and beta.dtype == torch.float32 and gamma.numel() == w.K and beta.numel() == w.K
     M = X.shape[0]
@@ -314,6 +327,10 @@ def layernorm(X: torch.Tensor, gamma: torch.Tensor, beta: torch.Tensor, eps: flo
 
 def rotate_smooth_quantize_c8_grouped(w: Weights, X: torch.Tensor, Xq8: torch.Tensor | None = None, a_scale: torch.Tensor | None = None):
     """One scale per token per 128 rotated channels, codes one per byte -> (Xq8 [M,K] int8, a_scale fp32 [M, K/128])."""
+    if _fast is not None:
+        r = _fast.rotate_smooth_quantize_c8_grouped(w._h, w.K, X, Xq8, a_scale)
+        if r is not None:
+            return r
     assert X.dim() == 2 and X.element_size() == 2 and X.stride(1) == 1 and X.shape[1] == w.K
     M = X.shape[0]
     if Xq8 is None:
@@ -328,6 +345,10 @@ def rotate_smooth_quantize_c8_grouped(w: Weights, X: torch.Tensor, Xq8: torch.Te
 def w4a4_linear_c8_grouped(w: Weights, Xq8: torch.Tensor, a_scale: torch.Tensor, Y: torch.Tensor | None = None,
                            acc_debug: torch.Tensor | None = None) -> torch.Tensor:
     """-> Y [M,N] bf16 from one-code-per-byte codes with group-128 scales; acc_debug: optional int32 [K/128, M, N]."""
+    if _fast is not None and acc_debug is None:
+        r = _fast.w4a4_linear_c8_grouped(w._h, w.N, w.K, Xq8, a_scale, Y)
+        if r is not None:
+            return r
     M = Xq8.shape[0]
     assert Xq8.dtype == torch.int8 and Xq8.is_contiguous() and Xq8.shape[1] == w.K
     assert a_scale.dtype == torch.float32 and a_scale.is_contiguous() and a_scale.shape == (M, w.K // 128)
@@ -352,6 +373,10 @@ def gelu(X: torch.Tensor, Y: torch.Tensor | None = None) -> torch.Tensor:
 
 def gelu_rotate_smooth_quantize_c8(w: Weights, X: torch.Tensor, Xq8: torch.Tensor | None = None, a_scale: torch.Tensor | None = None):
     """GELU fused in front of rotate_smooth_quantize_c8 -> (Xq8 [M,K] int8, a_scale [M])."""
+    if _fast is not None:
+        r = _fast.gelu_rotate_smooth_quantize_c8(w._h, w.K, X, Xq8, a_scale)
+        if r is not None:
+            return r
     assert X.dim() == 2 and X.element_size() == 2 and X.stride(1) == 1 and X.shape[1] == w.K
     M = X.shape[0]
     if Xq8 is None:
@@ -366,6 +391,10 @@ def gelu_rotate_smooth_quantize_c8(w: Weights, X: torch.Tensor, Xq8: torch.Tenso
 def w4a4_linear_c8(w: Weights, Xq8: torch.Tensor, a_scale: torch.Tensor, Y: torch.Tensor | None = None,
                    acc_debug: torch.Tensor | None = None) -> torch.Tensor:
     """-> Y [M,N] bf16 from codes held one per byte.  acc_debug: optional int32 [M,N] receiving the integer sums."""
+    if _fast is not None and acc_debug is None:
+        r = _fast.w4a4_linear_c8(w._h, w.N, w.K, Xq8, a_scale, Y)
+        if r is not None:
+            return r
     M = Xq8.shape[0]
     assert Xq8.dtype == torch.int8 and Xq8.is_contiguous() and Xq8.shape[1] == w.K
     assert a_scale.dtype == torch.float32 and a_scale.is_contiguous()
@@ -383,6 +412,10 @@ def w4a4_linear_c8(w: Weights, Xq8: torch.Tensor, a_scale: torch.Tensor, Y: torc
 def w4a4_linear_c8_packed_weights(w: Weights, Xq8: torch.Tensor, a_scale: torch.Tensor, w_scratch: torch.Tensor,
                                   Y: torch.Tensor | None = None, acc_debug: torch.Tensor | None = None) -> torch.Tensor:
     """The one-code-per-byte GEMM on a handle that keeps only packed weight codes; w_scratch: int8, at least N*K elements."""
+    if _fast is not None and acc_debug is None:
+        r = _fast.w4a4_linear_c8_packed_weights(w._h, w.N, w.K, Xq8, a_scale, w_scratch, Y)
+        if r is not None:
+            return r
     M = Xq8.shape[0]
     assert Xq8.dtype == torch.int8 and Xq8.is_contiguous() and Xq8.shape[1] == w.K
     assert w_scratch.dtype == torch.int8 and w_scratch.is_contiguous() and w_scratch.numel() >= w.N * w.K
@@ -398,6 +431,10 @@ def rotate_smooth_quantize_c8_expand(w: Weights, X: torch.Tensor, w_scratch: tor
                                      a_scale: torch.Tensor | None = None):
     """rotate_smooth_quantize_c8 whose launch also expands the handle's packed weight codes into w_scratch (int8, at
     least N*K elements) -> (Xq8 [M,K] int8, a_scale [M])."""
+    if _fast is not None:
+        r = _fast.rotate_smooth_quantize_c8_expand(w._h, w.N, w.K, X, w_scratch, Xq8, a_scale)
+        if r is not None:
+            return r
     assert X.dim() == 2 and X.element_size() == 2 and X.stride(1) == 1 and X.shape[1] == w.K
     assert w_scratch.dtype == torch.int8 and w_scratch.is_contiguous() and w_scratch.numel() >= w.N * w.K
     M = X.shape[0]
@@ -414,6 +451,10 @@ def w4a4_linear_c8_expanded(w: Weights, Xq8: torch.Tensor, a_scale: torch.Tensor
                             Y: torch.Tensor | None = None, acc_debug: torch.Tensor | None = None) -> torch.Tensor:
     """The one-code-per-byte GEMM reading this handle's weight codes from w_scratch, where rotate_smooth_quantize_c8_expand
     put them."""
+    if _fast is not None and acc_debug is None:
+        r = _fast.w4a4_linear_c8_expanded(w._h, w.N, w.K, Xq8, a_scale, w_scratch, Y)
+        if r is not None:
+            return r
     M = Xq8.shape[0]
     assert Xq8.dtype == torch.int8 and Xq8.is_contiguous() and Xq8.shape[1] == w.K
     assert w_scratch.dtype == torch.int8 and w_scratch.is_contiguous() and w_scratch.numel() >= w.N * w.K

@@ -1,13 +1,15 @@
-"""Builds libqvggt.so (CUDA kernels + C ABI) in-tree with nvcc for sm_100a."""
+"""Builds libqvggt.so (CUDA kernels + C ABI, nvcc, sm_100a) and the Python call path in front of it (g++) in-tree."""
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
+import sysconfig
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(_HERE, "csrc")
 LIB = os.path.join(_HERE, "libqvggt.so")
+FASTCALL = os.path.join(_HERE, "_qvggt_fastcall.so")
 INCLUDE = os.path.join(os.path.dirname(_HERE), "include")
 
 NVCC_FLAGS = [
@@ -21,27 +23,44 @@ def sources() -> list[str]:
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
 
 
-def _deps() -> list[str]:
-    return sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(INCLUDE, "*.h"))
+def _stale(target: str, deps: list[str]) -> bool:
+    if not os.path.exists(target):
+        return True
+    t = os.path.getmtime(target)
+    return any(os.path.getmtime(f) > t for f in deps)
+
+
+def _headers() -> list[str]:
+    return glob.glob(os.path.join(INCLUDE, "*.h"))
 
 
 def is_stale() -> bool:
-    if not os.path.exists(LIB):
-        return True
-    t = os.path.getmtime(LIB)
-    return any(os.path.getmtime(f) > t for f in _deps())
+    return (_stale(LIB, sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + _headers())
+            or _stale(FASTCALL, [os.path.join(CSRC, "fastcall.cpp")] + _headers()))
 
 
 def build(force: bool = False, verbose: bool = False) -> str:
-    if not (force or is_stale()):
-        return LIB
-    nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
-    tmp = LIB + f".tmp{os.getpid()}"
-    cmd = [nvcc, *NVCC_FLAGS, "-I", INCLUDE, "-o", tmp, *sources()]
-    if verbose:
-        cmd.insert(1, "-Xptxas=-v")
-    subprocess.check_call(cmd)
-    os.replace(tmp, LIB)
+    if force or _stale(LIB, sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + _headers()):
+        nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
+        tmp = LIB + f".tmp{os.getpid()}"
+        cmd = [nvcc, *NVCC_FLAGS, "-I", INCLUDE, "-o", tmp, *sources()]
+        if verbose:
+            cmd.insert(1, "-Xptxas=-v")
+        subprocess.check_call(cmd)
+        os.replace(tmp, LIB)
+    src = os.path.join(CSRC, "fastcall.cpp")
+    if force or _stale(FASTCALL, [src] + _headers()):
+        import torch
+
+        root = os.path.dirname(torch.__file__)
+        tmp = FASTCALL + f".tmp{os.getpid()}"
+        subprocess.check_call(
+            [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}",
+             "-I", INCLUDE, "-I", os.path.join(root, "include"), "-I", os.path.join(root, "include", "torch", "csrc", "api", "include"),
+             "-I", "/usr/local/cuda/include", "-I", sysconfig.get_paths()["include"], "-o", tmp, src,
+             "-L", _HERE, "-l:" + os.path.basename(LIB), "-Wl,-rpath,$ORIGIN", "-L", os.path.join(root, "lib"),
+             "-ltorch_python", "-ltorch_cpu", "-lc10", "-lc10_cuda"])
+        os.replace(tmp, FASTCALL)
     return LIB
 
 

@@ -1,0 +1,354 @@
+// The call path from Python into libqvggt, for the calls a program makes per layer and forward pass.
+//
+// Through ctypes a call costs 8.5 us on the host, 2.4 of it the launch itself: tensor attributes read one by one from Python, the
+// stream object, ctypes' argument conversion.  At a frame or less that is more than the work on the GPU.  Here the arguments go
+// from the tensors to the C entry points directly (3 us a call in all).
+//
+// A function returns what its namesake in binding.py returns, or None when an argument is not plainly what the call expects or
+// the library returned a status: binding.py then takes its own path, which checks, converts and reports.  Nothing
+// here keeps state.
+#include <Python.h>
+
+#include <ATen/core/Tensor.h>
+#include <ATen/ops/empty.h>
+#include <ATen/ops/from_blob.h>
+#include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/autograd/python_variable.h>
+
+#include "../../include/qvggt.h"
+
+namespace {
+
+using at::ScalarType;
+using at::Tensor;
+
+// Positional arguments of one call.  `ok` turns false at the first one that this path does not take.
+struct Args {
+    PyObject *const *a;
+    Py_ssize_t n, i = 0;
+    bool ok = true;
+
+    PyObject *next() { return (i < n) ? a[i++] : (ok = false, Py_None); }
+    const qvggt_weights_t *handle()
+    {
+        PyObject *o = next();
+        void *p = PyLong_Check(o) ? PyLong_AsVoidPtr(o) : nullptr;
+        if (!p) ok = false;
+        if (PyErr_Occurred()) PyErr_Clear();
+        return static_cast<const qvggt_weights_t *>(p);
+    }
+    long long integer()
+    {
+        PyObject *o = next();
+        const long long v = PyLong_Check(o) ? PyLong_AsLongLong(o) : (ok = false, 0);
+        if (PyErr_Occurred()) { PyErr_Clear(); ok = false; }
+        return v;
+    }
+    double real()
+    {
+        PyObject *o = next();
+        const double v = (PyFloat_Check(o) || PyLong_Check(o)) ? PyFloat_AsDouble(o) : (ok = false, 0.0);
+        if (PyErr_Occurred()) { PyErr_Clear(); ok = false; }
+        return v;
+    }
+    // A tensor on the current device, or an undefined one for None where `optional`.
+    const Tensor &tensor(bool optional = false)
+    {
+        static const Tensor none;
+        PyObject *o = next();
+        if (o == Py_None && optional) return none;
+        if (!THPVariable_Check(o)) { ok = false; return none; }
+        const Tensor &t = THPVariable_Unpack(o);
+        if (!t.is_cuda() || t.layout() != at::kStrided) ok = false;
+        return t;
+    }
+    // Activation rows: bf16 [M, K], unit stride along K.
+    const Tensor &rows(int64_t K)
+    {
+        const Tensor &t = tensor();
+        if (ok && !(t.dim() == 2 && t.element_size() == 2 && t.size(1) == K && t.stride(1) == 1)) ok = false;
+        return t;
+    }
+    // A contiguous tensor of the given type and shape.
+    const Tensor &exact(ScalarType type, int64_t d0, int64_t d1, bool optional = false)
+    {
+        const Tensor &t = tensor(optional);
+        if (ok && t.defined()) {
+            const bool shape = d1 < 0 ? (t.dim() == 1 && t.size(0) == d0) : (t.dim() == 2 && t.size(0) == d0 && t.size(1) == d1);
+            if (t.scalar_type() != type || !shape || !t.is_contiguous()) ok = false;
+        }
+        return t;
+    }
+    // A contiguous tensor of the given type with at least n elements.
+    const Tensor &at_least(ScalarType type, int64_t n_min)
+    {
+        const Tensor &t = tensor();
+        if (ok && !(t.scalar_type() == type && t.numel() >= n_min && t.is_contiguous())) ok = false;
+        return t;
+    }
+    bool done() const { return ok && i == n; }
+};
+
+int64_t pitch(const Tensor &t) { return t.size(0) > 1 ? t.stride(0) : t.size(1); }
+
+void *stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
+
+template <class F>
+int without_gil(F f)
+{
+    PyThreadState *s = PyEval_SaveThread();
+    const int st = f();
+    PyEval_RestoreThread(s);
+    return st;
+}
+
+PyObject *wrap(const Tensor &given, const Tensor &made, PyObject *obj)
+{
+    if (given.defined()) { Py_INCREF(obj); return obj; }
+    return THPVariable_Wrap(made);
+}
+
+#define QVGGT_GUARD_BEGIN try {
+#define QVGGT_GUARD_END                                     \
+    }                                                       \
+    catch (const std::exception &) { Py_RETURN_NONE; }
+
+// Quantize calls: f(handle, X, ldx, M, Xq, a_scale, stream); `X` and what precedes the outputs have been read from `in`.
+template <class F>
+PyObject *quantize(Args &in, const Tensor &X, ScalarType code, int64_t row_codes, int64_t row_scales, F f)
+{
+    if (!in.ok) Py_RETURN_NONE;
+    const int64_t M = X.size(0);
+    PyObject *oq = in.next(), *oa = in.next();
+    in.i -= 2;
+    const Tensor &xq = in.exact(code, M, row_codes, true), &as = in.exact(at::kFloat, M, row_scales, true);
+    if (!in.done() || M > INT32_MAX) Py_RETURN_NONE;
+    const Tensor made_q = xq.defined() ? Tensor() : at::empty({M, row_codes}, X.options().dtype(code));
+    const Tensor made_a = as.defined() ? Tensor() : (row_scales < 0 ? at::empty({M}, X.options().dtype(at::kFloat)) : at::empty({M, row_scales}, X.options().dtype(at::kFloat)));
+    const void *x = X.data_ptr();
+    void *q = (xq.defined() ? xq : made_q).data_ptr();
+    float *a = static_cast<float *>((as.defined() ? as : made_a).data_ptr());
+    void *st = stream();
+    if (without_gil([&] { return f(x, pitch(X), (int)M, q, a, st); }) != QVGGT_OK) Py_RETURN_NONE;
+    return PyTuple_Pack(2, wrap(xq, made_q, oq), wrap(as, made_a, oa));
+}
+
+// PyTuple_Pack adds references of its own: give back the ones wrap() made.
+PyObject *release_items(PyObject *t)
+{
+    if (t && PyTuple_Check(t))
+        for (Py_ssize_t i = 0; i < PyTuple_GET_SIZE(t); ++i) Py_DECREF(PyTuple_GET_ITEM(t, i));
+    return t;
+}
+
+// GEMM calls: f(codes, a_scale, M, Y, ldy, stream); reads Y (optional) and returns it.
+template <class F>
+PyObject *linear(Args &in, const Tensor &xq, const Tensor &as, int64_t N, F f)
+{
+    if (!in.ok) Py_RETURN_NONE;
+    const int64_t M = xq.size(0);
+    PyObject *oy = in.next();
+    --in.i;
+    const Tensor &y = in.tensor(true);
+    if (!in.done() || M > INT32_MAX) Py_RETURN_NONE;
+    if (y.defined() && !(y.dim() == 2 && y.element_size() == 2 && y.size(0) == M && y.size(1) == N && y.stride(1) == 1)) Py_RETURN_NONE;
+    const Tensor made = y.defined() ? Tensor() : at::empty({M, N}, xq.options().dtype(at::kBFloat16));
+    const Tensor &Y = y.defined() ? y : made;
+    const void *q = xq.data_ptr();
+    const float *a = static_cast<const float *>(as.data_ptr());
+    void *out = Y.data_ptr(), *st = stream();
+    if (without_gil([&] { return f(q, a, (int)M, out, pitch(Y), st); }) != QVGGT_OK) Py_RETURN_NONE;
+    return wrap(y, made, oy);
+}
+
+using U8 = unsigned char;
+using S8 = signed char;
+
+// (handle, K, X, group, Xq, a_scale)
+PyObject *rotate_smooth_quantize(PyObject *, PyObject *const *args, Py_ssize_t n)
+{
+    QVGGT_GUARD_BEGIN
+    Args in{args, n};
+    auto *h = in.handle();
+    const int64_t K = in.integer();
+    const Tensor &X = in.rows(K);
+    const int64_t group = in.integer();
+    if (group != 0 && group != 128) Py_RETURN_NONE;
+    return release_items(quantize(in, X, at::kByte, K / 2, group ? K / 128 : -1, [&](const void *x, int64_t ldx, int M, void *q, float *a, void *st) {
+        return qvggt_rotate_smooth_quantize(h, x, ldx, M, (int)group, static_cast<U8 *>(q), a, st);
+    }));
+    QVGGT_GUARD_END
+}
+
+// (handle, K, X, Xq8, a_scale)
+template <int (*FN)(const qvggt_weights_t *, const void *, long long, int, S8 *, float *, void *), bool GROUPED>
+PyObject *quantize_c8(PyObject *, PyObject *const *args, Py_ssize_t n)
+{
+    QVGGT_GUARD_BEGIN
+    Args in{args, n};
+    auto *h = in.handle();
+    const int64_t K = in.integer();
+    const Tensor &X = in.rows(K);
+    return release_items(quantize(in, X, at::kChar, K, GROUPED ? K / 128 : -1, [&](const void *x, int64_t ldx, int M, void *q, float *a, void *st) {
+        return FN(h, x, ldx, M, static_cast<S8 *>(q), a, st);
+    }));
+    QVGGT_GUARD_END
+}
+
+// (handle, K, X, c8, Xq, a_scale)
+PyObject *rotate_smooth_quantize_tc(PyObject *, PyObject *const *args, Py_ssize_t n)
+{
+    QVGGT_GUARD_BEGIN
+    Args in{args, n};
+    auto *h = in.handle();
+    const int64_t K = in.integer();
+    const Tensor &X = in.rows(K);
+    const bool c8 = in.integer() != 0;
+    return release_items(quantize(in, X, c8 ? at::kChar : at::kByte, c8 ? K : K / 2, -1, [&](const void *x, int64_t ldx, int M, void *q, float *a, void *st) {
+        return c8 ? qvggt_rotate_smooth_quantize_tc_c8(h, x, ldx, M, static_cast<S8 *>(q), a, nullptr, st)
+                  : qvggt_rotate_smooth_quantize_tc(h, x, ldx, M, static_cast<U8 *>(q), a, nullptr, st);
+    }));
+    QVGGT_GUARD_END
+}
+
+// (handle, K, X, delta, Xq8, a_scale)
+PyObject *rotate_smooth_quantize_static_c8(PyObject *, PyObject *const *args, Py_ssize_t n)
+{
+    QVGGT_GUARD_BEGIN
+    Args in{args, n};
+    auto *h = in.handle();
+    const int64_t K = in.integer();
+    const Tensor &X = in.rows(K);
+    const Tensor &delta = in.at_least(at::kFloat, 1);
+    if (in.ok && delta.numel() != 1) in.ok = false;
+    return release_items(quantize(in, X, at::kChar, K, -1, [&](const void *x, int64_t ldx, int M, void *q, float *a, void *st) {
+        return qvggt_rotate_smooth_quantize_static_c8(h, x, ldx, M, static_cast<const float *>(delta.data_ptr()), static_cast<S8 *>(q), a, st);
+    }));
+    QVGGT_GUARD_END
+}
+
+// (handle, K, X, gamma, beta, eps, Xq8, a_scale)
+PyObject *layernorm_rotate_smooth_quantize_c8(PyObject *, PyObject *const *args, Py_ssize_t n)
+{
+    QVGGT_GUARD_BEGIN
+    Args in{args, n};
+    auto *h = in.handle();
+    const int64_t K = in.integer();
+    const Tensor &X = in.rows(K);
+    const Tensor &gamma = in.exact(at::kFloat, K, -1), &beta = in.exact(at::kFloat, K, -1);
+    const float eps = (float)in.real();
+    return release_items(quantize(in, X, at::kChar, K, -1, [&](const void *x, int64_t ldx, int M, void *q, float *a, void *st) {
+        return qvggt_layernorm_rotate_smooth_quantize_c8(h, x, ldx, M, static_cast<const float *>(gamma.data_ptr()), static_cast<const float *>(beta.data_ptr()),
+                                                         eps, static_cast<S8 *>(q), a, st);
+    }));
+    QVGGT_GUARD_END
+}
+
+// (handle, N, K, X, w_scratch, Xq8, a_scale)
+PyObject *rotate_smooth_quantize_c8_expand(PyObject *, PyObject *const *args, Py_ssize_t n)
+{
+    QVGGT_GUARD_BEGIN
+    Args in{args, n};
+    auto *h = in.handle();
+    const int64_t N = in.integer(), K = in.integer();
+    const Tensor &X = in.rows(K);
+    const Tensor &scratch = in.at_least(at::kChar, N * K);
+    return release_items(quantize(in, X, at::kChar, K, -1, [&](const void *x, int64_t ldx, int M, void *q, float *a, void *st) {
+        return qvggt_rotate_smooth_quantize_c8_expand(h, x, ldx, M, static_cast<S8 *>(q), a, static_cast<S8 *>(scratch.data_ptr()), st);
+    }));
+    QVGGT_GUARD_END
+}
+
+// (handle, N, K, Xq, a_scale, group, Y)
+PyObject *w4a4_linear(PyObject *, PyObject *const *args, Py_ssize_t n)
+{
+    QVGGT_GUARD_BEGIN
+    Args in{args, n};
+    auto *h = in.handle();
+    const int64_t N = in.integer(), K = in.integer();
+    const Tensor &xq = in.at_least(at::kByte, 0);
+    if (!in.ok || xq.dim() != 2 || xq.size(1) != K / 2) Py_RETURN_NONE;
+    const Tensor &as = in.at_least(at::kFloat, 0);
+    const int64_t group = in.integer();
+    if (!in.ok || (group != 0 && group != 128) || as.numel() < xq.size(0) * (group ? K / 128 : 1)) Py_RETURN_NONE;
+    return linear(in, xq, as, N, [&](const void *q, const float *a, int M, void *y, int64_t ldy, void *st) {
+        return qvggt_w4a4_linear(h, static_cast<const U8 *>(q), a, M, (int)group, y, ldy, nullptr, st);
+    });
+    QVGGT_GUARD_END
+}
+
+// (handle, N, K, Xq8, a_scale, Y)
+template <int (*FN)(const qvggt_weights_t *, const S8 *, const float *, int, void *, long long, int *, void *), bool GROUPED>
+PyObject *linear_c8(PyObject *, PyObject *const *args, Py_ssize_t n)
+{
+    QVGGT_GUARD_BEGIN
+    Args in{args, n};
+    auto *h = in.handle();
+    const int64_t N = in.integer(), K = in.integer();
+    const Tensor &xq = in.at_least(at::kChar, 0);
+    if (!in.ok || xq.dim() != 2 || xq.size(1) != K) Py_RETURN_NONE;
+    const Tensor &as = in.at_least(at::kFloat, xq.size(0) * (GROUPED ? K / 128 : 1));
+    return linear(in, xq, as, N, [&](const void *q, const float *a, int M, void *y, int64_t ldy, void *st) {
+        return FN(h, static_cast<const S8 *>(q), a, M, y, ldy, nullptr, st);
+    });
+    QVGGT_GUARD_END
+}
+
+// (handle, N, K, Xq8, a_scale, w_scratch, Y)
+template <bool EXPANDED>
+PyObject *linear_scratch(PyObject *, PyObject *const *args, Py_ssize_t n)
+{
+    QVGGT_GUARD_BEGIN
+    Args in{args, n};
+    auto *h = in.handle();
+    const int64_t N = in.integer(), K = in.integer();
+    const Tensor &xq = in.at_least(at::kChar, 0);
+    if (!in.ok || xq.dim() != 2 || xq.size(1) != K) Py_RETURN_NONE;
+    const Tensor &as = in.at_least(at::kFloat, xq.size(0));
+    const Tensor &scratch = in.at_least(at::kChar, N * K);
+    return linear(in, xq, as, N, [&](const void *q, const float *a, int M, void *y, int64_t ldy, void *st) {
+        S8 *w = static_cast<S8 *>(scratch.data_ptr());
+        return EXPANDED ? qvggt_w4a4_linear_c8_expanded(h, static_cast<const S8 *>(q), a, M, y, ldy, w, nullptr, st)
+                        : qvggt_w4a4_linear_c8_packed_weights(h, static_cast<const S8 *>(q), a, M, y, ldy, w, nullptr, st);
+    });
+    QVGGT_GUARD_END
+}
+
+// (pointer, kind, d0, d1): copy of a device array as a new tensor on the current device; d1 < 0: one dimension.
+// kind: 0 uint8, 1 int8, 2 float32, 3 bfloat16
+PyObject *copy_array(PyObject *, PyObject *const *args, Py_ssize_t n)
+{
+    QVGGT_GUARD_BEGIN
+    Args in{args, n};
+    void *p = const_cast<qvggt_weights_t *>(in.handle());
+    const int64_t kind = in.integer(), d0 = in.integer(), d1 = in.integer();
+    if (!in.done() || kind < 0 || kind > 3) Py_RETURN_NONE;
+    static const ScalarType types[4] = {at::kByte, at::kChar, at::kFloat, at::kBFloat16};
+    const auto options = at::TensorOptions().dtype(types[kind]).device(at::kCUDA, c10::cuda::getCurrentCUDAStream().device_index());
+    return THPVariable_Wrap((d1 < 0 ? at::from_blob(p, {d0}, options) : at::from_blob(p, {d0, d1}, options)).clone());
+    QVGGT_GUARD_END
+}
+
+#define FAST(name, fn) {name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(static_cast<PyObject *(*)(PyObject *, PyObject *const *, Py_ssize_t)>(fn))), METH_FASTCALL, nullptr}
+PyMethodDef methods[] = {
+    FAST("rotate_smooth_quantize", rotate_smooth_quantize),
+    FAST("w4a4_linear", w4a4_linear),
+    FAST("rotate_smooth_quantize_c8", (quantize_c8<qvggt_rotate_smooth_quantize_c8, false>)),
+    FAST("rotate_smooth_quantize_c8_grouped", (quantize_c8<qvggt_rotate_smooth_quantize_c8_grouped, true>)),
+    FAST("gelu_rotate_smooth_quantize_c8", (quantize_c8<qvggt_gelu_rotate_smooth_quantize_c8, false>)),
+    FAST("layernorm_rotate_smooth_quantize_c8", layernorm_rotate_smooth_quantize_c8),
+    FAST("rotate_smooth_quantize_static_c8", rotate_smooth_quantize_static_c8),
+    FAST("rotate_smooth_quantize_tc", rotate_smooth_quantize_tc),
+    FAST("rotate_smooth_quantize_c8_expand", rotate_smooth_quantize_c8_expand),
+    FAST("w4a4_linear_c8", (linear_c8<qvggt_w4a4_linear_c8, false>)),
+    FAST("w4a4_linear_c8_grouped", (linear_c8<qvggt_w4a4_linear_c8_grouped, true>)),
+    FAST("w4a4_linear_c8_packed_weights", (linear_scratch<false>)),
+    FAST("w4a4_linear_c8_expanded", (linear_scratch<true>)),
+    FAST("copy_array", copy_array),
+    {nullptr, nullptr, 0, nullptr}};
+
+PyModuleDef module = {PyModuleDef_HEAD_INIT, "_qvggt_fastcall", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
+
+}  // namespace
+
+PyMODINIT_FUNC PyInit__qvggt_fastcall() { return PyModule_Create(&module); }

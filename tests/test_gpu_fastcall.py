@@ -1,0 +1,86 @@
+"""The extension module's call path against the ctypes one: same results, same objects handed back, same errors."""
+import pytest
+import torch
+
+import paper_2509_21302_b200 as q
+from paper_2509_21302_b200 import binding
+
+pytestmark = pytest.mark.gpu
+
+
+def _handles(K, N):
+    g = torch.Generator(device="cuda").manual_seed(K + N)
+    W = (torch.randn(N, K, generator=g, device="cuda") * 0.02).bfloat16()
+    b = (torch.randn(N, generator=g, device="cuda") * 0.01).bfloat16()
+    c = torch.rand(K, generator=g, device="cuda") + 0.5
+    return q.prepare_weights(W, b, c, None, c8=True), q.prepare_weights(W, b, c, None), g
+
+
+def _calls(h, hp, x, g, K, N, given):
+    """Every call of the fast path; `given`: the caller's own output tensors, or none."""
+    M = x.shape[0]
+    dev = dict(device="cuda")
+    gamma, beta = torch.rand(K, generator=g, **dev), torch.rand(K, generator=g, **dev)
+    delta, scratch = torch.tensor([0.2], **dev), torch.empty(N * K + 16, dtype=torch.int8, **dev)
+
+    def outs(codes, scales):
+        return (torch.empty(M, codes, dtype=torch.uint8 if codes < K else torch.int8, **dev), torch.empty((M, scales) if scales else (M,), **dev)) if given else (None, None)
+
+    y = (lambda: torch.empty(M, N + 8, dtype=torch.bfloat16, **dev)[:, :N]) if given else (lambda: None)
+    res = []
+    for f, lin, o in (
+            (lambda a, b: q.rotate_smooth_quantize(h, x, 0, a, b), lambda c, s: q.w4a4_linear(h, c, s, 0, y()), outs(K // 2, 0)),
+            (lambda a, b: q.rotate_smooth_quantize(h, x, 128, a, b), lambda c, s: q.w4a4_linear(h, c, s, 128, y()), outs(K // 2, K // 128)),
+            (lambda a, b: q.rotate_smooth_quantize_c8(h, x, a, b), lambda c, s: q.w4a4_linear_c8(h, c, s, y()), outs(K, 0)),
+            (lambda a, b: q.rotate_smooth_quantize_c8(hp, x, a, b), lambda c, s: q.w4a4_linear_c8_packed_weights(hp, c, s, scratch, y()), outs(K, 0)),
+            (lambda a, b: q.rotate_smooth_quantize_c8_expand(hp, x, scratch, a, b), lambda c, s: q.w4a4_linear_c8_expanded(hp, c, s, scratch, y()), outs(K, 0)),
+            (lambda a, b: q.rotate_smooth_quantize_c8_grouped(h, x, a, b), lambda c, s: q.w4a4_linear_c8_grouped(h, c, s, y()), outs(K, K // 128)),
+            (lambda a, b: q.rotate_smooth_quantize_static_c8(h, x, delta, a, b), None, outs(K, 0)),
+            (lambda a, b: q.layernorm_rotate_smooth_quantize_c8(h, x, gamma, beta, 1e-5, a, b), None, outs(K, 0)),
+            (lambda a, b: q.gelu_rotate_smooth_quantize_c8(h, x, a, b), None, outs(K, 0)),
+            (lambda a, b: q.rotate_smooth_quantize_tc(h, x, True, a, b), None, outs(K, 0)),
+            (lambda a, b: q.rotate_smooth_quantize_tc(h, x, False, a, b), None, outs(K // 2, 0))):
+        c, s = f(*o)
+        if given:
+            assert c is o[0] and s is o[1]
+        res += [c, s]
+        if lin is not None:
+            res.append(lin(c, s))
+    return res
+
+
+@pytest.mark.parametrize("given", [False, True])
+@pytest.mark.parametrize("K,N,M,pad", [(1024, 256, 1, 0), (1024, 256, 131, 64), (4096, 128, 3, 8), (1024, 128, 0, 0)])
+def test_same_results_as_through_ctypes(K, N, M, pad, given, monkeypatch):
+    h, hp, g = _handles(K, N)
+    x = torch.randn(M, K + pad, generator=g, device="cuda").bfloat16()[:, :K]
+    st = g.get_state()
+    fast = _calls(h, hp, x, g, K, N, given)
+    g.set_state(st)
+    monkeypatch.setattr(binding, "_fast", None)
+    slow = _calls(h, hp, x, g, K, N, given)
+    monkeypatch.undo()
+    assert len(fast) == len(slow)
+    for a, b in zip(fast, slow):
+        assert a.shape == b.shape and a.dtype == b.dtype and a.stride() == b.stride() and a.device == b.device and torch.equal(a, b)
+
+
+def test_same_errors_as_through_ctypes():
+    K, N, M = 1024, 128, 5
+    h, hp, g = _handles(K, N)
+    x = torch.randn(M, K, generator=g, device="cuda").bfloat16()
+    xq, a = q.rotate_smooth_quantize_c8(h, x)
+    for bad in (lambda: q.rotate_smooth_quantize_c8(h, x.float()), lambda: q.rotate_smooth_quantize_c8(h, x.cpu()), lambda: q.rotate_smooth_quantize_c8(h, x[:, :512]),
+                lambda: q.rotate_smooth_quantize_c8(h, x, xq.view(torch.uint8), a), lambda: q.w4a4_linear_c8(h, xq[:, ::2], a),
+                lambda: q.w4a4_linear_c8(h, xq, a.double()), lambda: q.w4a4_linear_c8(h, xq, a, torch.empty(M, N + 1, device="cuda").bfloat16())):
+        with pytest.raises(AssertionError):
+            bad()
+    with pytest.raises(q.QvggtError) as e:        # no one-code-per-byte copy in this handle
+        q.w4a4_linear_c8(hp, xq, a)
+    assert e.value.status == -4
+    with pytest.raises(q.QvggtError) as e:        # row stride not a multiple of 8
+        q.rotate_smooth_quantize_c8(h, torch.empty(M, K + 4, device="cuda").bfloat16()[:, :K])
+    assert e.value.status == -3
+    h.free()
+    with pytest.raises(RuntimeError):
+        q.rotate_smooth_quantize_c8(h, x)
