@@ -34,48 +34,54 @@ using gemmc::Ring;
 using gemmc::STG_BYTES;
 
 constexpr int BM = 128;            // token rows per CTA (TMEM lanes)
-constexpr int BN = 256;            // output channels per whole tile
 constexpr int BK = 128;            // codes along K per stage = one 128-byte swizzled row
 constexpr int ACC_BUFS = 2;        // TMEM accumulators: the epilogue of tile i overlaps the MMAs of tile i+1
 constexpr int EPI_WARPS = 8;       // warp w: TMEM lane quarter w % 4, column part w / 4
 constexpr int MMA_WARP = EPI_WARPS;
 constexpr int TMA_WARP = EPI_WARPS + 1;
 constexpr int THREADS = (EPI_WARPS + 2) * 32;
-constexpr int B_ROWS = BN / 2;                         // weight rows staged by one CTA for a whole tile
-constexpr int STAGE = (BM + B_ROWS) * BK;              // 32 KB
-constexpr int STAGES = 6;
-constexpr int OFF_STG = STAGES * STAGE;                // operand stages first: they need 1024-byte alignment
-constexpr int OFF_CH = OFF_STG + EPI_WARPS * STG_BYTES;          // per-channel scale and bias of two tiles, fp32
-constexpr int OFF_BAR = OFF_CH + 2 * ACC_BUFS * BN * 4;          // full[STAGES] empty[STAGES] tfull[2] tempty[2]
-constexpr int NBARS = 2 * STAGES + 2 * ACC_BUFS;
-constexpr int OFF_TMEM = OFF_BAR + NBARS * 8;
-constexpr int OFF_ABORT = OFF_TMEM + 4;
-constexpr int OFF_FLAGS = OFF_ABORT + 4;
-constexpr int SMEM_BYTES = OFF_FLAGS + 8;
-constexpr int DYN_SMEM = SMEM_BYTES + 1024;            // slack to align the base to 1024 bytes
-constexpr int TMEM_COLS = ACC_BUFS * BN;               // 512
-static_assert(DYN_SMEM <= 232448, "exceeds the 227 KB of shared memory a CTA may use");
-static_assert(2 * STAGE < (1 << 20), "transaction count of a stage must fit the barrier");
+
+// BN = output channels per tile: 256, or 128 where that keeps more of the chip busy (see wide_tiles()).
+template <int BN>
+struct Lay {
+    static constexpr int B_ROWS = BN / 2;                         // weight rows staged by one CTA
+    static constexpr int STAGE = (BM + B_ROWS) * BK;              // 32 / 24 KB
+    static constexpr int STAGES = BN == 256 ? 6 : 8;
+    static constexpr int OFF_STG = STAGES * STAGE;                // operand stages first: they need 1024-byte alignment
+    static constexpr int OFF_CH = OFF_STG + EPI_WARPS * STG_BYTES;          // per-channel scale and bias of two tiles, fp32
+    static constexpr int OFF_BAR = OFF_CH + 2 * ACC_BUFS * BN * 4;          // full[STAGES] empty[STAGES] tfull[2] tempty[2]
+    static constexpr int NBARS = 2 * STAGES + 2 * ACC_BUFS;
+    static constexpr int OFF_TMEM = OFF_BAR + NBARS * 8;
+    static constexpr int OFF_ABORT = OFF_TMEM + 4;
+    static constexpr int SMEM_BYTES = OFF_ABORT + 4;
+    static constexpr int DYN_SMEM = SMEM_BYTES + 1024;            // slack to align the base to 1024 bytes
+    static constexpr int TMEM_COLS = ACC_BUFS * BN;               // 512 / 256
+    static_assert(DYN_SMEM <= 232448, "exceeds the 227 KB of shared memory a CTA may use");
+    static_assert(2 * STAGE < (1 << 20), "transaction count of a stage must fit the barrier");
+    static_assert(STAGE % 1024 == 0, "operand tiles must stay 1024-byte aligned");
+};
 
 // DUMP: also write the int32 sums to acc_debug (its own instantiation keeps that code out of the production kernel).
 // wait_limit: bound of every device-side wait, in cycles.  skip_loads: the TMA producers issue nothing, so that the
 // first wait for operands runs out (used only to exercise the timeout path; no asynchronous operation is in flight).
-template <bool DUMP>
+template <int BN, bool DUMP>
 __global__ void __launch_bounds__(THREADS, 1)
 gemm_c8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
                const __grid_constant__ CUtensorMap map_y,
                const float *__restrict__ a_scale, const float *__restrict__ w_scale, const uint16_t *__restrict__ bias,
                int *__restrict__ acc_debug, int M, int N, int K, int *status, long long wait_limit, int skip_loads)
 {
+    using L = Lay<BN>;
+    constexpr int STAGES = L::STAGES, STAGE = L::STAGE, B_ROWS = L::B_ROWS, TMEM_COLS = L::TMEM_COLS;
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const uint32_t sbase = ptx::smem_addr(smem);
-    const uint32_t bar_full = sbase + OFF_BAR;
+    const uint32_t bar_full = sbase + L::OFF_BAR;
     const uint32_t bar_empty = bar_full + STAGES * 8;
     const uint32_t bar_tfull = bar_empty + STAGES * 8;
     const uint32_t bar_tempty = bar_tfull + ACC_BUFS * 8;
-    uint32_t *s_tmem = reinterpret_cast<uint32_t *>(smem + OFF_TMEM);
-    volatile int *s_abort = reinterpret_cast<volatile int *>(smem + OFF_ABORT);
+    uint32_t *s_tmem = reinterpret_cast<uint32_t *>(smem + L::OFF_TMEM);
+    volatile int *s_abort = reinterpret_cast<volatile int *>(smem + L::OFF_ABORT);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = ptx::cluster_ctarank();                       // 0 = leader of the pair
@@ -112,9 +118,9 @@ gemm_c8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     if (warp < EPI_WARPS) {
         // ------------------------------------------------------------ epilogue
         const int quarter = warp & 3, cpart = warp >> 2;   // TMEM lane quarter, column part
-        unsigned char *stg = smem + OFF_STG + warp * STG_BYTES;
-        const uint32_t stg_addr = sbase + OFF_STG + warp * STG_BYTES;
-        float *s_ws = reinterpret_cast<float *>(smem + OFF_CH);             // [2][BN] per-channel scale of the tile
+        unsigned char *stg = smem + L::OFF_STG + warp * STG_BYTES;
+        const uint32_t stg_addr = sbase + L::OFF_STG + warp * STG_BYTES;
+        float *s_ws = reinterpret_cast<float *>(smem + L::OFF_CH);             // [2][BN] per-channel scale of the tile
         float *s_bs = s_ws + ACC_BUFS * BN;                                  // [2][BN] bias as fp32
         const uint32_t leader_tempty = ptx::map_to_cta(bar_tempty, 0);
         bool alive = true;
@@ -130,7 +136,7 @@ gemm_c8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
             const bool cols_ok = n0 < N;                       // N is a multiple of 128: a part is all in or all out
             // per-channel scale and bias of the tile -> shared memory; buffer b was last read two tiles ago,
             // and every epilogue warp has passed the group barrier of the tile in between since then
-            gemmc::load_channel_params(s_ws + b * BN, s_bs + b * BN, w_scale, bias, nt0, N, threadIdx.x);
+            if (BN == EPI_WARPS * 32 || threadIdx.x < BN) gemmc::load_channel_params(s_ws + b * BN, s_bs + b * BN, w_scale, bias, nt0, N, threadIdx.x);
             const float as = row_ok ? __ldg(a_scale + gm) : 0.0f;
             const uint64_t as2 = ptx::f32x2_pack(as, as);
             // the epilogue warps meet (named barrier 1: publishes s_ws / s_bs), then every warp polls the accumulator barrier itself
@@ -172,34 +178,39 @@ gemm_c8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
         if (lane == 0) ptx::tma_store_wait_read<0>();
     } else if (warp == MMA_WARP) {
         // ------------------------------------------------------------ MMA issuer (one thread of the leader CTA)
-        if (lane == 0 && rank == 0) {
+        // The whole warp runs the loop and one elected lane issues: warp-uniform control flow lets the descriptors live in
+        // uniform registers, where tcgen05 wants them.
+        if (rank == 0) {
             constexpr uint32_t idesc = ptx::idesc_i8(2 * BM, BN);
             bool alive = true;
             Ring r;
             for (int t = 0; t < my_tiles && alive; ++t) {
                 const int b = t & 1;
                 if (t >= ACC_BUFS) {
-                    alive = ptx::mbar_wait_cluster(bar_tempty + 8 * b, ((t >> 1) - 1) & 1, s_abort, status, QVGGT_DEV_TIMEOUT_TMEM_FREE, wait_limit);
+                    alive = ptx::warp_agrees(ptx::mbar_wait_cluster(bar_tempty + 8 * b, ((t >> 1) - 1) & 1, s_abort, status, QVGGT_DEV_TIMEOUT_TMEM_FREE, wait_limit));
                     if (!alive) break;
                     ptx::tc_fence_after_sync();
                 }
                 const uint32_t d_tmem = tmem_base + b * BN;
                 for (int kb = 0; kb < KB; ++kb) {
-                    alive = ptx::mbar_wait_cluster(bar_full + 8 * r.s, r.ph, s_abort, status, QVGGT_DEV_TIMEOUT_FULL, wait_limit);
+                    alive = ptx::warp_agrees(ptx::mbar_wait_cluster(bar_full + 8 * r.s, r.ph, s_abort, status, QVGGT_DEV_TIMEOUT_FULL, wait_limit));
                     if (!alive) break;
                     ptx::tc_fence_after_sync();
                     const uint32_t a_addr = sbase + r.s * STAGE;
-                    gemmc::mma_kblock_i8<true>(d_tmem, a_addr, a_addr + BM * BK, idesc, kb == 0);
-                    ptx::mma_commit_pair(bar_empty + 8 * r.s, 3);      // frees the stage in both CTAs
+                    if (ptx::elect_one()) {
+                        gemmc::mma_kblock_i8<true>(d_tmem, a_addr, a_addr + BM * BK, idesc, kb == 0);
+                        ptx::mma_commit_pair(bar_empty + 8 * r.s, 3);      // frees the stage in both CTAs
+                        if (kb == KB - 1) ptx::mma_commit_pair(bar_tfull + 8 * b, 3);
+                    }
+                    __syncwarp();
                     r.advance(STAGES);
                 }
-                if (alive) ptx::mma_commit_pair(bar_tfull + 8 * b, 3);
             }
         }
         __syncwarp();
     } else {
-        // ------------------------------------------------------------ TMA producer (one thread per CTA)
-        if (lane == 0 && !skip_loads) {
+        // ------------------------------------------------------------ TMA producer (one thread per CTA; the warp runs uniformly, as above)
+        if (!skip_loads) {
             const uint32_t leader_full = ptx::map_to_cta(bar_full, 0);
             bool alive = true;
             Ring r;
@@ -210,15 +221,18 @@ gemm_c8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
                 const int n0 = (tile % n_tiles) * BN + (int)rank * B_ROWS;
                 for (int kb = 0; kb < KB; ++kb, ++it) {
                     if (it >= STAGES) {
-                        alive = ptx::mbar_wait(bar_empty + 8 * r.s, r.ph ^ 1, s_abort, status, QVGGT_DEV_TIMEOUT_EMPTY, 20, wait_limit);
+                        alive = ptx::warp_agrees(ptx::mbar_wait(bar_empty + 8 * r.s, r.ph ^ 1, s_abort, status, QVGGT_DEV_TIMEOUT_EMPTY, 20, wait_limit));
                         if (!alive) break;
                     }
                     const uint32_t dst = sbase + r.s * STAGE;
                     // the leader's barrier expects the bytes of both CTAs; the peer's completions may arrive first
                     // (the count goes negative for a while), the phase cannot end before the leader has arrived
-                    if (rank == 0) ptx::mbar_arrive_expect_tx(bar_full + 8 * r.s, 2 * STAGE);
-                    ptx::tma_load_2d_pair(&map_x, leader_full + 8 * r.s, dst, kb * BK, m0);
-                    ptx::tma_load_2d_pair(&map_w, leader_full + 8 * r.s, dst + BM * BK, kb * BK, n0);
+                    if (ptx::elect_one()) {
+                        if (rank == 0) ptx::mbar_arrive_expect_tx(bar_full + 8 * r.s, 2 * STAGE);
+                        ptx::tma_load_2d_pair(&map_x, leader_full + 8 * r.s, dst, kb * BK, m0);
+                        ptx::tma_load_2d_pair(&map_w, leader_full + 8 * r.s, dst + BM * BK, kb * BK, n0);
+                    }
+                    __syncwarp();
                     r.advance(STAGES);
                 }
             }
@@ -389,7 +403,7 @@ gemm_c8_grouped_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
         if (lane == 0) ptx::tma_store_wait_read<0>();
     } else if (warp == G_MMA_WARP) {
         // ------------------------------------------------------------ MMA issuer: one accumulator per K-block
-        if (lane == 0 && rank == 0) {
+        if (rank == 0) {                 // the whole warp, one elected lane issuing (see gemm_c8_kernel)
             constexpr uint32_t idesc = ptx::idesc_i8(2 * BM, GN);
             bool alive = true;
             Ring r;
@@ -397,24 +411,27 @@ gemm_c8_grouped_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
             for (int it = 0; it < total_kb && alive; ++it) {
                 const int b = it % GACC;
                 if (it >= GACC) {
-                    alive = ptx::mbar_wait_cluster(bar_tempty + 8 * b, ((it / GACC) - 1) & 1, s_abort, status, QVGGT_DEV_TIMEOUT_TMEM_FREE);
+                    alive = ptx::warp_agrees(ptx::mbar_wait_cluster(bar_tempty + 8 * b, ((it / GACC) - 1) & 1, s_abort, status, QVGGT_DEV_TIMEOUT_TMEM_FREE));
                     if (!alive) break;
                     ptx::tc_fence_after_sync();
                 }
-                alive = ptx::mbar_wait_cluster(bar_full + 8 * r.s, r.ph, s_abort, status, QVGGT_DEV_TIMEOUT_FULL);
+                alive = ptx::warp_agrees(ptx::mbar_wait_cluster(bar_full + 8 * r.s, r.ph, s_abort, status, QVGGT_DEV_TIMEOUT_FULL));
                 if (!alive) break;
                 ptx::tc_fence_after_sync();
                 const uint32_t a_addr = sbase + r.s * GSTAGE;
-                gemmc::mma_kblock_i8<true>(tmem_base + b * GN, a_addr, a_addr + BM * BK, idesc, true);
-                ptx::mma_commit_pair(bar_empty + 8 * r.s, 3);
-                ptx::mma_commit_pair(bar_tfull + 8 * b, 3);
+                if (ptx::elect_one()) {
+                    gemmc::mma_kblock_i8<true>(tmem_base + b * GN, a_addr, a_addr + BM * BK, idesc, true);
+                    ptx::mma_commit_pair(bar_empty + 8 * r.s, 3);
+                    ptx::mma_commit_pair(bar_tfull + 8 * b, 3);
+                }
+                __syncwarp();
                 r.advance(GSTAGES);
             }
         }
         __syncwarp();
     } else {
         // ------------------------------------------------------------ TMA producer (one thread per CTA)
-        if (lane == 0) {
+        {
             const uint32_t leader_full = ptx::map_to_cta(bar_full, 0);
             bool alive = true;
             Ring r;
@@ -425,13 +442,16 @@ gemm_c8_grouped_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
                 const int n0 = (tile % n_tiles) * GN + (int)rank * GB_ROWS;
                 for (int kb = 0; kb < KB; ++kb, ++it) {
                     if (it >= GSTAGES) {
-                        alive = ptx::mbar_wait(bar_empty + 8 * r.s, r.ph ^ 1, s_abort, status, QVGGT_DEV_TIMEOUT_EMPTY, 20);
+                        alive = ptx::warp_agrees(ptx::mbar_wait(bar_empty + 8 * r.s, r.ph ^ 1, s_abort, status, QVGGT_DEV_TIMEOUT_EMPTY, 20));
                         if (!alive) break;
                     }
                     const uint32_t dst = sbase + r.s * GSTAGE;
-                    if (rank == 0) ptx::mbar_arrive_expect_tx(bar_full + 8 * r.s, 2 * GSTAGE);
-                    ptx::tma_load_2d_pair(&map_x, leader_full + 8 * r.s, dst, kb * BK, m0);
-                    ptx::tma_load_2d_pair(&map_w, leader_full + 8 * r.s, dst + BM * BK, kb * BK, n0);
+                    if (ptx::elect_one()) {
+                        if (rank == 0) ptx::mbar_arrive_expect_tx(bar_full + 8 * r.s, 2 * GSTAGE);
+                        ptx::tma_load_2d_pair(&map_x, leader_full + 8 * r.s, dst, kb * BK, m0);
+                        ptx::tma_load_2d_pair(&map_w, leader_full + 8 * r.s, dst + BM * BK, kb * BK, n0);
+                    }
+                    __syncwarp();
                     r.advance(GSTAGES);
                 }
             }
@@ -494,18 +514,19 @@ __global__ void __launch_bounds__(256) unpack_w4_kernel(const uint4 *__restrict_
     qvggt_unpack_w4_item(packed, out, i);
 }
 
-template <bool DUMP>
-cudaError_t launch(const qvggt_weights *w, const signed char *wq8, const signed char *Xq8, const float *a_scale, int M, void *Y, long long ldy,
+template <int BN, bool DUMP>
+cudaError_t launch_tiles(const qvggt_weights *w, const signed char *wq8, const signed char *Xq8, const float *a_scale, int M, void *Y, long long ldy,
                    int *acc_debug, cudaStream_t st, long long wait_limit, int skip_loads)
 {
+    using L = Lay<BN>;
     static QvggtPerDevice cache;
     int max_workers = 0;
-    cudaError_t e = qvggt_configure_kernel(gemm_c8_kernel<DUMP>, THREADS, DYN_SMEM, 2, cache, &max_workers);
+    cudaError_t e = qvggt_configure_kernel(gemm_c8_kernel<BN, DUMP>, THREADS, L::DYN_SMEM, 2, cache, &max_workers);
     if (e != cudaSuccess) return e;
     const int K = w->K, N = w->N;
     CUtensorMap map_x, map_w, map_y;
     if (!qvggt_make_map(&map_x, CU_TENSOR_MAP_DATA_TYPE_UINT8, Xq8, K, M, K, BK, BM, CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !qvggt_make_map(&map_w, CU_TENSOR_MAP_DATA_TYPE_UINT8, wq8, K, N, K, BK, B_ROWS, CU_TENSOR_MAP_SWIZZLE_128B) ||
+        !qvggt_make_map(&map_w, CU_TENSOR_MAP_DATA_TYPE_UINT8, wq8, K, N, K, BK, L::B_ROWS, CU_TENSOR_MAP_SWIZZLE_128B) ||
         !qvggt_make_map(&map_y, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, Y, N, M, (uint64_t)ldy * 2, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B))
         return cudaErrorInvalidValue;
     const int total_tiles = ((M + 2 * BM - 1) / (2 * BM)) * ((N + BN - 1) / BN);
@@ -518,12 +539,34 @@ cudaError_t launch(const qvggt_weights *w, const signed char *wq8, const signed 
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(workers * 2);
     cfg.blockDim = dim3(THREADS);
-    cfg.dynamicSmemBytes = DYN_SMEM;
+    cfg.dynamicSmemBytes = L::DYN_SMEM;
     cfg.stream = st;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, gemm_c8_kernel<DUMP>, map_x, map_w, map_y, a_scale, (const float *)w->w_scale,
+    return cudaLaunchKernelEx(&cfg, gemm_c8_kernel<BN, DUMP>, map_x, map_w, map_y, a_scale, (const float *)w->w_scale,
                               (const uint16_t *)w->bias, acc_debug, M, N, K, w->status, wait_limit, skip_loads);
+}
+
+// Whether tiles of 256 channels are the faster ones for this shape.  A narrow tile takes 0.6 of a wide one's time per K-block (0.17
+// against 0.27 us) and half its epilogue, so the number of rounds decides: narrow tiles win while they need at most 1.5 times
+// as many (K = 4096, N = 1024: 13.4 -> 9.7 us at 1374 rows, 23.1 -> 21.5 at 5496, but 14.8 -> 15.2 at 2748, 33.1 -> 35.7 at
+// 10 992), and with K = 1024, where the epilogue behind the last K-block weighs as much as the K-blocks, also when they turn a
+// single round into two (N = 1024: 7.0 -> 5.4 us at 1374 rows, 7.6 -> 6.9 at 2748; N = 3072: 8.1 -> 7.8 at 1374; but two
+// rounds into four 11.0 -> 11.4 at 2748).
+bool wide_tiles(int M, int N, int K, int workers)
+{
+    const long long row_tiles = (M + 2 * BM - 1) / (2 * BM);
+    const long long wide = (row_tiles * ((N + 255) / 256) + workers - 1) / workers;
+    const long long narrow = (row_tiles * ((N + 127) / 128) + workers - 1) / workers;
+    return !(2 * narrow <= 3 * wide || (K == 1024 && wide == 1));
+}
+
+template <bool DUMP>
+cudaError_t launch(const qvggt_weights *w, const signed char *wq8, const signed char *Xq8, const float *a_scale, int M, void *Y, long long ldy,
+                   int *acc_debug, cudaStream_t st, long long wait_limit, int skip_loads)
+{
+    if (wide_tiles(M, w->N, w->K, qvggt_sm_count() / 2)) return launch_tiles<256, DUMP>(w, wq8, Xq8, a_scale, M, Y, ldy, acc_debug, st, wait_limit, skip_loads);
+    return launch_tiles<128, DUMP>(w, wq8, Xq8, a_scale, M, Y, ldy, acc_debug, st, wait_limit, skip_loads);
 }
 
 }  // namespace

@@ -115,6 +115,24 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols)   /
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
 
+// A warp-uniform answer: all lanes' waits succeeded.  (If one expires, the lanes may see it at different polls; they must leave
+// their common loop together.)
+__device__ __forceinline__ bool warp_agrees(bool ok) { return __all_sync(0xFFFFFFFFu, ok); }
+
+// One lane of the (converged) warp: true for exactly one thread.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t e;
+    asm volatile(
+        "{\n\t"
+        ".reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t"
+        "}\n"
+        : "=r"(e));
+    return e != 0;
+}
+
 __device__ __forceinline__ void tc_fence_before_sync()
 {
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -172,6 +190,29 @@ __device__ __forceinline__ void tmem_ld_32x32(uint32_t taddr, uint32_t (&r)[32])
         : "memory");
 }
 
+// 16 lanes x 64 consecutive columns as 16x256b fragments: of every block of 8 columns, thread i receives columns
+// 2 (i mod 4) and 2 (i mod 4) + 1 of lane base + i / 4, then the same columns of lane base + i / 4 + 8.
+__device__ __forceinline__ void tmem_ld_16x256b_x8(uint32_t taddr, uint32_t (&r)[32])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x256b.x8.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+        : "r"(taddr)
+        : "memory");
+}
+
+// Four 8 x 8 matrices of 16-bit values to shared memory: thread i holds, of matrix j, row i / 4, columns 2 (i mod 4) and + 1 in rj
+// and gives the address of row i mod 8 of matrix i / 8.
+__device__ __forceinline__ void stmatrix_x4(uint32_t saddr, uint32_t r0, uint32_t r1, uint32_t r2, uint32_t r3)
+{
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(saddr), "r"(r0), "r"(r1), "r"(r2), "r"(r3) : "memory");
+}
+
 // 32 lanes x 16 consecutive 32-bit columns
 __device__ __forceinline__ void tmem_ld_32x16(uint32_t taddr, uint32_t (&r)[16])
 {
@@ -201,6 +242,15 @@ __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.
 __device__ __forceinline__ void tmem_ld_wait()
 {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
+// The wait, and no use of the loaded values above it.
+template <int N>
+__device__ __forceinline__ void tmem_ld_wait_for(uint32_t (&r)[N])
+{
+    tmem_ld_wait();
+#pragma unroll
+    for (int i = 0; i < N; ++i) asm volatile("" : "+r"(r[i]));
 }
 
 // ---------------------------------------------------------------- descriptors
@@ -454,6 +504,21 @@ __device__ __forceinline__ uint64_t f32x2_fma(uint64_t a, uint64_t b, uint64_t c
     uint64_t d;
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
     return d;
+}
+
+// a + b on both halves, behind a multiplication that must keep its own rounding.  add.rn.f32x2 fed by mul.rn.f32x2 is contracted
+// into one fused operation by the assembler, and so is fma.rn.f32x2 with a literal 1; with a 1 that it cannot see (one2) the
+// sum a * 1 + b is what is computed: one rounding, one instruction for two additions.
+__device__ __forceinline__ uint64_t f32x2_add_uncontracted(uint64_t a, uint64_t b, uint64_t one2)
+{
+    return f32x2_fma(a, one2, b);
+}
+
+// 1.0f in both halves, from a value that is zero at run time only.
+__device__ __forceinline__ uint64_t f32x2_one(uint32_t zero)
+{
+    const float one = __uint_as_float(0x3F800000u + zero);
+    return f32x2_pack(one, one);
 }
 
 // two fp32 -> packed bf16 pair, round-to-nearest-even; `lo` lands in bits 0-15
