@@ -178,39 +178,37 @@ gemm_c8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
         if (lane == 0) ptx::tma_store_wait_read<0>();
     } else if (warp == MMA_WARP) {
         // ------------------------------------------------------------ MMA issuer (one thread of the leader CTA)
-        // The whole warp runs the loop and one elected lane issues: warp-uniform control flow lets the descriptors live in
-        // uniform registers, where tcgen05 wants them.
-        if (rank == 0) {
+        // The thread is chosen by elect.sync, not by its lane number: the assembler then knows that one thread is active and keeps
+        // the descriptors in uniform registers, where tcgen05 wants them (behind `lane == 0` every one is moved there anew, which
+        // made this loop, at 545 cycles per K-block, the bound of the kernel).
+        if (rank == 0 && ptx::elect_one()) {
             constexpr uint32_t idesc = ptx::idesc_i8(2 * BM, BN);
             bool alive = true;
             Ring r;
             for (int t = 0; t < my_tiles && alive; ++t) {
                 const int b = t & 1;
                 if (t >= ACC_BUFS) {
-                    alive = ptx::warp_agrees(ptx::mbar_wait_cluster(bar_tempty + 8 * b, ((t >> 1) - 1) & 1, s_abort, status, QVGGT_DEV_TIMEOUT_TMEM_FREE, wait_limit));
+                    alive = ptx::mbar_wait_cluster(bar_tempty + 8 * b, ((t >> 1) - 1) & 1, s_abort, status, QVGGT_DEV_TIMEOUT_TMEM_FREE, wait_limit);
                     if (!alive) break;
                     ptx::tc_fence_after_sync();
                 }
                 const uint32_t d_tmem = tmem_base + b * BN;
                 for (int kb = 0; kb < KB; ++kb) {
-                    alive = ptx::warp_agrees(ptx::mbar_wait_cluster(bar_full + 8 * r.s, r.ph, s_abort, status, QVGGT_DEV_TIMEOUT_FULL, wait_limit));
+                    alive = ptx::mbar_wait_cluster(bar_full + 8 * r.s, r.ph, s_abort, status, QVGGT_DEV_TIMEOUT_FULL, wait_limit);
                     if (!alive) break;
                     ptx::tc_fence_after_sync();
                     const uint32_t a_addr = sbase + r.s * STAGE;
-                    if (ptx::elect_one()) {
-                        gemmc::mma_kblock_i8<true>(d_tmem, a_addr, a_addr + BM * BK, idesc, kb == 0);
-                        ptx::mma_commit_pair(bar_empty + 8 * r.s, 3);      // frees the stage in both CTAs
-                        if (kb == KB - 1) ptx::mma_commit_pair(bar_tfull + 8 * b, 3);
-                    }
-                    __syncwarp();
+                    gemmc::mma_kblock_i8<true>(d_tmem, a_addr, a_addr + BM * BK, idesc, kb == 0);
+                    ptx::mma_commit_pair(bar_empty + 8 * r.s, 3);      // frees the stage in both CTAs
+                    if (kb == KB - 1) ptx::mma_commit_pair(bar_tfull + 8 * b, 3);
                     r.advance(STAGES);
                 }
             }
         }
         __syncwarp();
     } else {
-        // ------------------------------------------------------------ TMA producer (one thread per CTA; the warp runs uniformly, as above)
-        if (!skip_loads) {
+        // ------------------------------------------------------------ TMA producer (one thread per CTA)
+        if (!skip_loads && ptx::elect_one()) {
             const uint32_t leader_full = ptx::map_to_cta(bar_full, 0);
             bool alive = true;
             Ring r;
@@ -221,18 +219,15 @@ gemm_c8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
                 const int n0 = (tile % n_tiles) * BN + (int)rank * B_ROWS;
                 for (int kb = 0; kb < KB; ++kb, ++it) {
                     if (it >= STAGES) {
-                        alive = ptx::warp_agrees(ptx::mbar_wait(bar_empty + 8 * r.s, r.ph ^ 1, s_abort, status, QVGGT_DEV_TIMEOUT_EMPTY, 20, wait_limit));
+                        alive = ptx::mbar_wait(bar_empty + 8 * r.s, r.ph ^ 1, s_abort, status, QVGGT_DEV_TIMEOUT_EMPTY, 20, wait_limit);
                         if (!alive) break;
                     }
                     const uint32_t dst = sbase + r.s * STAGE;
                     // the leader's barrier expects the bytes of both CTAs; the peer's completions may arrive first
                     // (the count goes negative for a while), the phase cannot end before the leader has arrived
-                    if (ptx::elect_one()) {
-                        if (rank == 0) ptx::mbar_arrive_expect_tx(bar_full + 8 * r.s, 2 * STAGE);
-                        ptx::tma_load_2d_pair(&map_x, leader_full + 8 * r.s, dst, kb * BK, m0);
-                        ptx::tma_load_2d_pair(&map_w, leader_full + 8 * r.s, dst + BM * BK, kb * BK, n0);
-                    }
-                    __syncwarp();
+                    if (rank == 0) ptx::mbar_arrive_expect_tx(bar_full + 8 * r.s, 2 * STAGE);
+                    ptx::tma_load_2d_pair(&map_x, leader_full + 8 * r.s, dst, kb * BK, m0);
+                    ptx::tma_load_2d_pair(&map_w, leader_full + 8 * r.s, dst + BM * BK, kb * BK, n0);
                     r.advance(STAGES);
                 }
             }
@@ -403,7 +398,7 @@ gemm_c8_grouped_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
         if (lane == 0) ptx::tma_store_wait_read<0>();
     } else if (warp == G_MMA_WARP) {
         // ------------------------------------------------------------ MMA issuer: one accumulator per K-block
-        if (rank == 0) {                 // the whole warp, one elected lane issuing (see gemm_c8_kernel)
+        if (rank == 0 && ptx::elect_one()) {      // see gemm_c8_kernel
             constexpr uint32_t idesc = ptx::idesc_i8(2 * BM, GN);
             bool alive = true;
             Ring r;
@@ -411,27 +406,24 @@ gemm_c8_grouped_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
             for (int it = 0; it < total_kb && alive; ++it) {
                 const int b = it % GACC;
                 if (it >= GACC) {
-                    alive = ptx::warp_agrees(ptx::mbar_wait_cluster(bar_tempty + 8 * b, ((it / GACC) - 1) & 1, s_abort, status, QVGGT_DEV_TIMEOUT_TMEM_FREE));
+                    alive = ptx::mbar_wait_cluster(bar_tempty + 8 * b, ((it / GACC) - 1) & 1, s_abort, status, QVGGT_DEV_TIMEOUT_TMEM_FREE);
                     if (!alive) break;
                     ptx::tc_fence_after_sync();
                 }
-                alive = ptx::warp_agrees(ptx::mbar_wait_cluster(bar_full + 8 * r.s, r.ph, s_abort, status, QVGGT_DEV_TIMEOUT_FULL));
+                alive = ptx::mbar_wait_cluster(bar_full + 8 * r.s, r.ph, s_abort, status, QVGGT_DEV_TIMEOUT_FULL);
                 if (!alive) break;
                 ptx::tc_fence_after_sync();
                 const uint32_t a_addr = sbase + r.s * GSTAGE;
-                if (ptx::elect_one()) {
-                    gemmc::mma_kblock_i8<true>(tmem_base + b * GN, a_addr, a_addr + BM * BK, idesc, true);
-                    ptx::mma_commit_pair(bar_empty + 8 * r.s, 3);
-                    ptx::mma_commit_pair(bar_tfull + 8 * b, 3);
-                }
-                __syncwarp();
+                gemmc::mma_kblock_i8<true>(tmem_base + b * GN, a_addr, a_addr + BM * BK, idesc, true);
+                ptx::mma_commit_pair(bar_empty + 8 * r.s, 3);
+                ptx::mma_commit_pair(bar_tfull + 8 * b, 3);
                 r.advance(GSTAGES);
             }
         }
         __syncwarp();
     } else {
         // ------------------------------------------------------------ TMA producer (one thread per CTA)
-        {
+        if (ptx::elect_one()) {
             const uint32_t leader_full = ptx::map_to_cta(bar_full, 0);
             bool alive = true;
             Ring r;
@@ -442,16 +434,13 @@ gemm_c8_grouped_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
                 const int n0 = (tile % n_tiles) * GN + (int)rank * GB_ROWS;
                 for (int kb = 0; kb < KB; ++kb, ++it) {
                     if (it >= GSTAGES) {
-                        alive = ptx::warp_agrees(ptx::mbar_wait(bar_empty + 8 * r.s, r.ph ^ 1, s_abort, status, QVGGT_DEV_TIMEOUT_EMPTY, 20));
+                        alive = ptx::mbar_wait(bar_empty + 8 * r.s, r.ph ^ 1, s_abort, status, QVGGT_DEV_TIMEOUT_EMPTY, 20);
                         if (!alive) break;
                     }
                     const uint32_t dst = sbase + r.s * GSTAGE;
-                    if (ptx::elect_one()) {
-                        if (rank == 0) ptx::mbar_arrive_expect_tx(bar_full + 8 * r.s, 2 * GSTAGE);
-                        ptx::tma_load_2d_pair(&map_x, leader_full + 8 * r.s, dst, kb * BK, m0);
-                        ptx::tma_load_2d_pair(&map_w, leader_full + 8 * r.s, dst + BM * BK, kb * BK, n0);
-                    }
-                    __syncwarp();
+                    if (rank == 0) ptx::mbar_arrive_expect_tx(bar_full + 8 * r.s, 2 * GSTAGE);
+                    ptx::tma_load_2d_pair(&map_x, leader_full + 8 * r.s, dst, kb * BK, m0);
+                    ptx::tma_load_2d_pair(&map_w, leader_full + 8 * r.s, dst + BM * BK, kb * BK, n0);
                     r.advance(GSTAGES);
                 }
             }
@@ -547,12 +536,12 @@ cudaError_t launch_tiles(const qvggt_weights *w, const signed char *wq8, const s
                               (const uint16_t *)w->bias, acc_debug, M, N, K, w->status, wait_limit, skip_loads);
 }
 
-// Whether tiles of 256 channels are the faster ones for this shape.  A narrow tile takes 0.6 of a wide one's time per K-block (0.17
-// against 0.27 us) and half its epilogue, so the number of rounds decides: narrow tiles win while they need at most 1.5 times
-// as many (K = 4096, N = 1024: 13.4 -> 9.7 us at 1374 rows, 23.1 -> 21.5 at 5496, but 14.8 -> 15.2 at 2748, 33.1 -> 35.7 at
-// 10 992), and with K = 1024, where the epilogue behind the last K-block weighs as much as the K-blocks, also when they turn a
-// single round into two (N = 1024: 7.0 -> 5.4 us at 1374 rows, 7.6 -> 6.9 at 2748; N = 3072: 8.1 -> 7.8 at 1374; but two
-// rounds into four 11.0 -> 11.4 at 2748).
+// Whether tiles of 256 channels are the faster ones for this shape.  A narrow tile takes 0.55 of a wide one's time per K-block
+// (0.15 against 0.27 us) and half its epilogue, so the number of rounds decides: narrow tiles win while they need at most 1.5
+// times as many (wide / narrow, us: K = 4096, N = 1024: 13.4 / 9.4 at 1374 rows, 22.9 / 20.1 at 5496, but 24.0 / 26.1 at 8244,
+// 32.9 / 33.8 at 10 992), and with K = 1024, where the epilogue behind the last K-block weighs as much as the K-blocks, also when
+// they turn a single round into two (N = 1024: 7.0 / 5.4 at 1374 rows, 7.5 / 7.0 at 2748; two rounds into four: N = 3072
+// 10.7 / 11.5 at 2748 rows).
 bool wide_tiles(int M, int N, int K, int workers)
 {
     const long long row_tiles = (M + 2 * BM - 1) / (2 * BM);

@@ -215,7 +215,7 @@ gemm_w4a4_grouped_kernel(const __grid_constant__ CUtensorMap map_x, const __grid
                                                QVGGT_DEV_TIMEOUT_PACKED, QVGGT_DEV_TIMEOUT_EMPTY);
     } else if (warp == MMA_WARP) {
         // ------------------------------------------------------------ MMA issuer: one accumulator per K-block
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             constexpr uint32_t idesc = ptx::idesc_i8(BM, BN);
             bool alive = true;
             const int total_kb = my_tiles * KB;
@@ -237,7 +237,7 @@ gemm_w4a4_grouped_kernel(const __grid_constant__ CUtensorMap map_x, const __grid
         __syncwarp();
     } else {
         // ------------------------------------------------------------ TMA producer
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             bool alive = true;
             int it = 0;
             for (int t = 0; t < my_tiles && alive; ++t) {

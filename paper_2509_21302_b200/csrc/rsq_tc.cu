@@ -285,7 +285,7 @@ rsq_tc_kernel(const __grid_constant__ CUtensorMap map_x, int M, const float *__r
         }
     } else if (warp == MMA_WARP) {
         // ------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             constexpr uint32_t idesc = ptx::idesc_bf16_f32(128, NCOL, true);
             bool alive = true;
             int s = 0;
@@ -314,7 +314,7 @@ rsq_tc_kernel(const __grid_constant__ CUtensorMap map_x, int M, const float *__r
         __syncwarp();
     } else {
         // ------------------------------------------------------------ TMA producer
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             bool alive = true;
             int s = 0;
             uint32_t ph = 0;

@@ -115,10 +115,6 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols)   /
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols) : "memory");
 }
 
-// A warp-uniform answer: all lanes' waits succeeded.  (If one expires, the lanes may see it at different polls; they must leave
-// their common loop together.)
-__device__ __forceinline__ bool warp_agrees(bool ok) { return __all_sync(0xFFFFFFFFu, ok); }
-
 // One lane of the (converged) warp: true for exactly one thread.
 __device__ __forceinline__ bool elect_one()
 {
