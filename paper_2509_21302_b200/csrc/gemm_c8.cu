@@ -67,7 +67,7 @@ struct Lay {
 template <int BN, bool DUMP>
 __global__ void __launch_bounds__(THREADS, 1)
 gemm_c8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
-               const __grid_constant__ CUtensorMap map_y,
+               uint16_t *__restrict__ Y, long long ldy,
                const float *__restrict__ a_scale, const float *__restrict__ w_scale, const uint16_t *__restrict__ bias,
                int *__restrict__ acc_debug, int M, int N, int K, int *status, long long wait_limit, int skip_loads)
 {
@@ -103,7 +103,6 @@ gemm_c8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     if (warp == TMA_WARP && lane == 0) {
         ptx::prefetch_tensormap(&map_x);
         ptx::prefetch_tensormap(&map_w);
-        ptx::prefetch_tensormap(&map_y);
     }
     ptx::tc_fence_before_sync();
     __syncthreads();
@@ -123,22 +122,26 @@ gemm_c8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
         float *s_ws = reinterpret_cast<float *>(smem + L::OFF_CH);             // [2][BN] per-channel scale of the tile
         float *s_bs = s_ws + ACC_BUFS * BN;                                  // [2][BN] bias as fp32
         const uint32_t leader_tempty = ptx::map_to_cta(bar_tempty, 0);
+        const uint64_t one2 = ptx::f32x2_one(N & 127);                       // N is a multiple of 128
         bool alive = true;
-        constexpr int CW = BN / 2, NCH = CW / 32;              // columns and 32-column chunks of one warp's part
+        constexpr int CW = BN / 2, NCH = CW / 64;              // columns and 64-column chunks of one warp's part
         for (int t = 0; t < my_tiles; ++t) {
             const int tile = worker + t * workers;
             const int m0 = (tile / n_tiles) * (2 * BM) + (int)rank * BM + quarter * 32;
             const int nt0 = (tile % n_tiles) * BN;             // first channel of the tile
             const int n0 = nt0 + cpart * CW;                   // first channel of this warp's part
             const int b = t & 1;
-            const int gm = m0 + lane;
-            const bool row_ok = gm < M;
             const bool cols_ok = n0 < N;                       // N is a multiple of 128: a part is all in or all out
             // per-channel scale and bias of the tile -> shared memory; buffer b was last read two tiles ago,
             // and every epilogue warp has passed the group barrier of the tile in between since then
             if (BN == EPI_WARPS * 32 || threadIdx.x < BN) gemmc::load_channel_params(s_ws + b * BN, s_bs + b * BN, w_scale, bias, nt0, N, threadIdx.x);
-            const float as = row_ok ? __ldg(a_scale + gm) : 0.0f;
-            const uint64_t as2 = ptx::f32x2_pack(as, as);
+            uint64_t as2[2][2];                                // rows lane / 4 + 8 h of the warp's 16 u .. 16 u + 15
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int gm = m0 + 8 * u + (lane >> 2);
+                const float as = gm < M ? __ldg(a_scale + gm) : 0.0f;
+                as2[u >> 1][u & 1] = ptx::f32x2_pack(as, as);
+            }
             // the epilogue warps meet (named barrier 1: publishes s_ws / s_bs), then every warp polls the accumulator barrier itself
             asm volatile("bar.sync %0, %1;" ::"r"(1), "r"(EPI_WARPS * 32) : "memory");
             {
@@ -150,32 +153,29 @@ gemm_c8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
             if (alive) {
                 const float *wsb = s_ws + b * BN + cpart * CW;
                 const float *bsb = s_bs + b * BN + cpart * CW;
-                // the warp's whole share of the accumulator goes to registers first, so that tensor memory is
-                // handed back to the MMA thread a few hundred cycles after the tile completed, not after the
-                // conversions and stores of the first chunks
-                uint32_t raw[NCH][32];
-#pragma unroll
-                for (int c = 0; c < NCH; ++c)
-                    ptx::tmem_ld_32x32(tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + b * BN + cpart * CW + c * 32, raw[c]);
-                ptx::tmem_ld_wait();
-                ptx::tc_fence_before_sync();
-                __syncwarp();
-                if (lane == 0) ptx::mbar_arrive_cluster(leader_tempty + 8 * b);
 #pragma unroll
                 for (int c = 0; c < NCH; ++c) {
-                    const int col = c * 32;                               // within this warp's columns
+                    uint32_t raw[2][32];
+#pragma unroll
+                    for (int u = 0; u < 2; ++u)
+                        ptx::tmem_ld_16x256b_x8(tmem_base + (static_cast<uint32_t>(quarter * 32 + 16 * u) << 16) + b * BN + cpart * CW + c * 64, raw[u]);
+                    ptx::tmem_ld_wait();
+                    if (c == NCH - 1) {                        // tensor memory goes back to the MMA thread
+                        ptx::tc_fence_before_sync();
+                        __syncwarp();
+                        if (lane == 0) ptx::mbar_arrive_cluster(leader_tempty + 8 * b);
+                    }
                     if (cols_ok) {
-                        uint32_t out[16];
-                        gemmc::scale_bias_bf16_x32(raw[c], as2, wsb + col, bsb + col, out);
-                        gemmc::stage_row_32(stg, out, lane);
-                        if (DUMP && acc_debug && row_ok) gemmc::dump_acc_x32<0>(acc_debug + (long long)gm * N + n0 + col, raw[c]);
-                        gemmc::store_staged_32x32(&map_y, stg_addr, n0 + col, m0, m0 < M, lane);
+#pragma unroll
+                        for (int u = 0; u < 2; ++u) {
+                            const int m = m0 + 16 * u, n = n0 + 64 * c;
+                            gemmc::finish_16x64(raw[u], as2[u], wsb + 64 * c, bsb + 64 * c, stg, stg_addr, Y + (long long)m * ldy + n, ldy, M - m, lane, one2);
+                            if (DUMP && acc_debug) gemmc::dump_16x64<0>(acc_debug + (long long)m * N + n, N, raw[u], M - m, lane);
+                        }
                     }
                 }
             }
         }
-        // the staging tiles must outlive the stores' reads; the writes themselves are complete when the grid is
-        if (lane == 0) ptx::tma_store_wait_read<0>();
     } else if (warp == MMA_WARP) {
         // ------------------------------------------------------------ MMA issuer (one thread of the leader CTA)
         // The thread is chosen by elect.sync, not by its lane number: the assembler then knows that one thread is active and keeps
@@ -513,10 +513,9 @@ cudaError_t launch_tiles(const qvggt_weights *w, const signed char *wq8, const s
     cudaError_t e = qvggt_configure_kernel(gemm_c8_kernel<BN, DUMP>, THREADS, L::DYN_SMEM, 2, cache, &max_workers);
     if (e != cudaSuccess) return e;
     const int K = w->K, N = w->N;
-    CUtensorMap map_x, map_w, map_y;
+    CUtensorMap map_x, map_w;
     if (!qvggt_make_map(&map_x, CU_TENSOR_MAP_DATA_TYPE_UINT8, Xq8, K, M, K, BK, BM, CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !qvggt_make_map(&map_w, CU_TENSOR_MAP_DATA_TYPE_UINT8, wq8, K, N, K, BK, L::B_ROWS, CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !qvggt_make_map(&map_y, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, Y, N, M, (uint64_t)ldy * 2, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B))
+        !qvggt_make_map(&map_w, CU_TENSOR_MAP_DATA_TYPE_UINT8, wq8, K, N, K, BK, L::B_ROWS, CU_TENSOR_MAP_SWIZZLE_128B))
         return cudaErrorInvalidValue;
     const int total_tiles = ((M + 2 * BM - 1) / (2 * BM)) * ((N + BN - 1) / BN);
     const int workers = total_tiles < max_workers ? total_tiles : max_workers;
@@ -532,7 +531,7 @@ cudaError_t launch_tiles(const qvggt_weights *w, const signed char *wq8, const s
     cfg.stream = st;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, gemm_c8_kernel<BN, DUMP>, map_x, map_w, map_y, a_scale, (const float *)w->w_scale,
+    return cudaLaunchKernelEx(&cfg, gemm_c8_kernel<BN, DUMP>, map_x, map_w, static_cast<uint16_t *>(Y), ldy, a_scale, (const float *)w->w_scale,
                               (const uint16_t *)w->bias, acc_debug, M, N, K, w->status, wait_limit, skip_loads);
 }
 

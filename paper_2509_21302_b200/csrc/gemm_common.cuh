@@ -78,6 +78,61 @@ __device__ __forceinline__ void scale_bias_bf16_x32(const uint32_t (&raw)[32], u
     }
 }
 
+// 16 rows x 64 channels of a tile as 16x256b fragments (raw[4 b + 2 h + c]: row lane / 4 + 8 h, channel 8 b + 2 (lane mod 4) + c):
+// fl(fl(float(acc) * fl(a_scale * w_scale)) + bias), every operation rounded to nearest, then bf16 (round to nearest even).
+// as2[h] holds a_scale of the thread's row lane / 4 + 8 h in both halves; ws / bs point at the 64 channel scales / biases.
+// The rows then go through 2 KB of the warp's shared memory (16-byte chunk q of a row at q XOR (row mod 8), free of bank
+// conflicts both ways) and from there to global memory as whole 128-byte lines.  Against one row per thread and a TMA store per
+// 32 x 32 tile this reads the channel parameters from shared memory a quarter as often and leaves the TMA engine, which
+// also feeds the operands, alone: 39.0 -> 36.6 us at M = 10 992, K = 1024, N = 4096, 14.0 -> 13.1 us at N = 1024.
+// Y points at row 0, channel 0 of the 16 x 64; only the first `rows` rows are stored.  one2: see ptx::f32x2_add_uncontracted.
+__device__ __forceinline__ void finish_16x64(const uint32_t (&raw)[32], const uint64_t (&as2)[2], const float *ws, const float *bs, unsigned char *stg,
+                                             uint32_t stg_addr, uint16_t *__restrict__ Y, long long ldy, int rows, int lane,
+                                             uint64_t one2)
+{
+    const int t = lane & 3;
+    const uint32_t st_row = stg_addr + (lane & 15) * 128;
+    uint32_t out[16];
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+        const uint64_t w2 = *reinterpret_cast<const uint64_t *>(ws + 8 * b + 2 * t);
+        const uint64_t c2 = *reinterpret_cast<const uint64_t *>(bs + 8 * b + 2 * t);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const uint64_t z = ptx::f32x2_mul(ptx::f32x2_pack(static_cast<float>(static_cast<int>(raw[4 * b + 2 * h])), static_cast<float>(static_cast<int>(raw[4 * b + 2 * h + 1]))),
+                                              ptx::f32x2_mul(as2[h], w2));
+            float y0, y1;
+            ptx::f32x2_unpack(ptx::f32x2_add_uncontracted(z, c2, one2), y0, y1);
+            out[2 * b + h] = ptx::pack_bf16x2(y0, y1);
+        }
+    }
+    __syncwarp();                           // the previous 16 rows have left the staging tile
+#pragma unroll
+    for (int b = 0; b < 8; b += 2)          // matrices (rows 0-7, block b), (rows 8-15, b), (0-7, b + 1), (8-15, b + 1)
+        ptx::stmatrix_x4(st_row + (((b + (lane >> 4)) ^ (lane & 7)) << 4), out[2 * b], out[2 * b + 1], out[2 * b + 2], out[2 * b + 3]);
+    __syncwarp();
+    const int r0 = lane >> 3, q = lane & 7;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int r = 4 * k + r0;
+        const uint4 v = *reinterpret_cast<const uint4 *>(stg + r * 128 + ((q ^ (r & 7)) << 4));
+        if (r < rows) __stcs(reinterpret_cast<uint4 *>(Y + r * ldy + 8 * q), v);
+    }
+}
+
+// The same fragments, raw, to a row-major int32 matrix (debug dump), optionally shifted right (the packed kernel's sums carry a
+// factor of 256).
+template <int SHIFT>
+__device__ __forceinline__ void dump_16x64(int *dst, long long ld, const uint32_t (&raw)[32], int rows, int lane)
+{
+#pragma unroll
+    for (int b = 0; b < 8; ++b)
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            if ((lane >> 2) + 8 * h < rows)
+                *reinterpret_cast<uint2 *>(dst + ((lane >> 2) + 8 * h) * ld + 8 * b + 2 * (lane & 3)) = make_uint2(static_cast<int>(raw[4 * b + 2 * h]) >> SHIFT, static_cast<int>(raw[4 * b + 2 * h + 1]) >> SHIFT);
+}
+
 // Whole warp: waits until the previous TMA store has read the warp's staging tile, writes row `lane` (64-byte rows,
 // 16-byte chunk q kept at q XOR ((lane / 2) mod 4): the 64-byte swizzle the output tensor map expects).
 __device__ __forceinline__ void stage_row_32(unsigned char *stg, const uint32_t (&out)[16], int lane)
@@ -170,6 +225,14 @@ __device__ __forceinline__ void convert_packed_stages(unsigned char *smem, int c
             else ptx::mbar_arrive(ufull_arrive + 8 * us);
         }
     }
+}
+
+// 16 raw int32 sums of one row -> global memory (debug dump).
+__device__ __forceinline__ void dump_acc_x16(int *dst, const uint32_t (&raw)[16])
+{
+    uint4 *d = reinterpret_cast<uint4 *>(dst);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) d[q] = make_uint4(raw[4 * q], raw[4 * q + 1], raw[4 * q + 2], raw[4 * q + 3]);
 }
 
 // 32 raw int32 sums of one row -> global memory (debug dump), optionally shifted right (the packed kernels carry
