@@ -78,7 +78,7 @@ struct C {
 template <bool DUMP>
 __global__ void __launch_bounds__(THREADS, 1)
 gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
-                 const __grid_constant__ CUtensorMap map_y, const float *__restrict__ a_scale,
+                 uint16_t *__restrict__ Y, long long ldy, const float *__restrict__ a_scale,
                  const float *__restrict__ w_scale, const uint16_t *__restrict__ bias, int *__restrict__ acc_debug,
                  int M, int N, int K, int *status)
 {
@@ -123,13 +123,16 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
     if (warp == TMA_WARP && lane == 0) {
         ptx::prefetch_tensormap(&map_x);
         ptx::prefetch_tensormap(&map_w);
-        ptx::prefetch_tensormap(&map_y);
     }
     ptx::tc_fence_before_sync();
     __syncthreads();
     ptx::cluster_sync();                     // the peer's barriers exist before anything arrives on them remotely
     ptx::tc_fence_after_sync();
     const uint32_t tmem_base = *s_tmem;
+    // everything above touched only kernel parameters and on-chip state: it may overlap the tail of the previous
+    // kernel in the stream; the operands (and the output buffer) may not be touched before that kernel is done
+    ptx::grid_launch_dependents();
+    ptx::grid_dependency_wait();
 
     if (warp < EPI_WARPS) {
         // ------------------------------------------------------------ epilogue
@@ -139,6 +142,7 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
         float *s_ws = reinterpret_cast<float *>(smem + C::OFF_CH);          // [2][BN] per-channel scale of the tile
         float *s_bs = s_ws + ACC_BUFS * BN;                                   // [2][BN] bias as fp32
         const uint32_t leader_tempty = ptx::map_to_cta(bar_tempty, 0);
+        const uint64_t one2 = ptx::f32x2_one(N & 127);                       // N is a multiple of 128
         bool alive = true;
         for (int t = 0; t < my_tiles; ++t) {
             const int tile = worker + t * workers;
@@ -146,15 +150,18 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
             const int nt0 = (tile % n_tiles) * BN;             // first channel of the tile
             const int n0 = nt0 + chalf * 128;                  // first channel of this warp's half
             const int b = t & 1;
-            const int gm = m0 + lane;
-            const bool row_ok = gm < M;
             const bool cols_ok = n0 < N;                       // N is a multiple of 128: a half tile is all in or all out
             // per-channel scale and bias of the tile -> shared memory; buffer b was last read two tiles ago,
             // and every epilogue warp has passed the group barrier of the tile in between since then
             gemmc::load_channel_params(s_ws + b * BN, s_bs + b * BN, w_scale, bias, nt0, N, threadIdx.x);   // 256 threads, one channel each
             // a_scale / 256: exact (power of two), cancels the factor 256 carried by the raw accumulator
-            const float as = row_ok ? __fmul_rn(__ldg(a_scale + gm), 0.00390625f) : 0.0f;
-            const uint64_t as2 = ptx::f32x2_pack(as, as);
+            uint64_t as2[2][2];                                // rows lane / 4 + 8 h of the warp's 16 u .. 16 u + 15
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int gm = m0 + 8 * u + (lane >> 2);
+                const float as = gm < M ? __fmul_rn(__ldg(a_scale + gm), 0.00390625f) : 0.0f;
+                as2[u >> 1][u & 1] = ptx::f32x2_pack(as, as);
+            }
             // the epilogue warps meet (named barrier 1: publishes s_ws / s_bs), then every warp polls the accumulator barrier itself
             asm volatile("bar.sync %0, %1;" ::"r"(1), "r"(EPI_WARPS * 32) : "memory");
             {
@@ -166,12 +173,12 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
             if (alive) {
                 const float *wsb = s_ws + b * BN + chalf * 128;
                 const float *bsb = s_bs + b * BN + chalf * 128;
-#pragma unroll 1
-                for (int c = 0; c < 4; ++c) {
-                    const int col = c * 32;                               // within this warp's 128 columns
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {                  // rows 16 u .., channels 64 h .. of the warp's 32 x 128
+                    const int u = c & 1, h = c >> 1, m = m0 + 16 * u, n = n0 + 64 * h;
                     uint32_t raw[32];
-                    ptx::tmem_ld_32x32(tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + b * BN + chalf * 128 + col, raw);
-                    ptx::tmem_ld_wait();
+                    ptx::tmem_ld_16x256b_x8(tmem_base + (static_cast<uint32_t>(quarter * 32 + 16 * u) << 16) + b * BN + chalf * 128 + 64 * h, raw);
+                    ptx::tmem_ld_wait_for(raw);
                     if (c == 3) {
                         // last read of this accumulator: hand it back to the MMA thread before the math
                         ptx::tc_fence_before_sync();
@@ -179,17 +186,13 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
                         if (lane == 0) ptx::mbar_arrive_cluster(leader_tempty + 8 * b);
                     }
                     if (cols_ok) {
-                        uint32_t out[16];
-                        gemmc::scale_bias_bf16_x32(raw, as2, wsb + col, bsb + col, out);
-                        gemmc::stage_row_32(stg, out, lane);
+                        gemmc::finish_16x64(raw, as2[u], wsb + 64 * h, bsb + 64 * h, stg, stg_addr, Y + (long long)m * ldy + n, ldy, M - m, lane, one2);
                         // the raw sums carry a factor 256 (codes in the high half-byte)
-                        if (DUMP && acc_debug && row_ok) gemmc::dump_acc_x32<8>(acc_debug + (long long)gm * N + n0 + col, raw);
-                        gemmc::store_staged_32x32(&map_y, stg_addr, n0 + col, m0, m0 < M, lane);
+                        if (DUMP && acc_debug) gemmc::dump_16x64<8>(acc_debug + (long long)m * N + n, N, raw, M - m, lane);
                     }
                 }
             }
         }
-        if (lane == 0) ptx::tma_store_wait_all();
     } else if (warp < MMA_WARP) {
         // ------------------------------------------------------------ converters
         gemmc::convert_packed_stages<C, true>(smem, warp - CONV_WARP0, lane, my_tiles * KB, bar_pfull, bar_pempty, bar_uempty,
@@ -197,7 +200,10 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
                                               s_flags + 1 + 2 * CONV_WARPS, QVGGT_DEV_TIMEOUT_PACKED, QVGGT_DEV_TIMEOUT_EMPTY);
     } else if (warp == MMA_WARP) {
         // ------------------------------------------------------------ MMA issuer (one thread of the leader CTA)
-        if (lane == 0 && rank == 0) {
+        // The thread is chosen by elect.sync, not by its lane number: the assembler then knows that one thread is active and keeps
+        // the descriptors in uniform registers, where tcgen05 wants them (behind `lane == 0` every one is moved there anew, which
+        // made this loop, at 545 cycles per K-block, the bound of the kernel).
+        if (rank == 0 && ptx::elect_one()) {
             constexpr uint32_t idesc = ptx::idesc_i8(BM * CG, BN);
             bool alive = true;
             int us = 0;
@@ -217,15 +223,15 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
                     const uint32_t a_addr = sbase + C::OFF_UP + us * C::UP_STAGE;
                     gemmc::mma_kblock_i8<true>(d_tmem, a_addr, a_addr + BM * BK, idesc, kb == 0);
                     ptx::mma_commit_pair(bar_uempty + 8 * us, 3);
+                    if (kb == KB - 1) ptx::mma_commit_pair(bar_tfull + 8 * b, 3);
                     if (++us == C::US) { us = 0; uph ^= 1; }
                 }
-                if (alive) ptx::mma_commit_pair(bar_tfull + 8 * b, 3);
             }
         }
         __syncwarp();
     } else {
         // ------------------------------------------------------------ TMA producer (one thread)
-        if (lane == 0) {
+        if (ptx::elect_one()) {
             bool alive = true;
             int ps = 0;
             uint32_t pph = 0;
@@ -268,10 +274,9 @@ cudaError_t launch(const qvggt_weights *w, const unsigned char *Xq, const float 
     cudaError_t e = qvggt_configure_kernel(gemm_w4a4_kernel<DUMP>, THREADS, C::DYN_SMEM, CG, cache, &max_workers);
     if (e != cudaSuccess) return e;
     const int K = w->K, N = w->N;
-    CUtensorMap map_x, map_w, map_y;
+    CUtensorMap map_x, map_w;
     if (!qvggt_make_map(&map_x, CU_TENSOR_MAP_DATA_TYPE_UINT8, Xq, K / 2, M, K / 2, BK / 2, BM, CU_TENSOR_MAP_SWIZZLE_NONE) ||
-        !qvggt_make_map(&map_w, CU_TENSOR_MAP_DATA_TYPE_UINT8, w->Wq, K / 2, N, K / 2, BK / 2, C::B_ROWS, CU_TENSOR_MAP_SWIZZLE_NONE) ||
-        !qvggt_make_map(&map_y, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, Y, N, M, (uint64_t)ldy * 2, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B))
+        !qvggt_make_map(&map_w, CU_TENSOR_MAP_DATA_TYPE_UINT8, w->Wq, K / 2, N, K / 2, BK / 2, C::B_ROWS, CU_TENSOR_MAP_SWIZZLE_NONE))
         return cudaErrorInvalidValue;
     const int total_tiles = ((M + BM * CG - 1) / (BM * CG)) * ((N + BN - 1) / BN);
     const int workers = total_tiles < max_workers ? total_tiles : max_workers;
@@ -280,12 +285,14 @@ cudaError_t launch(const qvggt_weights *w, const unsigned char *Xq, const float 
     cfg.blockDim = dim3(THREADS);
     cfg.dynamicSmemBytes = C::DYN_SMEM;
     cfg.stream = st;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = CG; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, gemm_w4a4_kernel<DUMP>, map_x, map_w, map_y, a_scale, (const float *)w->w_scale,
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = CG; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;      // see grid_dependency_wait()
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, gemm_w4a4_kernel<DUMP>, map_x, map_w, static_cast<uint16_t *>(Y), ldy, a_scale, (const float *)w->w_scale,
                               (const uint16_t *)w->bias, acc_debug, M, N, K, w->status);
 }
 
