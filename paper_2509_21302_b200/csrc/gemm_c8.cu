@@ -331,6 +331,7 @@ gemm_c8_grouped_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
         float *s_ws = reinterpret_cast<float *>(smem + OFF_CH);    // [2][GN]
         float *s_bs = s_ws + 2 * GN;                                // [2][GN]
         const uint32_t leader_tempty = ptx::map_to_cta(bar_tempty, 0);
+        const uint64_t one2 = ptx::f32x2_one(N & 127);                       // N is a multiple of 128
         const uint32_t lane_base = static_cast<uint32_t>(quarter * 32) << 16;
         bool alive = true;
         int it = 0;                                                 // K-blocks seen so far (all tiles)
@@ -344,40 +345,53 @@ gemm_c8_grouped_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
             const bool row_ok = gm < M;
             // buffer tb was last read two tiles ago; every epilogue warp has passed a group barrier since
             if (threadIdx.x < GN) gemmc::load_channel_params(s_ws + tb * GN, s_bs + tb * GN, w_scale, bias, nt0, N, threadIdx.x);
-            float sum[32];
+            uint64_t sum2[16];                                      // running sums of 32 channels, two per register pair
 #pragma unroll
-            for (int j = 0; j < 32; ++j) sum[j] = 0.0f;
-            // the group's scale is fetched one K-block ahead (it comes from L2)
-            float as_next = row_ok ? __ldg(a_scale + (long long)gm * KB) : 0.0f;
-#pragma unroll 1
-            for (int kb = 0; kb < KB; ++kb, ++it) {
-                const int b = it % GACC;
-                const float as = as_next;
-                if (kb + 1 < KB && row_ok) as_next = __ldg(a_scale + (long long)gm * KB + kb + 1);
-                {   // every warp polls for itself (lane 0; the warp follows): no warp waits for a slower one between K-blocks
-                    int ok = 1;
-                    if (lane == 0) ok = (alive && ptx::mbar_wait(bar_tfull + 8 * b, (it / GACC) & 1, s_abort, status, QVGGT_DEV_TIMEOUT_ACCUM, 20)) ? 1 : 0;
-                    alive = __shfl_sync(0xFFFFFFFFu, ok, 0) != 0;
-                }
+            for (int j = 0; j < 16; ++j) sum2[j] = 0;
+            // The row's scales come from L2, four groups per load, one load ahead (fetched one by one they set the pace: the latency
+            // of one load per K-block).
+            const float4 *as_row = reinterpret_cast<const float4 *>(a_scale + (long long)(row_ok ? gm : 0) * KB);
+            float4 as_next = __ldg(as_row);
+            auto wait_full = [&](int i) {      // every warp polls for itself: no warp waits for a slower one between K-blocks
+                const bool ok = alive && ptx::mbar_wait(bar_tfull + 8 * (i % GACC), (i / GACC) & 1, s_abort, status, QVGGT_DEV_TIMEOUT_ACCUM, 20);
+                alive = __all_sync(0xFFFFFFFFu, ok);
                 ptx::tc_fence_after_sync();
-                if (!alive) continue;
-                uint32_t raw[32];
-                ptx::tmem_ld_32x32(tmem_base + lane_base + b * GN + cpart * 32, raw);
-                ptx::tmem_ld_wait();
-                ptx::tc_fence_before_sync();
-                __syncwarp();
-                if (lane == 0) ptx::mbar_arrive_cluster(leader_tempty + 8 * b);
-                // two elements per multiply (one issue slot for two IEEE multiplications); the additions stay scalar: a packed
-                // multiply feeding a packed add was seen contracted into one fused operation, one rounding instead of two
+            };
+            auto add_group = [&](const uint32_t (&raw)[16], int half, float as) {
                 const uint64_t as2 = ptx::f32x2_pack(as, as);
 #pragma unroll
-                for (int j = 0; j < 32; j += 2) {
-                    float p0, p1;
-                    ptx::f32x2_unpack(ptx::f32x2_mul(ptx::f32x2_pack(static_cast<float>(static_cast<int>(raw[j])), static_cast<float>(static_cast<int>(raw[j + 1]))), as2), p0, p1);
-                    sum[j] = __fadd_rn(sum[j], p0);
-                    sum[j + 1] = __fadd_rn(sum[j + 1], p1);
+                for (int j = 0; j < 16; j += 2)
+                    sum2[8 * half + j / 2] = ptx::f32x2_add_uncontracted(
+                        ptx::f32x2_mul(ptx::f32x2_pack(static_cast<float>(static_cast<int>(raw[j])), static_cast<float>(static_cast<int>(raw[j + 1]))), as2),
+                        sum2[8 * half + j / 2], one2);
+            };
+            // The accumulator comes in halves of 16 columns, each in flight while the other is rescaled.
+            uint32_t lo[16], hi[16];
+            wait_full(it);
+            if (alive) ptx::tmem_ld_32x16(tmem_base + lane_base + (it % GACC) * GN + cpart * 32, lo);
+#pragma unroll 1
+            for (int kb = 0; kb < KB; kb += 4) {
+                const float as4[4] = {as_next.x, as_next.y, as_next.z, as_next.w};
+                if (kb + 4 < KB) as_next = __ldg(as_row + kb / 4 + 1);
+#pragma unroll
+                for (int g = 0; g < 4; ++g, ++it) {
+                    if (!alive) continue;
+                    const int b = it % GACC;
+                    ptx::tmem_ld_wait_for(lo);
+                    ptx::tmem_ld_32x16(tmem_base + lane_base + b * GN + cpart * 32 + 16, hi);
+                    add_group(lo, 0, as4[g]);
+                    if (DUMP && acc_debug && row_ok) gemmc::dump_acc_x16(acc_debug + ((long long)(kb + g) * M + gm) * N + n0, lo);
+                    ptx::tmem_ld_wait_for(hi);
+                    ptx::tc_fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) ptx::mbar_arrive_cluster(leader_tempty + 8 * b);
+                    if (g < 3 || kb + 4 < KB) {
+                        wait_full(it + 1);
+                        if (alive) ptx::tmem_ld_32x16(tmem_base + lane_base + ((it + 1) % GACC) * GN + cpart * 32, lo);
+                    }
+                    add_group(hi, 1, as4[g]);
+                    if (DUMP && acc_debug && row_ok) gemmc::dump_acc_x16(acc_debug + ((long long)(kb + g) * M + gm) * N + n0 + 16, hi);
                 }
-                if (DUMP && acc_debug && row_ok) gemmc::dump_acc_x32<0>(acc_debug + ((long long)kb * M + gm) * N + n0, raw);
             }
             // once per tile the epilogue warps meet: publishes s_ws / s_bs of this tile and orders their reuse two tiles on
             asm volatile("bar.sync %0, %1;" ::"r"(1), "r"(GEPI * 32) : "memory");
@@ -387,8 +401,9 @@ gemm_c8_grouped_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
                 uint32_t out[16];
 #pragma unroll
                 for (int j = 0; j < 32; j += 2) {
-                    const float z0 = __fadd_rn(__fmul_rn(sum[j], wsb[j]), bsb[j]);
-                    const float z1 = __fadd_rn(__fmul_rn(sum[j + 1], wsb[j + 1]), bsb[j + 1]);
+                    float z0, z1;
+                    ptx::f32x2_unpack(ptx::f32x2_add_uncontracted(ptx::f32x2_mul(sum2[j / 2], *reinterpret_cast<const uint64_t *>(wsb + j)),
+                                                                  *reinterpret_cast<const uint64_t *>(bsb + j), one2), z0, z1);
                     out[j >> 1] = ptx::pack_bf16x2(z0, z1);
                 }
                 gemmc::stage_row_32(stg, out, lane);
