@@ -9,11 +9,14 @@
 //
 // The same kernel serves the activations (multiplier amul) and the weight rows (multiplier wmul).
 #include "qvggt_internal.cuh"
+#include "rsq_common.cuh"
 #include "sm100_ptx.cuh"
 #include "tensor_map.cuh"
 #include "unpack_w4.cuh"
 
 namespace {
+
+using namespace rsqc;
 
 constexpr int kThreads = 512;      // CTA of the calibration statistics kernel
 
@@ -111,14 +114,6 @@ __device__ __forceinline__ void rotate_row_to_smem(const uint16_t *x, float *s, 
     }
 }
 
-// (a0, a1) <- (a0 + b0, a1 + b1), (b0, b1) <- (a0 - b0, a1 - b1): two butterflies per instruction pair
-__device__ __forceinline__ void bfly2(float &a0, float &a1, float &b0, float &b1)
-{
-    const uint64_t A = ptx::f32x2_pack(a0, a1), B = ptx::f32x2_pack(b0, b1);
-    ptx::f32x2_unpack(ptx::f32x2_add(A, B), a0, a1);
-    ptx::f32x2_unpack(ptx::f32x2_sub(A, B), b0, b1);
-}
-
 // ------------------------------------------------------------------------------------------------
 // K = T * T (T = 32: one warp per row; T = 64: two warps per row), T values per thread, a single
 // transpose.  The bf16 row is staged in shared memory with 16-byte asynchronous copies (coalesced
@@ -129,14 +124,6 @@ __device__ __forceinline__ void bfly2(float &a0, float &a1, float &b0, float &b1
 //   strides T .. T*T/2    in registers (thread t' holds elements T t + t', bits of t)
 // The codes of thread t' then belong to elements T t + t': eight neighbouring lanes exchange
 // nibbles with three shuffle steps so that every lane ends up with whole 32-bit output words.
-__device__ __forceinline__ void cp_async16(void *smem_dst, const void *gmem_src)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(ptx::smem_addr(smem_dst)), "l"(gmem_src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
 template <int LOGT>
 struct SqGeom {
     static constexpr int T = 1 << LOGT;              // threads per row = values per thread
@@ -179,51 +166,6 @@ __device__ __forceinline__ void stages_in_registers(float (&v)[N])
         for (int k = 0; k < N; k += 2)
             if (!(k & h)) bfly2(v[k], v[k + 1], v[k + h], v[k + 1 + h]);
 }
-
-// Pairwise sum of N registers: adjacent pairs, recursively (the tree of the LayerNorm statistics).
-template <int N>
-__device__ __forceinline__ float tree_sum(const float (&a)[N])
-{
-    if constexpr (N == 1) {
-        return a[0];
-    } else {
-        float b[N / 2];
-#pragma unroll
-        for (int i = 0; i < N / 2; ++i) b[i] = __fadd_rn(a[2 * i], a[2 * i + 1]);
-        return tree_sum<N / 2>(b);
-    }
-}
-
-// GELU x Phi(x) (the activation between the two linears of the MLP: the producer of fc2's input), evaluated so that the
-// negative tail keeps its RELATIVE accuracy.  With t = |x|, z = t / sqrt(2):
-//   Q(t) = 1 - Phi(t) = exp(-z^2) E(z) / 2,   E(z) = exp(z^2) erfc(z)  (smooth, from 1 down to ~1 / (z sqrt(pi))),
-//   E(z) ~ s P(s),  s = 1 / (1 + 0.55 z),  P a degree-4 polynomial (own weighted least-squares fit on z in [0, 9.6]: relative
-//   error below 6e-5), then gelu(x) = x - x Q for x >= 0 and x Q for x < 0.
-// About 16 instructions, two of them special-function (reciprocal, exp2); relative error ~1e-4 wherever the result is a
-// normal number above 2^-120, i.e. at most one bf16 ulp after rounding; below that (x < -12.9) the exponential
-// flushes to zero.  The fused multiply-adds are written explicitly (the file is compiled without contraction).
-__device__ __forceinline__ float gelu_f32(float x)
-{
-    const float z = __fmul_rn(fabsf(x), 0.70710678f);
-    float s;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(s) : "f"(__fmaf_rn(0.55f, z, 1.0f)));
-    float p = -0.17450283f;
-    p = __fmaf_rn(p, s, 0.33387650f);
-    p = __fmaf_rn(p, s, 0.21415194f);
-    p = __fmaf_rn(p, s, 0.31633197f);
-    p = __fmaf_rn(p, s, 0.31008677f);
-    float e;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(__fmul_rn(__fmul_rn(z, z), -1.44269504f)));
-    const float q = __fmul_rn(__fmul_rn(0.5f, e), __fmul_rn(s, p));
-    return x >= 0.0f ? __fmaf_rn(-x, q, x) : __fmul_rn(x, q);
-}
-
-// Parameters of the LayerNorm that may run in front of the rotation (gamma == nullptr: none).
-struct LnArgs {
-    const float *gamma, *beta;   // fp32 [K]
-    float eps;
-    uint16_t *out;               // LN == 2 / 4 only: bf16 [M, K], the normalized / activated rows (nothing else is computed)
-};
 
 // C8: one code per byte (int8, natural element order, row pitch K) instead of two per byte.
 // QMAX: largest code magnitude, 2^(N-1) - 1 of Eq. "quantization": 7 (N = 4) or, with C8 only, 127 (N = 8).
@@ -327,9 +269,10 @@ rsq_sq_kernel(const uint16_t *__restrict__ X, long long ldx, int M, const float 
                 const uint32_t w[4] = {w4.x, w4.y, w4.z, w4.w};
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    if (LN) {                               // plain conversion: the normalization comes first
-                        v[8 * c + 2 * j] = __uint_as_float(w[j] << 16);
-                        v[8 * c + 2 * j + 1] = __uint_as_float(w[j] & 0xFFFF0000u);
+                    if (LN) {                               // plain conversion: the prologue comes first
+                        const uint32_t x = (LN >= 3) ? gelu_bf16x2(w[j]) : w[j];
+                        v[8 * c + 2 * j] = __uint_as_float(x << 16);
+                        v[8 * c + 2 * j + 1] = __uint_as_float(x & 0xFFFF0000u);
                         continue;
                     }
                     // a 32-bit word holds elements 2i (low half) and 2i + 1 of the row: the first stage joins exactly
@@ -343,18 +286,15 @@ rsq_sq_kernel(const uint16_t *__restrict__ X, long long ldx, int M, const float 
             }
         }
         if constexpr (LN == 3 || LN == 4) {
-            uint32_t packed[T / 2];
-#pragma unroll
-            for (int k = 0; k < T; k += 2) {
-                const uint32_t p01 = ptx::pack_bf16x2(gelu_f32(v[k]), gelu_f32(v[k + 1]));   // what an activation kernel would store
-                v[k] = __uint_as_float(p01 << 16);
-                v[k + 1] = __uint_as_float(p01 & 0xFFFF0000u);
-                packed[k / 2] = p01;
-            }
             if constexpr (LN == 4) {
                 uint4 *dst = reinterpret_cast<uint4 *>(ln.out + row * K + T * t);
 #pragma unroll
-                for (int k = 0; k < T / 8; ++k) dst[k] = make_uint4(packed[4 * k], packed[4 * k + 1], packed[4 * k + 2], packed[4 * k + 3]);
+                for (int k = 0; k < T / 8; ++k) {
+                    uint32_t w[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) w[j] = __byte_perm(__float_as_uint(v[8 * k + 2 * j]), __float_as_uint(v[8 * k + 2 * j + 1]), 0x7632);
+                    dst[k] = make_uint4(w[0], w[1], w[2], w[3]);
+                }
                 // every thread of the row has read its share of this stage before any of them starts the copy that will
                 // overwrite it (the next iteration's prefetch goes into this buffer; the other paths meet further down)
                 group_sync<T>(slot);
