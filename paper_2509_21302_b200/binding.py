@@ -1,5 +1,5 @@
 """Thin Python binding of libqvggt: argument marshalling only.  The calls made per layer and forward pass go through a small
-extension module (csrc/fastcall.cpp, 3 us a call instead of 8.5); everything else, and every call that is not plainly
+extension module (csrc/fastcall.cpp, 2.7 us a call instead of 8.5); everything else, and every call that is not plainly
 well-formed, through ctypes.
 
 Every step of the path runs in the CUDA kernels behind the C ABI declared in include/qvggt.h;
@@ -128,25 +128,18 @@ class Weights:
 
     def view(self) -> dict:
         """Copies of the handle's device arrays as torch tensors: wq [N,K/2] u8, w_scale [N], amul [K], bias [N] or None."""
-        ptrs = [ctypes.c_void_p() for _ in range(4)]
-        n, k = ctypes.c_int(), ctypes.c_int()
-        _check(lib().qvggt_weights_view(self.handle, *[ctypes.byref(p) for p in ptrs], ctypes.byref(n), ctypes.byref(k)),
-               "qvggt_weights_view")
-        N, K = n.value, k.value
-
-        def copy(p, kind, d0, d1=-1):
-            return _fast.copy_array(p.value, kind, d0, d1) if p.value else None
-
-        return dict(wq=copy(ptrs[0], 0, N, K // 2), w_scale=copy(ptrs[1], 2, N), amul=copy(ptrs[2], 2, K), bias=copy(ptrs[3], 3, N))
+        r = _fast.weights_view(self.handle)
+        if r is None:
+            raise QvggtError(-1, "qvggt_weights_view")
+        return dict(zip(("wq", "w_scale", "amul", "bias"), r))
 
     def view_c8(self) -> torch.Tensor | None:
         """Copy of the int8 [N, K] codes (None if prepared without c8=True)."""
-        p, bits = ctypes.c_void_p(), ctypes.c_int()
-        _check(lib().qvggt_weights_view_c8(self.handle, ctypes.byref(p), ctypes.byref(bits)), "qvggt_weights_view_c8")
-        self.bits = bits.value
-        if not p.value:
-            return None
-        return _fast.copy_array(p.value, 1, self.N, self.K)
+        r = _fast.weights_view_c8(self.handle, self.N, self.K)
+        if r is None:
+            raise QvggtError(-1, "qvggt_weights_view_c8")
+        codes, self.bits = r
+        return codes
 
     def device_status(self) -> int:
         code = ctypes.c_int(0)
@@ -174,6 +167,11 @@ def prepare_weights(W: torch.Tensor, bias: torch.Tensor | None, smooth_c: torch.
     bits: 4 (W4A4) or 8 (W8A8: one code per byte only; use the *_c8 entry points).
     w_tensorwise: one weight step size for the whole tensor instead of one per output channel (needs c8="only" or bits=8)."""
     assert bits in (4, 8) and c8 in (False, True, "only")
+    flags = (PREP_W8A8 if bits == 8 else (PREP_C8_ONLY if c8 == "only" else (PREP_C8 if c8 else 0))) | (PREP_W_TENSORWISE if w_tensorwise else 0)
+    if _fast is not None:
+        h = _fast.prepare_weights(W, bias, smooth_c, sign_v, flags)
+        if h is not None:
+            return Weights(h, *W.shape)
     assert W.dim() == 2 and W.element_size() == 2 and W.is_contiguous()
     N, K = W.shape
     assert smooth_c.dtype == torch.float32 and smooth_c.numel() == K and smooth_c.is_contiguous()
@@ -182,10 +180,8 @@ def prepare_weights(W: torch.Tensor, bias: torch.Tensor | None, smooth_c: torch.
     if sign_v is not None:
         assert sign_v.dtype == torch.int8 and sign_v.numel() == K and sign_v.is_contiguous()
     h = ctypes.c_void_p()
-    _check(lib().qvggt_prepare_weights(_ptr(W), _ptr(bias), _ptr(smooth_c), _ptr(sign_v), N, K,
-                                       (PREP_W8A8 if bits == 8 else (PREP_C8_ONLY if c8 == "only" else (PREP_C8 if c8 else 0))) | (PREP_W_TENSORWISE if w_tensorwise else 0),
-                                       _stream(),
-                                       ctypes.byref(h)), "qvggt_prepare_weights")
+    _check(lib().qvggt_prepare_weights(_ptr(W), _ptr(bias), _ptr(smooth_c), _ptr(sign_v), N, K, flags, _stream(), ctypes.byref(h)),
+           "qvggt_prepare_weights")
     return Weights(h.value, N, K)
 
 
@@ -477,6 +473,10 @@ def debug_starved_linear_c8(w: Weights, Xq8: torch.Tensor, a_scale: torch.Tensor
 def calibrate_smooth(X_calib: torch.Tensor, W: torch.Tensor, alpha: float = 0.5, lo: float = 1e-2,
                      hi: float = 1e2) -> torch.Tensor:
     """Smoothing factors c [K] fp32 from calibration activations [Mc,K] bf16 and weights [N,K] bf16."""
+    if _fast is not None:
+        c = _fast.calibrate_smooth(X_calib, W, alpha, lo, hi)
+        if c is not None:
+            return c
     assert X_calib.is_contiguous() and W.is_contiguous() and X_calib.element_size() == 2 and W.element_size() == 2
     Mc, K = X_calib.shape
     N = W.shape[0]

@@ -1,8 +1,8 @@
-// The call path from Python into libqvggt, for the calls a program makes per layer and forward pass.
+// The call path from Python into libqvggt, for the calls a program makes per layer: forward passes and preparation.
 //
 // Through ctypes a call costs 8.5 us on the host, 2.4 of it the launch itself: tensor attributes read one by one from Python, the
 // stream object, ctypes' argument conversion.  At a frame or less that is more than the work on the GPU.  Here the arguments go
-// from the tensors to the C entry points directly (3 us a call in all).
+// from the tensors to the C entry points directly (2.7 us a call in all).
 //
 // A function returns what its namesake in binding.py returns, or None when an argument is not plainly what the call expects or
 // the library returned a status: binding.py then takes its own path, which checks, converts and reports.  Nothing
@@ -314,18 +314,84 @@ PyObject *linear_scratch(PyObject *, PyObject *const *args, Py_ssize_t n)
     QVGGT_GUARD_END
 }
 
-// (pointer, kind, d0, d1): copy of a device array as a new tensor on the current device; d1 < 0: one dimension.
-// kind: 0 uint8, 1 int8, 2 float32, 3 bfloat16
-PyObject *copy_array(PyObject *, PyObject *const *args, Py_ssize_t n)
+// (X_calib, W, alpha, lo, hi) -> c
+PyObject *calibrate_smooth(PyObject *, PyObject *const *args, Py_ssize_t n)
 {
     QVGGT_GUARD_BEGIN
     Args in{args, n};
-    void *p = const_cast<qvggt_weights_t *>(in.handle());
-    const int64_t kind = in.integer(), d0 = in.integer(), d1 = in.integer();
-    if (!in.done() || kind < 0 || kind > 3) Py_RETURN_NONE;
-    static const ScalarType types[4] = {at::kByte, at::kChar, at::kFloat, at::kBFloat16};
-    const auto options = at::TensorOptions().dtype(types[kind]).device(at::kCUDA, c10::cuda::getCurrentCUDAStream().device_index());
-    return THPVariable_Wrap((d1 < 0 ? at::from_blob(p, {d0}, options) : at::from_blob(p, {d0, d1}, options)).clone());
+    const Tensor &X = in.tensor(), &W = in.tensor();
+    const float alpha = (float)in.real(), lo = (float)in.real(), hi = (float)in.real();
+    if (!in.done() || X.dim() != 2 || W.dim() != 2 || X.element_size() != 2 || W.element_size() != 2 || !X.is_contiguous() || !W.is_contiguous() ||
+        X.size(1) != W.size(1) || X.size(0) > INT32_MAX || W.size(0) > INT32_MAX || W.size(1) > INT32_MAX)
+        Py_RETURN_NONE;
+    const int64_t K = W.size(1);
+    const Tensor scratch = at::empty({2 * K}, W.options().dtype(at::kFloat)), c = at::empty({K}, W.options().dtype(at::kFloat));
+    const void *x = X.data_ptr(), *w = W.data_ptr();
+    float *s = static_cast<float *>(scratch.data_ptr()), *out = static_cast<float *>(c.data_ptr());
+    void *st = stream();
+    if (without_gil([&] { return qvggt_calibrate_smooth(x, (int)X.size(0), w, (int)W.size(0), (int)K, alpha, lo, hi, s, out, st); }) != QVGGT_OK) Py_RETURN_NONE;
+    return THPVariable_Wrap(c);
+    QVGGT_GUARD_END
+}
+
+// (W, bias, smooth_c, sign_v, flags) -> handle as an integer
+PyObject *prepare_weights(PyObject *, PyObject *const *args, Py_ssize_t n)
+{
+    QVGGT_GUARD_BEGIN
+    Args in{args, n};
+    const Tensor &W = in.tensor(), &bias = in.tensor(true), &c = in.tensor(), &v = in.tensor(true);
+    const int flags = (int)in.integer();
+    if (!in.done() || W.dim() != 2 || W.element_size() != 2 || !W.is_contiguous() || W.size(0) > INT32_MAX || W.size(1) > INT32_MAX) Py_RETURN_NONE;
+    const int64_t N = W.size(0), K = W.size(1);
+    if (c.scalar_type() != at::kFloat || c.numel() != K || !c.is_contiguous()) Py_RETURN_NONE;
+    if (bias.defined() && (bias.element_size() != 2 || bias.numel() != N || !bias.is_contiguous())) Py_RETURN_NONE;
+    if (v.defined() && (v.scalar_type() != at::kChar || v.numel() != K || !v.is_contiguous())) Py_RETURN_NONE;
+    const void *w = W.data_ptr(), *b = bias.defined() ? bias.data_ptr() : nullptr;
+    const float *cp = static_cast<const float *>(c.data_ptr());
+    const S8 *vp = v.defined() ? static_cast<const S8 *>(v.data_ptr()) : nullptr;
+    void *st = stream();
+    qvggt_weights_t *h = nullptr;
+    if (without_gil([&] { return qvggt_prepare_weights(w, b, cp, vp, (int)N, (int)K, flags, st, &h); }) != QVGGT_OK) Py_RETURN_NONE;
+    return PyLong_FromVoidPtr(h);
+    QVGGT_GUARD_END
+}
+
+// Copy of a device array as a new tensor on the current device (d1 < 0: one dimension), None for a null pointer.
+PyObject *copy_array(const void *p, ScalarType type, int64_t d0, int64_t d1)
+{
+    if (!p) Py_RETURN_NONE;
+    const auto options = at::TensorOptions().dtype(type).device(at::kCUDA, c10::cuda::getCurrentCUDAStream().device_index());
+    void *q = const_cast<void *>(p);
+    return THPVariable_Wrap((d1 < 0 ? at::from_blob(q, {d0}, options) : at::from_blob(q, {d0, d1}, options)).clone());
+}
+
+// (handle) -> copies (wq, w_scale, amul, bias), None where the handle has no such array
+PyObject *weights_view(PyObject *, PyObject *const *args, Py_ssize_t n)
+{
+    QVGGT_GUARD_BEGIN
+    Args in{args, n};
+    auto *h = in.handle();
+    const U8 *wq = nullptr;
+    const float *ws = nullptr, *am = nullptr;
+    const void *bias = nullptr;
+    int N = 0, K = 0;
+    if (!in.done() || qvggt_weights_view(h, &wq, &ws, &am, &bias, &N, &K) != QVGGT_OK) Py_RETURN_NONE;
+    return release_items(PyTuple_Pack(4, copy_array(wq, at::kByte, N, K / 2), copy_array(ws, at::kFloat, N, -1), copy_array(am, at::kFloat, K, -1),
+                                      copy_array(bias, at::kBFloat16, N, -1)));
+    QVGGT_GUARD_END
+}
+
+// (handle, N, K) -> (copy of the codes one per byte or None, code width)
+PyObject *weights_view_c8(PyObject *, PyObject *const *args, Py_ssize_t n)
+{
+    QVGGT_GUARD_BEGIN
+    Args in{args, n};
+    auto *h = in.handle();
+    const int64_t N = in.integer(), K = in.integer();
+    const S8 *wq8 = nullptr;
+    int bits = 0;
+    if (!in.done() || qvggt_weights_view_c8(h, &wq8, &bits) != QVGGT_OK) Py_RETURN_NONE;
+    return release_items(PyTuple_Pack(2, copy_array(wq8, at::kChar, N, K), PyLong_FromLong(bits)));
     QVGGT_GUARD_END
 }
 
@@ -344,7 +410,10 @@ PyMethodDef methods[] = {
     FAST("w4a4_linear_c8_grouped", (linear_c8<qvggt_w4a4_linear_c8_grouped, true>)),
     FAST("w4a4_linear_c8_packed_weights", (linear_scratch<false>)),
     FAST("w4a4_linear_c8_expanded", (linear_scratch<true>)),
-    FAST("copy_array", copy_array),
+    FAST("calibrate_smooth", calibrate_smooth),
+    FAST("prepare_weights", prepare_weights),
+    FAST("weights_view", weights_view),
+    FAST("weights_view_c8", weights_view_c8),
     {nullptr, nullptr, 0, nullptr}};
 
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_qvggt_fastcall", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};

@@ -84,3 +84,42 @@ def test_same_errors_as_through_ctypes():
     h.free()
     with pytest.raises(RuntimeError):
         q.rotate_smooth_quantize_c8(h, x)
+
+
+def test_preparation_calls_give_the_same_and_refuse_the_same(monkeypatch):
+    K, N = 1024, 256
+    g = torch.Generator(device="cuda").manual_seed(5)
+    W = (torch.randn(N, K, generator=g, device="cuda") * 0.02).bfloat16()
+    b, X = torch.randn(N, generator=g, device="cuda").bfloat16(), torch.randn(37, K, generator=g, device="cuda").bfloat16()
+    v = (torch.randint(0, 2, (K,), generator=g, device="cuda") * 2 - 1).to(torch.int8)
+
+    def run():
+        c = q.calibrate_smooth(X, W, 0.5, 0.02, 50.0)
+        out = [c]
+        for bias, sign, c8, bits in ((b, None, True, 4), (None, v, "only", 4), (b, v, False, 4), (b, None, False, 8)):
+            h = q.prepare_weights(W, bias, c, sign, c8=c8, bits=bits)
+            view = h.view()
+            out += [view["wq"], view["w_scale"], view["amul"], view["bias"], h.view_c8()]
+            assert h.bits == bits
+            h.free()
+        return out
+
+    fast = run()
+    lib = binding._fast
+
+    class OnlyViews:                      # the other calls through ctypes
+        weights_view, weights_view_c8 = staticmethod(lib.weights_view), staticmethod(lib.weights_view_c8)
+        calibrate_smooth = prepare_weights = staticmethod(lambda *a: None)
+
+    monkeypatch.setattr(binding, "_fast", OnlyViews)
+    slow = run()
+    monkeypatch.undo()
+    for a, s in zip(fast, slow):
+        assert (a is None) == (s is None) and (a is None or (a.dtype == s.dtype and torch.equal(a, s)))
+    for bad in (lambda: q.calibrate_smooth(X, W.float()), lambda: q.calibrate_smooth(X[:, ::2], W), lambda: q.prepare_weights(W.float(), None, fast[0]),
+                lambda: q.prepare_weights(W, b[:5], fast[0]), lambda: q.prepare_weights(W, None, fast[0][:5]), lambda: q.prepare_weights(W, None, fast[0], v.float())):
+        with pytest.raises(AssertionError):
+            bad()
+    with pytest.raises(q.QvggtError) as e:
+        q.prepare_weights(W[:100], None, fast[0])
+    assert e.value.status == -2
