@@ -183,7 +183,8 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
                         // last read of this accumulator: hand it back to the MMA thread before the math
                         ptx::tc_fence_before_sync();
                         __syncwarp();
-                        if (lane == 0) ptx::mbar_arrive_cluster(leader_tempty + 8 * b);
+                        // (nobody waits for the last tiles' arrivals: none may be on its way when the leader CTA exits)
+                        if (lane == 0 && t + ACC_BUFS < my_tiles) ptx::mbar_arrive_cluster(leader_tempty + 8 * b);
                     }
                     if (cols_ok) {
                         gemmc::finish_16x64(raw, as2[u], wsb + 64 * h, bsb + 64 * h, stg, stg_addr, Y + (long long)m * ldy + n, ldy, M - m, lane, one2);
@@ -206,7 +207,7 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
         if (rank == 0 && ptx::elect_one()) {
             constexpr uint32_t idesc = ptx::idesc_i8(BM * CG, BN);
             bool alive = true;
-            int us = 0;
+            int us = 0, left = my_tiles * KB;                              // K-blocks to come, this one included
             uint32_t uph = 0;
             for (int t = 0; t < my_tiles && alive; ++t) {
                 const int b = t & 1;
@@ -222,7 +223,7 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
                     ptx::tc_fence_after_sync();
                     const uint32_t a_addr = sbase + C::OFF_UP + us * C::UP_STAGE;
                     gemmc::mma_kblock_i8<true>(d_tmem, a_addr, a_addr + BM * BK, idesc, kb == 0);
-                    ptx::mma_commit_pair(bar_uempty + 8 * us, 3);
+                    if (left-- > C::US) ptx::mma_commit_pair(bar_uempty + 8 * us, 3);
                     if (kb == KB - 1) ptx::mma_commit_pair(bar_tfull + 8 * b, 3);
                     if (++us == C::US) { us = 0; uph ^= 1; }
                 }
@@ -258,7 +259,7 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
 
     ptx::tc_fence_before_sync();
     __syncthreads();
-    ptx::cluster_sync();                     // no remote arrival or multicast commit may target a CTA that has exited
+    ptx::cluster_sync_relaxed();             // no remote arrival or multicast commit may target a CTA that has exited: each one is waited for
     if (warp == MMA_WARP) {
         ptx::tc_fence_after_sync();
         ptx::tmem_dealloc_pair(tmem_base, C::TMEM_COLS);

@@ -163,7 +163,8 @@ gemm_c8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
                     if (c == NCH - 1) {                        // tensor memory goes back to the MMA thread
                         ptx::tc_fence_before_sync();
                         __syncwarp();
-                        if (lane == 0) ptx::mbar_arrive_cluster(leader_tempty + 8 * b);
+                        // (nobody waits for the last tiles' arrivals: none may be on its way when the leader CTA exits)
+                        if (lane == 0 && t + ACC_BUFS < my_tiles) ptx::mbar_arrive_cluster(leader_tempty + 8 * b);
                     }
                     if (cols_ok) {
 #pragma unroll
@@ -185,6 +186,7 @@ gemm_c8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
             constexpr uint32_t idesc = ptx::idesc_i8(2 * BM, BN);
             bool alive = true;
             Ring r;
+            int left = my_tiles * KB;                                      // K-blocks to come, this one included
             for (int t = 0; t < my_tiles && alive; ++t) {
                 const int b = t & 1;
                 if (t >= ACC_BUFS) {
@@ -199,7 +201,7 @@ gemm_c8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
                     ptx::tc_fence_after_sync();
                     const uint32_t a_addr = sbase + r.s * STAGE;
                     gemmc::mma_kblock_i8<true>(d_tmem, a_addr, a_addr + BM * BK, idesc, kb == 0);
-                    ptx::mma_commit_pair(bar_empty + 8 * r.s, 3);      // frees the stage in both CTAs
+                    if (left-- > STAGES) ptx::mma_commit_pair(bar_empty + 8 * r.s, 3);   // frees the stage in both CTAs, if a load waits for it
                     if (kb == KB - 1) ptx::mma_commit_pair(bar_tfull + 8 * b, 3);
                     r.advance(STAGES);
                 }
@@ -237,7 +239,7 @@ gemm_c8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
 
     ptx::tc_fence_before_sync();
     __syncthreads();
-    ptx::cluster_sync();        // no remote arrival or multicast commit may target a CTA that has exited
+    ptx::cluster_sync_relaxed();        // no remote arrival or multicast commit may target a CTA that has exited: each one is waited for
     if (warp == MMA_WARP) {
         ptx::tc_fence_after_sync();
         ptx::tmem_dealloc_pair(tmem_base, TMEM_COLS);
@@ -384,7 +386,7 @@ gemm_c8_grouped_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
                     ptx::tmem_ld_wait_for(hi);
                     ptx::tc_fence_before_sync();
                     __syncwarp();
-                    if (lane == 0) ptx::mbar_arrive_cluster(leader_tempty + 8 * b);
+                    if (lane == 0 && it + GACC < my_tiles * KB) ptx::mbar_arrive_cluster(leader_tempty + 8 * b);   // if an MMA will wait for it
                     if (g < 3 || kb + 4 < KB) {
                         wait_full(it + 1);
                         if (alive) ptx::tmem_ld_32x16(tmem_base + lane_base + ((it + 1) % GACC) * GN + cpart * 32, lo);
@@ -430,7 +432,7 @@ gemm_c8_grouped_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
                 ptx::tc_fence_after_sync();
                 const uint32_t a_addr = sbase + r.s * GSTAGE;
                 gemmc::mma_kblock_i8<true>(tmem_base + b * GN, a_addr, a_addr + BM * BK, idesc, true);
-                ptx::mma_commit_pair(bar_empty + 8 * r.s, 3);
+                if (it + GSTAGES < total_kb) ptx::mma_commit_pair(bar_empty + 8 * r.s, 3);
                 ptx::mma_commit_pair(bar_tfull + 8 * b, 3);
                 r.advance(GSTAGES);
             }
@@ -465,7 +467,7 @@ gemm_c8_grouped_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
 
     ptx::tc_fence_before_sync();
     __syncthreads();
-    ptx::cluster_sync();
+    ptx::cluster_sync_relaxed();        // every remote arrival was waited for
     if (warp == G_MMA_WARP) {
         ptx::tc_fence_after_sync();
         ptx::tmem_dealloc_pair(tmem_base, TMEM_COLS);

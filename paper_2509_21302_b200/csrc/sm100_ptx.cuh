@@ -310,6 +310,13 @@ __device__ __forceinline__ void cluster_sync()   // every thread of every CTA in
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+// The same meeting without any ordering of memory: for the way out, where it only keeps a CTA's shared memory alive until its peer
+// is done.  (The release form waits for the outstanding global stores of the whole epilogue first, about 0.5 us.)
+__device__ __forceinline__ void cluster_sync_relaxed()
+{
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;\n\tbarrier.cluster.wait.aligned;" ::: "memory");
+}
+
 // shared::cluster address of `local_addr` (a shared::cta address) inside CTA `rank` of the cluster
 __device__ __forceinline__ uint32_t map_to_cta(uint32_t local_addr, uint32_t rank)
 {
