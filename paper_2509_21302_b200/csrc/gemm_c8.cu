@@ -264,12 +264,12 @@ constexpr int G_MMA_WARP = GEPI, G_TMA_WARP = GEPI + 1;
 constexpr int GTHREADS = (GEPI + 2) * 32;
 constexpr int GB_ROWS = GN / 2;                        // weight rows staged by one CTA
 constexpr int GSTAGE = (BM + GB_ROWS) * BK;            // 24 KB
-constexpr int GACC = 4;                                // accumulators of 128 columns (a ring of four instead of two: 5-8 % faster)
+constexpr int GACC = 4, GPAIRS = GACC / 2;             // accumulators of 128 columns; they are handed over two K-blocks at a time
 constexpr int GSTAGES = 7;
 constexpr int OFF_STG = GSTAGES * GSTAGE;
-constexpr int OFF_CH = OFF_STG + GEPI * STG_BYTES;          // [2][GN] channel scales, [2][GN] bias, fp32
-constexpr int OFF_BAR = OFF_CH + 2 * 2 * GN * 4;                 // full[GSTAGES] empty[GSTAGES] tfull[2] tempty[2]
-constexpr int NBARS = 2 * GSTAGES + 2 * GACC;
+constexpr int OFF_CH = OFF_STG + GEPI * STG_BYTES;          // per warp: 32 channel scales, 32 biases, fp32
+constexpr int OFF_BAR = OFF_CH + GEPI * 64 * 4;                 // full[GSTAGES] empty[GSTAGES] tfull[2] tempty[2]
+constexpr int NBARS = 2 * GSTAGES + 2 * GPAIRS;
 constexpr int OFF_TMEM = OFF_BAR + NBARS * 8;
 constexpr int OFF_ABORT = OFF_TMEM + 4;
 constexpr int OFF_FLAGS = OFF_ABORT + 4;
@@ -291,7 +291,7 @@ gemm_c8_grouped_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
     const uint32_t bar_full = sbase + OFF_BAR;
     const uint32_t bar_empty = bar_full + GSTAGES * 8;
     const uint32_t bar_tfull = bar_empty + GSTAGES * 8;
-    const uint32_t bar_tempty = bar_tfull + GACC * 8;
+    const uint32_t bar_tempty = bar_tfull + GPAIRS * 8;
     uint32_t *s_tmem = reinterpret_cast<uint32_t *>(smem + OFF_TMEM);
     volatile int *s_abort = reinterpret_cast<volatile int *>(smem + OFF_ABORT);
 
@@ -306,8 +306,8 @@ gemm_c8_grouped_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
     if (threadIdx.x == 0) {
         gemmc::init_barriers(bar_full, GSTAGES, 1);
         gemmc::init_barriers(bar_empty, GSTAGES, 1);
-        gemmc::init_barriers(bar_tfull, GACC, 1);
-        gemmc::init_barriers(bar_tempty, GACC, GEPI * 2);
+        gemmc::init_barriers(bar_tfull, GPAIRS, 1);
+        gemmc::init_barriers(bar_tempty, GPAIRS, GEPI * 2);
         *s_abort = 0;
         ptx::fence_mbar_init();
     }
@@ -330,23 +330,22 @@ gemm_c8_grouped_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
         const int quarter = warp & 3, cpart = warp >> 2;   // TMEM lane quarter, 32-column part
         unsigned char *stg = smem + OFF_STG + warp * STG_BYTES;
         const uint32_t stg_addr = sbase + OFF_STG + warp * STG_BYTES;
-        float *s_ws = reinterpret_cast<float *>(smem + OFF_CH);    // [2][GN]
-        float *s_bs = s_ws + 2 * GN;                                // [2][GN]
+        float *wsb = reinterpret_cast<float *>(smem + OFF_CH) + warp * 64, *bsb = wsb + 32;   // the warp's channel scales, biases
         const uint32_t leader_tempty = ptx::map_to_cta(bar_tempty, 0);
         const uint64_t one2 = ptx::f32x2_one(N & 127);                       // N is a multiple of 128
         const uint32_t lane_base = static_cast<uint32_t>(quarter * 32) << 16;
         bool alive = true;
-        int it = 0;                                                 // K-blocks seen so far (all tiles)
+        int pair = 0;                                               // pairs of K-blocks seen so far (all tiles)
         for (int t = 0; t < my_tiles; ++t) {
             const int tile = worker + t * workers;
             const int m0 = (tile / n_tiles) * (2 * BM) + (int)rank * BM + quarter * 32;
-            const int nt0 = (tile % n_tiles) * GN;
-            const int n0 = nt0 + cpart * 32;
-            const int tb = t & 1;
+            const int n0 = (tile % n_tiles) * GN + cpart * 32;
             const int gm = m0 + lane;
             const bool row_ok = gm < M;
-            // buffer tb was last read two tiles ago; every epilogue warp has passed a group barrier since
-            if (threadIdx.x < GN) gemmc::load_channel_params(s_ws + tb * GN, s_bs + tb * GN, w_scale, bias, nt0, N, threadIdx.x);
+            // The scales and biases of the warp's 32 channels, one channel per lane, fetched here and needed at the end of the tile: each
+            // warp keeps its own copy, so that no warp ever waits for another.
+            const float my_ws = __ldg(w_scale + n0 + lane);
+            const float my_bs = bias ? __uint_as_float(static_cast<uint32_t>(__ldg(bias + n0 + lane)) << 16) : 0.0f;
             uint64_t sum2[16];                                      // running sums of 32 channels, two per register pair
 #pragma unroll
             for (int j = 0; j < 16; ++j) sum2[j] = 0;
@@ -354,8 +353,8 @@ gemm_c8_grouped_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
             // of one load per K-block).
             const float4 *as_row = reinterpret_cast<const float4 *>(a_scale + (long long)(row_ok ? gm : 0) * KB);
             float4 as_next = __ldg(as_row);
-            auto wait_full = [&](int i) {      // every warp polls for itself: no warp waits for a slower one between K-blocks
-                const bool ok = alive && ptx::mbar_wait(bar_tfull + 8 * (i % GACC), (i / GACC) & 1, s_abort, status, QVGGT_DEV_TIMEOUT_ACCUM, 20);
+            auto wait_full = [&](int p) {      // every warp polls for itself: no warp waits for a slower one between K-blocks
+                const bool ok = alive && ptx::mbar_wait(bar_tfull + 8 * (p % GPAIRS), (p / GPAIRS) & 1, s_abort, status, QVGGT_DEV_TIMEOUT_ACCUM, 20);
                 alive = __all_sync(0xFFFFFFFFu, ok);
                 ptx::tc_fence_after_sync();
             };
@@ -367,39 +366,45 @@ gemm_c8_grouped_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
                         ptx::f32x2_mul(ptx::f32x2_pack(static_cast<float>(static_cast<int>(raw[j])), static_cast<float>(static_cast<int>(raw[j + 1]))), as2),
                         sum2[8 * half + j / 2], one2);
             };
-            // The accumulator comes in halves of 16 columns, each in flight while the other is rescaled.
+            // The accumulators come in halves of 16 columns, each in flight while the other is rescaled.
             uint32_t lo[16], hi[16];
-            wait_full(it);
-            if (alive) ptx::tmem_ld_32x16(tmem_base + lane_base + (it % GACC) * GN + cpart * 32, lo);
+            const uint32_t my_cols = tmem_base + lane_base + cpart * 32;
+            wait_full(pair);
+            if (alive) ptx::tmem_ld_32x16(my_cols + (pair % GPAIRS) * 2 * GN, lo);
 #pragma unroll 1
             for (int kb = 0; kb < KB; kb += 4) {
                 const float as4[4] = {as_next.x, as_next.y, as_next.z, as_next.w};
                 if (kb + 4 < KB) as_next = __ldg(as_row + kb / 4 + 1);
 #pragma unroll
-                for (int g = 0; g < 4; ++g, ++it) {
+                for (int g = 0; g < 4; ++g) {
                     if (!alive) continue;
-                    const int b = it % GACC;
+                    const int b = pair % GPAIRS;
+                    const uint32_t acc = my_cols + (2 * b + (g & 1)) * GN;
                     ptx::tmem_ld_wait_for(lo);
-                    ptx::tmem_ld_32x16(tmem_base + lane_base + b * GN + cpart * 32 + 16, hi);
+                    ptx::tmem_ld_32x16(acc + 16, hi);
                     add_group(lo, 0, as4[g]);
                     if (DUMP && acc_debug && row_ok) gemmc::dump_acc_x16(acc_debug + ((long long)(kb + g) * M + gm) * N + n0, lo);
                     ptx::tmem_ld_wait_for(hi);
-                    ptx::tc_fence_before_sync();
-                    __syncwarp();
-                    if (lane == 0 && it + GACC < my_tiles * KB) ptx::mbar_arrive_cluster(leader_tempty + 8 * b);   // if an MMA will wait for it
-                    if (g < 3 || kb + 4 < KB) {
-                        wait_full(it + 1);
-                        if (alive) ptx::tmem_ld_32x16(tmem_base + lane_base + ((it + 1) % GACC) * GN + cpart * 32, lo);
+                    if (g & 1) {
+                        ptx::tc_fence_before_sync();
+                        __syncwarp();
+                        if (lane == 0 && pair + GPAIRS < my_tiles * KB / 2) ptx::mbar_arrive_cluster(leader_tempty + 8 * b);   // if an MMA will wait for it
+                        ++pair;
+                        if (g < 3 || kb + 4 < KB) {
+                            wait_full(pair);
+                            if (alive) ptx::tmem_ld_32x16(my_cols + (pair % GPAIRS) * 2 * GN, lo);
+                        }
+                    } else {
+                        ptx::tmem_ld_32x16(acc + GN, lo);
                     }
                     add_group(hi, 1, as4[g]);
                     if (DUMP && acc_debug && row_ok) gemmc::dump_acc_x16(acc_debug + ((long long)(kb + g) * M + gm) * N + n0 + 16, hi);
                 }
             }
-            // once per tile the epilogue warps meet: publishes s_ws / s_bs of this tile and orders their reuse two tiles on
-            asm volatile("bar.sync %0, %1;" ::"r"(1), "r"(GEPI * 32) : "memory");
+            wsb[lane] = my_ws;
+            bsb[lane] = my_bs;
+            __syncwarp();
             if (alive) {
-                const float *wsb = s_ws + tb * GN + cpart * 32;
-                const float *bsb = s_bs + tb * GN + cpart * 32;
                 uint32_t out[16];
 #pragma unroll
                 for (int j = 0; j < 32; j += 2) {
@@ -411,6 +416,7 @@ gemm_c8_grouped_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
                 gemmc::stage_row_32(stg, out, lane);
                 gemmc::store_staged_32x32(&map_y, stg_addr, n0, m0, m0 < M, lane);
             }
+            __syncwarp();                                           // wsb and bsb are rewritten at the end of the next tile
         }
         if (lane == 0) ptx::tma_store_wait_read<0>();
     } else if (warp == G_MMA_WARP) {
@@ -420,10 +426,10 @@ gemm_c8_grouped_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
             bool alive = true;
             Ring r;
             const int total_kb = my_tiles * KB;
-            for (int it = 0; it < total_kb && alive; ++it) {
-                const int b = it % GACC;
-                if (it >= GACC) {
-                    alive = ptx::mbar_wait_cluster(bar_tempty + 8 * b, ((it / GACC) - 1) & 1, s_abort, status, QVGGT_DEV_TIMEOUT_TMEM_FREE);
+            for (int it = 0; it < total_kb && alive; ++it) {       // K / 128 is even: pairs never straddle a tile
+                const int b = it % GACC, p = it / 2;
+                if (it >= GACC && !(it & 1)) {
+                    alive = ptx::mbar_wait_cluster(bar_tempty + 8 * (p % GPAIRS), ((p / GPAIRS) - 1) & 1, s_abort, status, QVGGT_DEV_TIMEOUT_TMEM_FREE);
                     if (!alive) break;
                     ptx::tc_fence_after_sync();
                 }
@@ -433,7 +439,7 @@ gemm_c8_grouped_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
                 const uint32_t a_addr = sbase + r.s * GSTAGE;
                 gemmc::mma_kblock_i8<true>(tmem_base + b * GN, a_addr, a_addr + BM * BK, idesc, true);
                 if (it + GSTAGES < total_kb) ptx::mma_commit_pair(bar_empty + 8 * r.s, 3);
-                ptx::mma_commit_pair(bar_tfull + 8 * b, 3);
+                if (it & 1) ptx::mma_commit_pair(bar_tfull + 8 * (p % GPAIRS), 3);
                 r.advance(GSTAGES);
             }
         }
