@@ -48,8 +48,8 @@ struct Lay {
     static constexpr int STAGE = (BM + B_ROWS) * BK;              // 32 / 24 KB
     static constexpr int STAGES = BN == 256 ? 6 : 8;
     static constexpr int OFF_STG = STAGES * STAGE;                // operand stages first: they need 1024-byte alignment
-    static constexpr int OFF_CH = OFF_STG + EPI_WARPS * STG_BYTES;          // per-channel scale and bias of two tiles, fp32
-    static constexpr int OFF_BAR = OFF_CH + 2 * ACC_BUFS * BN * 4;          // full[STAGES] empty[STAGES] tfull[2] tempty[2]
+    static constexpr int OFF_CH = OFF_STG + EPI_WARPS * STG_BYTES;          // per warp: scales and biases of its BN / 2 channels, fp32
+    static constexpr int OFF_BAR = OFF_CH + EPI_WARPS * BN * 4;             // full[STAGES] empty[STAGES] tfull[2] tempty[2]
     static constexpr int NBARS = 2 * STAGES + 2 * ACC_BUFS;
     static constexpr int OFF_TMEM = OFF_BAR + NBARS * 8;
     static constexpr int OFF_ABORT = OFF_TMEM + 4;
@@ -119,8 +119,7 @@ gemm_c8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
         const int quarter = warp & 3, cpart = warp >> 2;   // TMEM lane quarter, column part
         unsigned char *stg = smem + L::OFF_STG + warp * STG_BYTES;
         const uint32_t stg_addr = sbase + L::OFF_STG + warp * STG_BYTES;
-        float *s_ws = reinterpret_cast<float *>(smem + L::OFF_CH);             // [2][BN] per-channel scale of the tile
-        float *s_bs = s_ws + ACC_BUFS * BN;                                  // [2][BN] bias as fp32
+        float *wsb = reinterpret_cast<float *>(smem + L::OFF_CH) + warp * BN, *bsb = wsb + BN / 2;     // the warp's channel scales, biases
         const uint32_t leader_tempty = ptx::map_to_cta(bar_tempty, 0);
         const uint64_t one2 = ptx::f32x2_one(N & 127);                       // N is a multiple of 128
         bool alive = true;
@@ -128,13 +127,18 @@ gemm_c8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
         for (int t = 0; t < my_tiles; ++t) {
             const int tile = worker + t * workers;
             const int m0 = (tile / n_tiles) * (2 * BM) + (int)rank * BM + quarter * 32;
-            const int nt0 = (tile % n_tiles) * BN;             // first channel of the tile
-            const int n0 = nt0 + cpart * CW;                   // first channel of this warp's part
+            const int n0 = (tile % n_tiles) * BN + cpart * CW; // first channel of this warp's part
             const int b = t & 1;
             const bool cols_ok = n0 < N;                       // N is a multiple of 128: a part is all in or all out
-            // per-channel scale and bias of the tile -> shared memory; buffer b was last read two tiles ago,
-            // and every epilogue warp has passed the group barrier of the tile in between since then
-            if (BN == EPI_WARPS * 32 || threadIdx.x < BN) gemmc::load_channel_params(s_ws + b * BN, s_bs + b * BN, w_scale, bias, nt0, N, threadIdx.x);
+            // The scales and biases of the warp's channels: each warp keeps its own copy in shared memory, so that no warp ever
+            // waits for another.
+            float my_ws[CW / 32], my_bs[CW / 32];
+#pragma unroll
+            for (int e = 0; e < CW / 32; ++e) {
+                const int n = n0 + 32 * e + lane;
+                my_ws[e] = cols_ok ? __ldg(w_scale + n) : 0.0f;
+                my_bs[e] = (cols_ok && bias) ? __uint_as_float(static_cast<uint32_t>(__ldg(bias + n)) << 16) : 0.0f;
+            }
             uint64_t as2[2][2];                                // rows lane / 4 + 8 h of the warp's 16 u .. 16 u + 15
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
@@ -142,8 +146,13 @@ gemm_c8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
                 const float as = gm < M ? __ldg(a_scale + gm) : 0.0f;
                 as2[u >> 1][u & 1] = ptx::f32x2_pack(as, as);
             }
-            // the epilogue warps meet (named barrier 1: publishes s_ws / s_bs), then every warp polls the accumulator barrier itself
-            asm volatile("bar.sync %0, %1;" ::"r"(1), "r"(EPI_WARPS * 32) : "memory");
+            __syncwarp();                                      // the previous tile's last reads
+#pragma unroll
+            for (int e = 0; e < CW / 32; ++e) {
+                wsb[32 * e + lane] = my_ws[e];
+                bsb[32 * e + lane] = my_bs[e];
+            }
+            __syncwarp();
             {
                 int ok = 1;
                 if (lane == 0) ok = (alive && ptx::mbar_wait(bar_tfull + 8 * b, (t >> 1) & 1, s_abort, status, QVGGT_DEV_TIMEOUT_ACCUM, 32, wait_limit)) ? 1 : 0;
@@ -151,8 +160,6 @@ gemm_c8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
             }
             ptx::tc_fence_after_sync();
             if (alive) {
-                const float *wsb = s_ws + b * BN + cpart * CW;
-                const float *bsb = s_bs + b * BN + cpart * CW;
 #pragma unroll
                 for (int c = 0; c < NCH; ++c) {
                     uint32_t raw[2][32];
