@@ -31,8 +31,7 @@
  *     stream); no call synchronises the device except where stated.
  *     The quantize and GEMM kernels are launched with programmatic stream serialization allowed:
  *     their blocks may become resident while the previous kernel of the stream drains, but they touch
- *     no global memory before that kernel has completed -- except that a GEMM may read the handle's own
- *     weights, which were complete before -- so stream order is what the caller sees.
+ *     no global memory before that kernel has completed, so stream order is what the caller sees.
  *   - Return value: QVGGT_OK or a negative qvggt_status_t.  Arguments are validated on the host
  *     before anything is launched; nothing throws or exits.
  *   - Device-side waits are bounded.  If one expires the kernel records a code in the handle's

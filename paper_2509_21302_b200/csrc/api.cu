@@ -82,13 +82,13 @@ int qvggt_prepare_weights(const void *W_bf16, const void *bias_bf16, const float
     w->status = reinterpret_cast<int *>(base + at_status);
     float *wmul = reinterpret_cast<float *>(base + at_wmul);
     cudaError_t e = qvggt_launch_multipliers(smooth_c, sign_v, K, w->amul, wmul, st, static_cast<const uint16_t *>(bias_bf16), N, w->bias, w->status);
-    if (e == cudaSuccess && w->Wq) e = qvggt_launch_rsq(W_bf16, K, N, K, wmul, 0, w->Wq, w->w_scale, st, true);
-    if (e == cudaSuccess && w->Wq8) e = qvggt_launch_rsq_c8(W_bf16, K, N, K, wmul, w->bits, w->Wq8, w->w_scale, st, 0, nullptr, nullptr, 0, true);
+    if (e == cudaSuccess && w->Wq) e = qvggt_launch_rsq(W_bf16, K, N, K, wmul, 0, w->Wq, w->w_scale, st);
+    if (e == cudaSuccess && w->Wq8) e = qvggt_launch_rsq_c8(W_bf16, K, N, K, wmul, w->bits, w->Wq8, w->w_scale, st);
     if (e == cudaSuccess && tensorwise) {
         // one step size for the whole tensor (Tab. "granularity"): the largest of the per-row step sizes just computed,
         // i.e. max|W~| / qmax (the division is monotone), then the static quantizer, which also writes that step as every row's scale
         e = qvggt_launch_max_reduce(w->w_scale, N, wmul + K, st);
-        if (e == cudaSuccess) e = qvggt_launch_rsq_static_c8(W_bf16, K, N, K, wmul, w->bits, wmul + K, w->Wq8, w->w_scale, st, true);
+        if (e == cudaSuccess) e = qvggt_launch_rsq_static_c8(W_bf16, K, N, K, wmul, w->bits, wmul + K, w->Wq8, w->w_scale, st);
     }
     if (e != cudaSuccess) {
         cudaStreamSynchronize(st);

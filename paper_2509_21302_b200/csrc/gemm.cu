@@ -304,7 +304,7 @@ cudaError_t qvggt_launch_gemm(const qvggt_weights *w, const unsigned char *Xq, c
 {
     if (M == 0) return cudaSuccess;
     if (!acc_debug && (group == 0 || group == 128) && qvggt_gemm_small_wins(w, M, true, group == 128))
-        return qvggt_launch_gemm_small(w, Xq, w->Wq, true, a_scale, group == 128, M, Y, ldy, true, st);
+        return qvggt_launch_gemm_small(w, Xq, w->Wq, true, a_scale, group == 128, M, Y, ldy, st);
     if (group == 128) return qvggt_launch_gemm_grouped(w, Xq, a_scale, M, Y, ldy, acc_debug, st);
     if (group != 0) return cudaErrorNotSupported;
     return acc_debug ? launch<true>(w, Xq, a_scale, M, Y, ldy, acc_debug, st) : launch<false>(w, Xq, a_scale, M, Y, ldy, acc_debug, st);

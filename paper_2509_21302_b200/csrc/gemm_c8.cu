@@ -594,7 +594,7 @@ cudaError_t qvggt_launch_gemm_c8(const qvggt_weights *w, const signed char *Xq8,
 {
     if (M == 0) return cudaSuccess;
     if (!w->Wq8) return cudaErrorNotSupported;      // the handle was prepared without the 8-bit-container copy
-    if (!acc_debug && qvggt_gemm_small_wins(w, M, false, false)) return qvggt_launch_gemm_small(w, Xq8, w->Wq8, false, a_scale, false, M, Y, ldy, true, st);
+    if (!acc_debug && qvggt_gemm_small_wins(w, M, false, false)) return qvggt_launch_gemm_small(w, Xq8, w->Wq8, false, a_scale, false, M, Y, ldy, st);
     return acc_debug ? launch<true>(w, w->Wq8, Xq8, a_scale, M, Y, ldy, acc_debug, st, ptx::kWaitLimitCycles, 0)
                      : launch<false>(w, w->Wq8, Xq8, a_scale, M, Y, ldy, acc_debug, st, ptx::kWaitLimitCycles, 0);
 }
@@ -621,7 +621,7 @@ cudaError_t qvggt_launch_gemm_c8_packed_weights(const qvggt_weights *w, const si
     if (M == 0) return cudaSuccess;
     cudaError_t e = qvggt_launch_unpack_w4(w, w_scratch, st);
     if (e != cudaSuccess) return e;
-    if (!acc_debug && qvggt_gemm_small_wins(w, M, false, false)) return qvggt_launch_gemm_small(w, Xq8, w_scratch, false, a_scale, false, M, Y, ldy, false, st);
+    if (!acc_debug && qvggt_gemm_small_wins(w, M, false, false)) return qvggt_launch_gemm_small(w, Xq8, w_scratch, false, a_scale, false, M, Y, ldy, st);
     return acc_debug ? launch<true>(w, w_scratch, Xq8, a_scale, M, Y, ldy, acc_debug, st, ptx::kWaitLimitCycles, 0)
                      : launch<false>(w, w_scratch, Xq8, a_scale, M, Y, ldy, acc_debug, st, ptx::kWaitLimitCycles, 0);
 }
@@ -630,7 +630,7 @@ cudaError_t qvggt_launch_gemm_c8_expanded(const qvggt_weights *w, const signed c
                                           long long ldy, const signed char *w_expanded, int *acc_debug, cudaStream_t st)
 {
     if (M == 0) return cudaSuccess;
-    if (!acc_debug && qvggt_gemm_small_wins(w, M, false, false)) return qvggt_launch_gemm_small(w, Xq8, w_expanded, false, a_scale, false, M, Y, ldy, false, st);
+    if (!acc_debug && qvggt_gemm_small_wins(w, M, false, false)) return qvggt_launch_gemm_small(w, Xq8, w_expanded, false, a_scale, false, M, Y, ldy, st);
     return acc_debug ? launch<true>(w, w_expanded, Xq8, a_scale, M, Y, ldy, acc_debug, st, ptx::kWaitLimitCycles, 0)
                      : launch<false>(w, w_expanded, Xq8, a_scale, M, Y, ldy, acc_debug, st, ptx::kWaitLimitCycles, 0);
 }
@@ -648,6 +648,6 @@ cudaError_t qvggt_launch_gemm_c8_grouped(const qvggt_weights *w, const signed ch
 {
     if (M == 0) return cudaSuccess;
     if (!w->Wq8 || w->bits != 4) return cudaErrorNotSupported;
-    if (!acc_debug && qvggt_gemm_small_wins(w, M, false, true)) return qvggt_launch_gemm_small(w, Xq8, w->Wq8, false, a_scale, true, M, Y, ldy, true, st);
+    if (!acc_debug && qvggt_gemm_small_wins(w, M, false, true)) return qvggt_launch_gemm_small(w, Xq8, w->Wq8, false, a_scale, true, M, Y, ldy, st);
     return acc_debug ? grp::launch<true>(w, Xq8, a_scale, M, Y, ldy, acc_debug, st) : grp::launch<false>(w, Xq8, a_scale, M, Y, ldy, acc_debug, st);
 }

@@ -3,12 +3,11 @@
 //
 // With a handful of rows nothing is bound by the tensor core: the layer is its N K bytes of weights (0.15 - 0.6 us of memory
 // bandwidth) plus latency.  The persistent kernels give such a layer N / 256 CTA pairs, each of which walks all of K at the pace
-// of full 256-row MMAs behind TMA and tensor-memory set-up: 6.8 us at 5 rows of K = N = 1024, 13.6 us at K = 4096.
+// of full 256-row MMAs behind TMA and tensor-memory set-up.
 // Here a CTA owns 16 channels and its warps share K, so that all weight bytes of the layer are in flight at once; they go from
 // global memory straight into the fragments of mma.sync (whose rate does not matter here), a lane's 16 consecutive bytes of a
 // row standing for whichever k the fragment asks for: the same permutation of K for both operands, which an integer sum does not
-// see.  The warps' partial sums meet in shared memory.  The weights do not depend on the previous kernel of the stream
-// (unless they come from a scratch): their loads are issued before the wait for it.
+// see.  The warps' partial sums meet in shared memory.
 #include <cuda_bf16.h>
 
 #include "qvggt_internal.cuh"
@@ -59,12 +58,10 @@ struct Piece {
 };
 
 // NT: tiles of 8 token rows per CTA.  WARPS x BLOCKS x 128 = K: a warp takes the 128-code blocks warp, warp + WARPS, ...
-// w_early: the weights were complete before the previous kernel of the stream began (see qvggt_launch_rsq).
 template <bool PACKED, bool GROUPED, int NT, int WARPS, int BLOCKS>
 __global__ void __launch_bounds__(WARPS * 32)
 gemm_small_kernel(const unsigned char *__restrict__ Xq, const unsigned char *__restrict__ Wq, const float *__restrict__ a_scale,
-                  const float *__restrict__ w_scale, const uint16_t *__restrict__ bias, uint16_t *__restrict__ Y, long long ldy, int M,
-                  int w_early)
+                  const float *__restrict__ w_scale, const uint16_t *__restrict__ bias, uint16_t *__restrict__ Y, long long ldy, int M)
 {
     constexpr int TOK = 8 * NT, KB = WARPS * BLOCKS, ROW = KB * (PACKED ? 64 : 128);    // bytes of a row of codes
     constexpr int PARTS = GROUPED ? KB : WARPS;             // partial sums per output
@@ -73,7 +70,7 @@ gemm_small_kernel(const unsigned char *__restrict__ Xq, const unsigned char *__r
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const int n0 = blockIdx.x * CH, m0 = blockIdx.y * TOK;
     ptx::grid_launch_dependents();
-    if (!w_early) ptx::grid_dependency_wait();
+    ptx::grid_dependency_wait();
     const unsigned char *w0 = Wq + (long long)(n0 + g) * ROW, *w1 = w0 + 8 * ROW;
     Piece<PACKED> wa[BLOCKS], wb[BLOCKS];
 #pragma unroll
@@ -81,7 +78,6 @@ gemm_small_kernel(const unsigned char *__restrict__ Xq, const unsigned char *__r
         wa[i].load(w0, warp + WARPS * i, t);
         wb[i].load(w1, warp + WARPS * i, t);
     }
-    if (w_early) ptx::grid_dependency_wait();
     int acc[NT][4];
 #pragma unroll
     for (int j = 0; j < NT; ++j)
@@ -152,7 +148,7 @@ gemm_small_kernel(const unsigned char *__restrict__ Xq, const unsigned char *__r
 }
 
 template <bool PACKED, bool GROUPED, int NT, int WARPS, int BLOCKS>
-cudaError_t launch(const qvggt_weights *w, const void *Xq, const void *Wq, const float *a_scale, int M, void *Y, long long ldy, bool w_early, cudaStream_t st)
+cudaError_t launch(const qvggt_weights *w, const void *Xq, const void *Wq, const float *a_scale, int M, void *Y, long long ldy, cudaStream_t st)
 {
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -165,42 +161,43 @@ cudaError_t launch(const qvggt_weights *w, const void *Xq, const void *Wq, const
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, gemm_small_kernel<PACKED, GROUPED, NT, WARPS, BLOCKS>, static_cast<const unsigned char *>(Xq),
                               static_cast<const unsigned char *>(Wq), a_scale, (const float *)w->w_scale, (const uint16_t *)w->bias,
-                              static_cast<uint16_t *>(Y), ldy, M, w_early ? 1 : 0);
+                              static_cast<uint16_t *>(Y), ldy, M);
 }
 
 template <bool PACKED, bool GROUPED>
-cudaError_t dispatch(const qvggt_weights *w, const void *Xq, const void *Wq, const float *a_scale, int M, void *Y, long long ldy, bool w_early, cudaStream_t st)
+cudaError_t dispatch(const qvggt_weights *w, const void *Xq, const void *Wq, const float *a_scale, int M, void *Y, long long ldy, cudaStream_t st)
 {
     if (w->K == 1024) {
-        if (M <= 8) return launch<PACKED, GROUPED, 1, 8, 1>(w, Xq, Wq, a_scale, M, Y, ldy, w_early, st);
-        if (M <= 16) return launch<PACKED, GROUPED, 2, 8, 1>(w, Xq, Wq, a_scale, M, Y, ldy, w_early, st);
-        return launch<PACKED, GROUPED, 4, 8, 1>(w, Xq, Wq, a_scale, M, Y, ldy, w_early, st);
+        if (M <= 8) return launch<PACKED, GROUPED, 1, 8, 1>(w, Xq, Wq, a_scale, M, Y, ldy, st);
+        if (M <= 16) return launch<PACKED, GROUPED, 2, 8, 1>(w, Xq, Wq, a_scale, M, Y, ldy, st);
+        return launch<PACKED, GROUPED, 4, 8, 1>(w, Xq, Wq, a_scale, M, Y, ldy, st);
     }
-    if (M <= 8) return launch<PACKED, GROUPED, 1, 16, 2>(w, Xq, Wq, a_scale, M, Y, ldy, w_early, st);
-    return launch<PACKED, GROUPED, 2, 16, 2>(w, Xq, Wq, a_scale, M, Y, ldy, w_early, st);
+    if (M <= 8) return launch<PACKED, GROUPED, 1, 16, 2>(w, Xq, Wq, a_scale, M, Y, ldy, st);
+    return launch<PACKED, GROUPED, 2, 16, 2>(w, Xq, Wq, a_scale, M, Y, ldy, st);
 }
 
 }  // namespace
 
 // Where the lines lie: this kernel's time grows with M N K (its rate is that of mma.sync), the persistent kernels' hardly moves
 // below one round of tiles.  Measured (us, this kernel / the other one):
-//   one code per byte   K = 1024: N = 3072, M = 64 4.8 / 5.0, M = 128 6.3 / 5.0; N = 1024, M = 128 3.6 / 4.9, M = 256 4.4 / 5.0
-//                       K = 4096: N = 1024, M = 128 6.7 / 9.0, M = 256 12.8 / 9.1
-//   packed              K = 1024: N = 3072, M = 256 7.6 / 8.2; N = 4096, M = 256 9.7 / 8.3; N = 1024, M = 512 5.5 / 8.2
-//                       K = 4096: N = 1024, M = 256 9.4 / 16.2, M = 512 15.9 / 16.3
-//   group scales        K = 1024: N = 3072, M = 128 6.5 / 7.0; N = 4096, M = 128 8.0 / 7.1; N = 1024, M = 256 4.7 / 7.0
-//                       K = 4096: N = 1024, M = 256 15.5 / 16.9, M = 512 29.8 / 17
+//   one code per byte   K = 1024: N = 3072, M = 64 4.9 / 4.6, M = 128 6.3 / 4.7; N = 1024, M = 192 4.1 / 4.6; N = 4096, M = 32 4.3 / 4.9
+//                       K = 4096: N = 1024, M = 128 7.3 / 8.2, M = 192 10.2 / 8.2
+//   packed              K = 1024: N = 3072, M = 256 7.1 / 8.2; N = 4096, M = 192 7.2 / 8.2, M = 256 9.3 / 8.2
+//                       K = 4096: N = 1024, M = 256 8.9 / 16.7, M = 512 15.9 / 16.7
+//   group scales        K = 1024: N = 3072, M = 128 6.6 / 6.6, M = 192 8.1 / 6.6; N = 4096, M = 96 6.6 / 6.8; N = 1024, M = 256 4.3 / 6.5
+//                       K = 4096: N = 1024, M = 192 13.3 / 15.1, M = 256 17.3 / 15.1
+// and at 5 rows           K = 1024, N = 3072 2.3 / 4.5, packed 2.0 / 7.8, groups 2.4 / 6.3; K = 4096 2.5 / 8.0, 2.2 / 16.4, 3.1 / 14.8
 bool qvggt_gemm_small_wins(const qvggt_weights *w, int M, bool packed, bool grouped)
 {
     const long long outputs = (long long)M * w->N;
     if (w->K == 1024) return outputs <= (packed ? 3LL << 18 : grouped ? 3LL << 17 : 3LL << 16);
-    return outputs <= (packed ? 3LL << 17 : grouped ? 1LL << 18 : 1LL << 17);
+    return outputs <= (packed ? 3LL << 17 : grouped ? 3LL << 16 : 1LL << 17);
 }
 
 cudaError_t qvggt_launch_gemm_small(const qvggt_weights *w, const void *Xq, const void *Wq, bool packed, const float *a_scale, bool grouped, int M,
-                                    void *Y, long long ldy, bool w_early, cudaStream_t st)
+                                    void *Y, long long ldy, cudaStream_t st)
 {
     if (packed)
-        return grouped ? dispatch<true, true>(w, Xq, Wq, a_scale, M, Y, ldy, w_early, st) : dispatch<true, false>(w, Xq, Wq, a_scale, M, Y, ldy, w_early, st);
-    return grouped ? dispatch<false, true>(w, Xq, Wq, a_scale, M, Y, ldy, w_early, st) : dispatch<false, false>(w, Xq, Wq, a_scale, M, Y, ldy, w_early, st);
+        return grouped ? dispatch<true, true>(w, Xq, Wq, a_scale, M, Y, ldy, st) : dispatch<true, false>(w, Xq, Wq, a_scale, M, Y, ldy, st);
+    return grouped ? dispatch<false, true>(w, Xq, Wq, a_scale, M, Y, ldy, st) : dispatch<false, false>(w, Xq, Wq, a_scale, M, Y, ldy, st);
 }

@@ -39,16 +39,13 @@ void qvggt_block_release(int device, void *block, size_t block_bytes);
 // multipliers; also copies the bias and clears the status word, if given
 cudaError_t qvggt_launch_multipliers(const float *c, const signed char *v, int K, float *amul, float *wmul, cudaStream_t st,
                                      const uint16_t *bias = nullptr, int N = 0, uint16_t *bias_out = nullptr, int *status = nullptr);
-// is_weight: the rows are a handle's weights.  The launch then does not let the next kernel of the stream start before it is
-// complete, so that every later kernel -- which may itself start before ITS predecessor is complete -- can read the handle's
-// weights at once, without waiting for anything.
 cudaError_t qvggt_launch_rsq(const void *X, long long ldx, int M, int K, const float *mul, int group,
-                             unsigned char *Xq, float *scales, cudaStream_t st, bool is_weight = false);
+                             unsigned char *Xq, float *scales, cudaStream_t st);
 cudaError_t qvggt_launch_rsq_c8(const void *X, long long ldx, int M, int K, const float *mul, int bits, signed char *Xq8,
                                 float *scales, cudaStream_t st, int group = 0, const void *w_packed = nullptr,
-                                void *w_expanded = nullptr, long long w_codes = 0, bool is_weight = false);
+                                void *w_expanded = nullptr, long long w_codes = 0);
 cudaError_t qvggt_launch_rsq_static_c8(const void *X, long long ldx, int M, int K, const float *mul, int bits, const float *delta,
-                                       signed char *Xq8, float *scales, cudaStream_t st, bool is_weight = false);
+                                       signed char *Xq8, float *scales, cudaStream_t st);
 cudaError_t qvggt_launch_ln_rsq_c8(const void *X, long long ldx, int M, int K, const float *mul, int bits, const float *gamma,
                                    const float *beta, float eps, signed char *Xq8, float *scales, void *ln_out, cudaStream_t st);
 cudaError_t qvggt_launch_gelu_rsq_c8(const void *X, long long ldx, int M, int K, const float *mul, int bits, signed char *Xq8,
@@ -64,10 +61,9 @@ cudaError_t qvggt_launch_rsq_tc(const void *X, long long ldx, int M, int K, cons
                                 float *scales, float *y_debug, int *status, cudaStream_t st);
 
 // gemm_small.cu: few rows; codes of both operands packed or one per byte, scales per token or per 128 channels.
-// w_early: the weights are the handle's own (not a scratch that an earlier kernel of the stream wrote).
 bool qvggt_gemm_small_wins(const qvggt_weights *w, int M, bool packed, bool grouped);
 cudaError_t qvggt_launch_gemm_small(const qvggt_weights *w, const void *Xq, const void *Wq, bool packed, const float *a_scale, bool grouped, int M,
-                                    void *Y, long long ldy, bool w_early, cudaStream_t st);
+                                    void *Y, long long ldy, cudaStream_t st);
 
 // gemm.cu
 cudaError_t qvggt_launch_gemm(const qvggt_weights *w, const unsigned char *Xq, const float *a_scale, int M,

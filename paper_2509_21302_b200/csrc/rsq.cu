@@ -180,7 +180,7 @@ template <int LOGT, int GROUP, bool C8 = false, int QMAX = 7, bool STATIC = fals
 __global__ void __launch_bounds__(SqGeom<LOGT>::CTA_THREADS, sq_ctas_per_sm(LOGT, LN))
 rsq_sq_kernel(const uint16_t *__restrict__ X, long long ldx, int M, const float *__restrict__ mul,
               unsigned char *__restrict__ Xq, float *__restrict__ scales, const float *__restrict__ static_delta,
-              const LnArgs ln, const QvggtExpand ex, int is_weight)
+              const LnArgs ln, const QvggtExpand ex)
 {
     static_assert(!STATIC || (C8 && GROUP == 0), "the static step size is built for one code per byte");
     static_assert(LN == 0 || (C8 && GROUP == 0 && !STATIC), "the fused LayerNorm is built for the dynamic one-code-per-byte path");
@@ -218,7 +218,7 @@ rsq_sq_kernel(const uint16_t *__restrict__ X, long long ldx, int M, const float 
     long long row = (long long)blockIdx.x * G::ROWS + slot;
     // the blocks may have become resident before the previous kernel in the stream finished (programmatic
     // dependent launch): no global memory is touched before that kernel is done
-    if (!is_weight) ptx::grid_launch_dependents();
+    ptx::grid_launch_dependents();
     ptx::grid_dependency_wait();
     if (row < M) {
         const unsigned char *src = reinterpret_cast<const unsigned char *>(X + row * ldx);
@@ -608,7 +608,7 @@ namespace {
 template <int LOGT, int GROUP, bool C8, int QMAX = 7, bool STATIC = false, int LN = 0>
 cudaError_t launch_sq(const uint16_t *x, long long ldx, int M, const float *mul, unsigned char *out, float *scales,
                       cudaStream_t st, const float *static_delta = nullptr, LnArgs ln = LnArgs{nullptr, nullptr, 0.0f, nullptr},
-                      QvggtExpand ex = QvggtExpand{nullptr, nullptr, 0}, bool is_weight = false)
+                      QvggtExpand ex = QvggtExpand{nullptr, nullptr, 0})
 {
     using G = SqGeom<LOGT>;
     constexpr int SMEM = G::SMEM + ((LN == 1 || LN == 2) ? 2 * G::K * 4 : 0);   // + the CTA's copy of gamma and beta
@@ -638,24 +638,22 @@ cudaError_t launch_sq(const uint16_t *x, long long ldx, int M, const float *mul,
     cfg.stream = st;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, rsq_sq_kernel<LOGT, GROUP, C8, QMAX, STATIC, LN>, x, ldx, M, mul, out, scales, static_delta, ln, ex, is_weight ? 1 : 0);
+    return cudaLaunchKernelEx(&cfg, rsq_sq_kernel<LOGT, GROUP, C8, QMAX, STATIC, LN>, x, ldx, M, mul, out, scales, static_delta, ln, ex);
 }
 
 }  // namespace
 
 cudaError_t qvggt_launch_rsq_c8(const void *X, long long ldx, int M, int K, const float *mul, int bits, signed char *Xq8,
-                                float *scales, cudaStream_t st, int group, const void *w_packed, void *w_expanded, long long w_codes,
-                                bool is_weight)
+                                float *scales, cudaStream_t st, int group, const void *w_packed, void *w_expanded, long long w_codes)
 {
     if (M == 0) return cudaSuccess;
     const uint16_t *x = static_cast<const uint16_t *>(X);
     unsigned char *out = reinterpret_cast<unsigned char *>(Xq8);
-    const LnArgs none{nullptr, nullptr, 0.0f, nullptr};
-    const QvggtExpand nothing{nullptr, nullptr, 0};
     if (w_packed) {
         // the same launch also expands w_codes packed weight codes (4-bit, token-wise activations only)
         if (group != 0 || bits != 4) return cudaErrorNotSupported;
         const QvggtExpand ex{static_cast<const uint4 *>(w_packed), static_cast<uint4 *>(w_expanded), w_codes / 32};
+        const LnArgs none{nullptr, nullptr, 0.0f, nullptr};
         return K == 1024 ? launch_sq<5, 0, true>(x, ldx, M, mul, out, scales, st, nullptr, none, ex)
                          : launch_sq<6, 0, true>(x, ldx, M, mul, out, scales, st, nullptr, none, ex);
     }
@@ -664,25 +662,23 @@ cudaError_t qvggt_launch_rsq_c8(const void *X, long long ldx, int M, int K, cons
         return K == 1024 ? launch_sq<5, 128, true>(x, ldx, M, mul, out, scales, st) : launch_sq<6, 128, true>(x, ldx, M, mul, out, scales, st);
     }
     if (bits == 8)
-        return K == 1024 ? launch_sq<5, 0, true, 127>(x, ldx, M, mul, out, scales, st, nullptr, none, nothing, is_weight)
-                         : launch_sq<6, 0, true, 127>(x, ldx, M, mul, out, scales, st, nullptr, none, nothing, is_weight);
-    return K == 1024 ? launch_sq<5, 0, true>(x, ldx, M, mul, out, scales, st, nullptr, none, nothing, is_weight)
-                     : launch_sq<6, 0, true>(x, ldx, M, mul, out, scales, st, nullptr, none, nothing, is_weight);
+        return K == 1024 ? launch_sq<5, 0, true, 127>(x, ldx, M, mul, out, scales, st)
+                         : launch_sq<6, 0, true, 127>(x, ldx, M, mul, out, scales, st);
+    return K == 1024 ? launch_sq<5, 0, true>(x, ldx, M, mul, out, scales, st)
+                     : launch_sq<6, 0, true>(x, ldx, M, mul, out, scales, st);
 }
 
 cudaError_t qvggt_launch_rsq_static_c8(const void *X, long long ldx, int M, int K, const float *mul, int bits, const float *delta,
-                                       signed char *Xq8, float *scales, cudaStream_t st, bool is_weight)
+                                       signed char *Xq8, float *scales, cudaStream_t st)
 {
     if (M == 0) return cudaSuccess;
     const uint16_t *x = static_cast<const uint16_t *>(X);
     unsigned char *out = reinterpret_cast<unsigned char *>(Xq8);
-    const LnArgs none{nullptr, nullptr, 0.0f, nullptr};
-    const QvggtExpand nothing{nullptr, nullptr, 0};
     if (bits == 8)
-        return K == 1024 ? launch_sq<5, 0, true, 127, true>(x, ldx, M, mul, out, scales, st, delta, none, nothing, is_weight)
-                         : launch_sq<6, 0, true, 127, true>(x, ldx, M, mul, out, scales, st, delta, none, nothing, is_weight);
-    return K == 1024 ? launch_sq<5, 0, true, 7, true>(x, ldx, M, mul, out, scales, st, delta, none, nothing, is_weight)
-                     : launch_sq<6, 0, true, 7, true>(x, ldx, M, mul, out, scales, st, delta, none, nothing, is_weight);
+        return K == 1024 ? launch_sq<5, 0, true, 127, true>(x, ldx, M, mul, out, scales, st, delta)
+                         : launch_sq<6, 0, true, 127, true>(x, ldx, M, mul, out, scales, st, delta);
+    return K == 1024 ? launch_sq<5, 0, true, 7, true>(x, ldx, M, mul, out, scales, st, delta)
+                     : launch_sq<6, 0, true, 7, true>(x, ldx, M, mul, out, scales, st, delta);
 }
 
 cudaError_t qvggt_launch_ln_rsq_c8(const void *X, long long ldx, int M, int K, const float *mul, int bits, const float *gamma,
@@ -720,16 +716,14 @@ cudaError_t qvggt_launch_gelu_rsq_c8(const void *X, long long ldx, int M, int K,
 }
 
 cudaError_t qvggt_launch_rsq(const void *X, long long ldx, int M, int K, const float *mul, int group,
-                             unsigned char *Xq, float *scales, cudaStream_t st, bool is_weight)
+                             unsigned char *Xq, float *scales, cudaStream_t st)
 {
     if (M == 0) return cudaSuccess;
     const uint16_t *x = static_cast<const uint16_t *>(X);
-    const LnArgs none{nullptr, nullptr, 0.0f, nullptr};
-    const QvggtExpand nothing{nullptr, nullptr, 0};
     if (group == 128)
         return K == 1024 ? launch_sq<5, 128, false>(x, ldx, M, mul, Xq, scales, st) : launch_sq<6, 128, false>(x, ldx, M, mul, Xq, scales, st);
-    return K == 1024 ? launch_sq<5, 0, false>(x, ldx, M, mul, Xq, scales, st, nullptr, none, nothing, is_weight)
-                     : launch_sq<6, 0, false>(x, ldx, M, mul, Xq, scales, st, nullptr, none, nothing, is_weight);
+    return K == 1024 ? launch_sq<5, 0, false>(x, ldx, M, mul, Xq, scales, st)
+                     : launch_sq<6, 0, false>(x, ldx, M, mul, Xq, scales, st);
 }
 
 cudaError_t qvggt_launch_max_reduce(const float *in, int n, float *out, cudaStream_t st)
