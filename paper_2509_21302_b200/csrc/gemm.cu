@@ -13,7 +13,7 @@
 // CTA stages 128 token rows and 128 weight rows, one thread of the leader CTA issues tcgen05.mma.cta_group::2
 // for both; a single-CTA configuration measured 10-35 % slower on every VGGT shape: the pair halves the
 // weight traffic).
-//   warps 0-7    epilogue: TMEM -> registers -> scale, bias, bf16 -> swizzled staging -> TMA store
+//   warps 0-7    epilogue: TMEM -> registers -> scale, bias, bf16 -> swizzled staging -> whole-line stores
 //   warps 8-15   converters: packed stage -> registers -> int8 operand stage
 //   warp  16     one thread issues tcgen05.mma and the commits that release stages / publish accumulators
 //   warp  17     one thread issues the TMA loads of packed tiles

@@ -7,16 +7,14 @@
 // stages by TMA and nothing in this kernel touches an operand byte with an ordinary instruction.  Per K-block
 // a CTA's shared memory sees one TMA write and one tensor-core read of its 32 KB of operands, the minimum.
 //
-// Persistent and warp-specialised; a worker is a pair of CTAs on neighbouring SMs (tile 256 tokens x 256
-// channels, each CTA stages 128 token rows and 128 weight rows; one thread of the leader CTA issues
-// tcgen05.mma.cta_group::2.kind::i8 for both; accumulators int32 in tensor memory, two buffers of 256 columns).
-//   warps 0..7   epilogue: TMEM -> registers -> scale, bias, bf16 -> swizzled staging -> TMA store
-//   warp  8      one thread issues tcgen05.mma and the commits that release stages / publish accumulators
+// Persistent and warp-specialised; a worker is a pair of CTAs on neighbouring SMs (tile 256 tokens x BN = 256 or 128
+// channels, each CTA stages 128 token rows and BN / 2 weight rows; one thread of the leader CTA issues
+// tcgen05.mma.cta_group::2.kind::i8 for both; accumulators int32 in tensor memory, two buffers of BN columns).
+//   warps 0..7   epilogue: TMEM -> registers -> scale, bias, bf16 -> swizzled staging -> whole-line stores; no warp waits for another
+//   warp  8      one elected thread issues tcgen05.mma and the commits that release stages / publish accumulators
 //   warp  9      one thread per CTA issues the TMA loads of its half of every operand stage; both CTAs signal
 //                the leader's "full" barrier (cta_group::2 form of the load)
-// The tiles are dealt round-robin to the workers.  (Cutting the tiles of a short last round into halves of 128
-// channels was built and measured: an N = 128 MMA takes ~0.75 of an N = 256 one, a half tile ~0.9 of a whole
-// one, and the extra bookkeeping cost the main path 5 %: not kept.)
+// The tiles are dealt round-robin to the workers.
 // Every wait is bounded; on expiry the kernel records a code in *status and all roles fall through to the
 // common exit, where tensor memory is released.
 #include <cuda.h>
@@ -256,12 +254,17 @@ gemm_c8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
 // ------------------------------------------------------------------------------------------------
 // The same TMA-fed CTA-pair design for one activation scale per token per 128 rotated channels (an extension of the
 // paper's token-wise granularity; the weights keep one scale per output channel).  A K-block of 128 codes is one scale
-// group, so every K-block accumulates into its own tensor-memory buffer (two of 128 columns, ping-pong) and the
-// epilogue warps rescale it while the next one runs:
+// group, so every K-block accumulates into its own tensor-memory buffer (four of 128 columns, handed over two at a
+// time) and the epilogue warps rescale a pair while the next one runs:
 //   s = fl(s + fl(float(acc_g) * a_scale[m][g])), g ascending;  Y = bf16(fl(fl(s * w_scale[n]) + bias[n])).
-// Tile 256 tokens x 128 channels per pair; an epilogue thread keeps the 64 running sums of its row in registers (10
-// warps per CTA leave 168 registers per thread).  Per K-block the pair does 376 cycles of MMA work (four N = 128
-// instructions) against 3 instructions per output element in the epilogue: the epilogue sets the pace.
+// Tile 256 tokens x 128 channels per pair; an epilogue thread keeps 32 running sums of its row in registers.  The epilogue
+// sets the pace: per K-block ~280 cycles of MMA work against 725 (K = 4096) - 1000 (K = 1024), of which the arithmetic
+// (conversion, packed multiply, packed uncontracted add) is ~250, the wait for the pair and its hand-over ~200 and, at
+// K = 1024, the end of a tile ~250 (2050 cycles for eight K-blocks).  With the arithmetic taken out of a copy for timing the launch
+// takes 58 instead of 82 us (10 992 rows, K = 1024, N = 4096), without the operand loads as well 52.  Measured and slower:
+// the whole next K-block's sums in registers (they do not fit beside the running sums, not even with the issuing warps' registers
+// moved to these), accumulators released one by one (84 us), ordinary stores instead of the TMA store (87 us: the
+// warp then waits for its own lines), the next tile's first scales fetched ahead (84 us).
 namespace grp {
 
 constexpr int GN = 128;                                // channels per tile

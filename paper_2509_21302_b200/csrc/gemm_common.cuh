@@ -1,6 +1,6 @@
 // Pieces shared by the integer GEMM kernels (gemm.cu, gemm_c8.cu, gemm_grouped.cu): the per-K-block MMA issue,
 // the rescale + bias + bf16 arithmetic of the epilogue (Sec. 3.2: both scales stay outside the integer sum), the
-// staging tile behind every TMA store, and the host-side per-device configuration of a kernel.
+// staging tiles behind the output stores, and the host-side per-device configuration of a kernel.
 #pragma once
 #include <cuda.h>
 #include <cuda_runtime.h>
@@ -50,32 +50,6 @@ __device__ __forceinline__ void load_channel_params(float *s_ws, float *s_bs, co
     const bool ch_ok = nt0 + e < N;
     s_ws[e] = ch_ok ? __ldg(w_scale + nt0 + e) : 0.0f;
     s_bs[e] = (ch_ok && bias) ? __uint_as_float(static_cast<uint32_t>(__ldg(bias + nt0 + e)) << 16) : 0.0f;
-}
-
-// 32 consecutive channels of one token row: fl(fl(float(acc) * fl(a_scale * w_scale)) + bias), every operation
-// rounded to nearest, then bf16 (round to nearest even), two per word.  `as2` holds a_scale in both halves; ws / bs
-// point at the 32 channel scales / biases (fp32, 16-byte aligned, shared memory).
-// The additions are scalar intrinsics: a packed multiply feeding a packed add was observed to be contracted
-// into one fused operation (single rounding).
-__device__ __forceinline__ void scale_bias_bf16_x32(const uint32_t (&raw)[32], uint64_t as2, const float *ws, const float *bs,
-                                                    uint32_t (&out)[16])
-{
-#pragma unroll
-    for (int j = 0; j < 32; j += 4) {
-        const ulonglong2 w2 = *reinterpret_cast<const ulonglong2 *>(ws + j);
-        const ulonglong2 b2 = *reinterpret_cast<const ulonglong2 *>(bs + j);
-        uint64_t z01 = ptx::f32x2_pack(static_cast<float>(static_cast<int>(raw[j])), static_cast<float>(static_cast<int>(raw[j + 1])));
-        uint64_t z23 = ptx::f32x2_pack(static_cast<float>(static_cast<int>(raw[j + 2])), static_cast<float>(static_cast<int>(raw[j + 3])));
-        z01 = ptx::f32x2_mul(z01, ptx::f32x2_mul(as2, w2.x));
-        z23 = ptx::f32x2_mul(z23, ptx::f32x2_mul(as2, w2.y));
-        float y0, y1, y2, y3, c0, c1, c2, c3;
-        ptx::f32x2_unpack(z01, y0, y1);
-        ptx::f32x2_unpack(z23, y2, y3);
-        ptx::f32x2_unpack(b2.x, c0, c1);
-        ptx::f32x2_unpack(b2.y, c2, c3);
-        out[j >> 1] = ptx::pack_bf16x2(__fadd_rn(y0, c0), __fadd_rn(y1, c1));
-        out[(j >> 1) + 1] = ptx::pack_bf16x2(__fadd_rn(y2, c2), __fadd_rn(y3, c3));
-    }
 }
 
 // 16 rows x 64 channels of a tile as 16x256b fragments (raw[4 b + 2 h + c]: row lane / 4 + 8 h, channel 8 b + 2 (lane mod 4) + c):
@@ -233,18 +207,6 @@ __device__ __forceinline__ void dump_acc_x16(int *dst, const uint32_t (&raw)[16]
     uint4 *d = reinterpret_cast<uint4 *>(dst);
 #pragma unroll
     for (int q = 0; q < 4; ++q) d[q] = make_uint4(raw[4 * q], raw[4 * q + 1], raw[4 * q + 2], raw[4 * q + 3]);
-}
-
-// 32 raw int32 sums of one row -> global memory (debug dump), optionally shifted right (the packed kernels carry
-// the codes in the high half-byte, so their raw sums are 256 x the integer sums).
-template <int SHIFT>
-__device__ __forceinline__ void dump_acc_x32(int *dst, const uint32_t (&raw)[32])
-{
-    uint4 *d = reinterpret_cast<uint4 *>(dst);
-#pragma unroll
-    for (int q = 0; q < 8; ++q)
-        d[q] = make_uint4(static_cast<int>(raw[4 * q]) >> SHIFT, static_cast<int>(raw[4 * q + 1]) >> SHIFT,
-                          static_cast<int>(raw[4 * q + 2]) >> SHIFT, static_cast<int>(raw[4 * q + 3]) >> SHIFT);
 }
 
 }  // namespace gemmc
