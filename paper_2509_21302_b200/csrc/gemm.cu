@@ -59,8 +59,8 @@ struct C {
     static constexpr int CHUNKS = ROWS * 4 / GROUP_THREADS;   // 16-byte packed pieces per thread per stage
     static constexpr int OFF_UP = 0;                       // operand stages first: they need 1024-byte alignment
     static constexpr int OFF_STG = OFF_UP + US * UP_STAGE;
-    static constexpr int OFF_CH = OFF_STG + EPI_WARPS * STG_BYTES;   // per-channel scale and bias of two tiles, fp32
-    static constexpr int OFF_PK = OFF_CH + 2 * ACC_BUFS * BN * 4;
+    static constexpr int OFF_CH = OFF_STG + EPI_WARPS * STG_BYTES;   // per warp: scales and biases of its BN / 2 channels, fp32
+    static constexpr int OFF_PK = OFF_CH + EPI_WARPS * BN * 4;
     static constexpr int OFF_BAR = OFF_PK + PS * PK_STAGE; // pfull[PS] pempty[PS] ufull[US] uempty[US] tfull[2] tempty[2]
     static constexpr int NBARS = 2 * PS + 2 * US + 2 * ACC_BUFS;
     static constexpr int OFF_TMEM = OFF_BAR + NBARS * 8;
@@ -139,21 +139,25 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
         const int quarter = warp & 3, chalf = warp >> 2;   // TMEM lane quarter, column half
         unsigned char *stg = smem + C::OFF_STG + warp * STG_BYTES;
         const uint32_t stg_addr = sbase + C::OFF_STG + warp * STG_BYTES;
-        float *s_ws = reinterpret_cast<float *>(smem + C::OFF_CH);          // [2][BN] per-channel scale of the tile
-        float *s_bs = s_ws + ACC_BUFS * BN;                                   // [2][BN] bias as fp32
+        float *wsb = reinterpret_cast<float *>(smem + C::OFF_CH) + warp * BN, *bsb = wsb + BN / 2;    // the warp's channel scales, biases
         const uint32_t leader_tempty = ptx::map_to_cta(bar_tempty, 0);
         const uint64_t one2 = ptx::f32x2_one(N & 127);                       // N is a multiple of 128
         bool alive = true;
         for (int t = 0; t < my_tiles; ++t) {
             const int tile = worker + t * workers;
             const int m0 = (tile / n_tiles) * (BM * CG) + (int)rank * BM + quarter * 32;
-            const int nt0 = (tile % n_tiles) * BN;             // first channel of the tile
-            const int n0 = nt0 + chalf * 128;                  // first channel of this warp's half
+            const int n0 = (tile % n_tiles) * BN + chalf * 128;    // first channel of this warp's half
             const int b = t & 1;
             const bool cols_ok = n0 < N;                       // N is a multiple of 128: a half tile is all in or all out
-            // per-channel scale and bias of the tile -> shared memory; buffer b was last read two tiles ago,
-            // and every epilogue warp has passed the group barrier of the tile in between since then
-            gemmc::load_channel_params(s_ws + b * BN, s_bs + b * BN, w_scale, bias, nt0, N, threadIdx.x);   // 256 threads, one channel each
+            // The scales and biases of the warp's channels: each warp keeps its own copy in shared memory, so that no warp ever
+            // waits for another.
+            float my_ws[4], my_bs[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int n = n0 + 32 * e + lane;
+                my_ws[e] = cols_ok ? __ldg(w_scale + n) : 0.0f;
+                my_bs[e] = (cols_ok && bias) ? __uint_as_float(static_cast<uint32_t>(__ldg(bias + n)) << 16) : 0.0f;
+            }
             // a_scale / 256: exact (power of two), cancels the factor 256 carried by the raw accumulator
             uint64_t as2[2][2];                                // rows lane / 4 + 8 h of the warp's 16 u .. 16 u + 15
 #pragma unroll
@@ -162,8 +166,13 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
                 const float as = gm < M ? __fmul_rn(__ldg(a_scale + gm), 0.00390625f) : 0.0f;
                 as2[u >> 1][u & 1] = ptx::f32x2_pack(as, as);
             }
-            // the epilogue warps meet (named barrier 1: publishes s_ws / s_bs), then every warp polls the accumulator barrier itself
-            asm volatile("bar.sync %0, %1;" ::"r"(1), "r"(EPI_WARPS * 32) : "memory");
+            __syncwarp();                                      // the previous tile's last reads
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                wsb[32 * e + lane] = my_ws[e];
+                bsb[32 * e + lane] = my_bs[e];
+            }
+            __syncwarp();
             {
                 int ok = 1;
                 if (lane == 0) ok = (alive && ptx::mbar_wait(bar_tfull + 8 * b, (t >> 1) & 1, s_abort, status, QVGGT_DEV_TIMEOUT_ACCUM, 32)) ? 1 : 0;
@@ -171,8 +180,6 @@ gemm_w4a4_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constan
             }
             ptx::tc_fence_after_sync();
             if (alive) {
-                const float *wsb = s_ws + b * BN + chalf * 128;
-                const float *bsb = s_bs + b * BN + chalf * 128;
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {                  // rows 16 u .., channels 64 h .. of the warp's 32 x 128
                     const int u = c & 1, h = c >> 1, m = m0 + 16 * u, n = n0 + 64 * h;

@@ -1,5 +1,4 @@
-// Pieces shared by the two exact rotate-smooth-quantize kernels (rsq.cu, rsq_wide.cu): butterflies, the statistics' summation
-// tree, GELU, asynchronous copies.
+// Pieces of the exact rotate-smooth-quantize kernel (rsq.cu): butterflies, the statistics' summation tree, GELU, asynchronous copies.
 #pragma once
 #include "sm100_ptx.cuh"
 
