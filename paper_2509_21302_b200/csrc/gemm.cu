@@ -288,6 +288,7 @@ cudaError_t launch(const qvggt_weights *w, const unsigned char *Xq, const float 
         return cudaErrorInvalidValue;
     const int total_tiles = ((M + BM * CG - 1) / (BM * CG)) * ((N + BN - 1) / BN);
     const int workers = total_tiles < max_workers ? total_tiles : max_workers;
+    const bool programmatic = (long long)((total_tiles + workers - 1) / workers) * (K / BK) <= 100;      // K-blocks per worker
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(workers * CG);
     cfg.blockDim = dim3(THREADS);
@@ -299,7 +300,7 @@ cudaError_t launch(const qvggt_weights *w, const unsigned char *Xq, const float 
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;      // see grid_dependency_wait()
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 2;
+    cfg.numAttrs = programmatic ? 2 : 1;
     return cudaLaunchKernelEx(&cfg, gemm_w4a4_kernel<DUMP>, map_x, map_w, static_cast<uint16_t *>(Y), ldy, a_scale, (const float *)w->w_scale,
                               (const uint16_t *)w->bias, acc_debug, M, N, K, w->status);
 }
