@@ -253,7 +253,8 @@ int qvggt_debug_starved_linear_c8(const qvggt_weights_t *w, const signed char *X
  * The other half of the upstream fusion: fc2's input is the MLP's activation function applied to fc1's output.  The
  * paper does not name the function; the transformer blocks VGGT is built from use the exact GELU x Phi(x) (Phi the
  * standard normal distribution function), which is what is computed here, in fp32, to within one bf16 ulp of the
- * exactly rounded value (results of magnitude below 2^-120, i.e. x < -12.9, may be flushed to zero).
+ * exactly rounded value (results of magnitude below 2^-120, i.e. x < -12.9, may be flushed to zero).  NaN and infinite
+ * inputs give NaN.
  * qvggt_gelu_rotate_smooth_quantize_c8 applies it to every element on its way into the activation path of
  * qvggt_rotate_smooth_quantize_c8 -- the activated tensor (the largest activation of the block) never goes to memory --
  * and returns, bit for bit, the result of qvggt_gelu followed by qvggt_rotate_smooth_quantize_c8.

@@ -43,29 +43,38 @@ __device__ __forceinline__ float tree_sum_squares(const float (&a)[T])
 }
 
 // GELU x Phi(x) (the activation between the two linears of the MLP: the producer of fc2's input) of two bf16 values, rounded to
-// bf16.  With t = |x| the tail Q(t) = 1 - Phi(t) is taken as 2^P(t), P a polynomial of degree 9 (own minimax fit of log2 Q on
-// [0, 13.25], by iteratively reweighted least squares), so that the negative tail keeps its RELATIVE accuracy; then
-// gelu(x) = max(x, 0) - t Q(t).  Relative error of Q with the fp32 evaluation below 5e-5; beyond 13.25 the tail is below 2^-126 and
-// flushes to zero.  The fused multiply-adds are written explicitly (the file is compiled without contraction).
-// One special-function operation per element (8 cycles of that unit each) and everything else two elements per instruction: with a
-// reciprocal beside the exponential and scalar arithmetic (37 instructions per pair instead of 19) the fused kernel was bound by both.
+// bf16, evaluated so that the negative tail keeps its RELATIVE accuracy.  With t = |x|, z = t / sqrt(2):
+//   Q(t) = 1 - Phi(t) = exp(-z^2) E(z) / 2,   E(z) = exp(z^2) erfc(z)  (smooth, from 1 down to ~1 / (z sqrt(pi))),
+//   E(z) ~ s P(s),  s = 1 / (1 + 0.55 z),  P a degree-4 polynomial (own weighted least-squares fit on z in [0, 9.6]: relative
+//   error below 6e-5), then gelu(x) = x - t Q for x >= 0 and -t Q for x < 0.
+// At most one bf16 ulp wherever the result is a normal number above 2^-120; below that (x < -12.9) the exponential flushes to
+// zero, with the sign of x.  NaN stays NaN, and an infinite x gives NaN (the product of infinity and a flushed tail).
+// Everything but the two special-function operations of an element (reciprocal, exp2) runs on two elements per instruction; each of
+// these operations rounds exactly like its scalar form, and no product feeds an addition that is not written as a fused one.
 __device__ __forceinline__ uint32_t gelu_bf16x2(uint32_t x)
 {
-    uint32_t a = x | 0x80008000u, pos;                     // -t
-    asm("max.bf16x2 %0, %1, %2;" : "=r"(a) : "r"(a), "r"(0xC154C154u));          // -13.25
-    asm("max.bf16x2 %0, %1, %2;" : "=r"(pos) : "r"(x), "r"(0u));
+    const uint32_t a = x | 0x80008000u;                    // -t
+    uint32_t pos;                                          // x, or -0 for x < 0; x = -0 counts as +0
+    asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(pos) : "r"(x), "r"(0x3F803F80u), "r"(0u));
+    asm("max.bf16x2 %0, %0, %1;" : "+r"(pos) : "r"(0x80008000u));
     const uint64_t nt = ptx::f32x2_pack(__uint_as_float(a << 16), __uint_as_float(a & 0xFFFF0000u));
-    constexpr float c[10] = {-1.00003052f, 1.15097892f, -0.458792716f, 0.053958077f, 0.00866845064f,       // P(-(-t)): odd terms negated
-                             0.00102148089f, 8.3747007e-05f, 4.47421826e-06f, 1.39110185e-07f, 1.90157845e-09f};
-    uint64_t p = ptx::f32x2_pack(c[9], c[9]);
-#pragma unroll
-    for (int i = 8; i >= 0; --i) p = ptx::f32x2_fma(p, nt, ptx::f32x2_pack(c[i], c[i]));
-    float p0, p1, q0, q1, y0, y1;
-    ptx::f32x2_unpack(p, p0, p1);
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(q0) : "f"(p0));
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(q1) : "f"(p1));
-    const uint64_t y = ptx::f32x2_fma(nt, ptx::f32x2_pack(q0, q1), ptx::f32x2_pack(__uint_as_float(pos << 16), __uint_as_float(pos & 0xFFFF0000u)));
-    ptx::f32x2_unpack(y, y0, y1);
+    auto both = [](float v) { return ptx::f32x2_pack(v, v); };
+    const uint64_t z = ptx::f32x2_mul(nt, both(-0.70710678f));
+    float d0, d1, s0, s1, w0, w1, e0, e1, y0, y1;
+    ptx::f32x2_unpack(ptx::f32x2_fma(both(0.55f), z, both(1.0f)), d0, d1);
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(s0) : "f"(d0));
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(s1) : "f"(d1));
+    const uint64_t s = ptx::f32x2_pack(s0, s1);
+    uint64_t p = both(-0.17450283f);
+    p = ptx::f32x2_fma(p, s, both(0.33387650f));
+    p = ptx::f32x2_fma(p, s, both(0.21415194f));
+    p = ptx::f32x2_fma(p, s, both(0.31633197f));
+    p = ptx::f32x2_fma(p, s, both(0.31008677f));
+    ptx::f32x2_unpack(ptx::f32x2_mul(ptx::f32x2_mul(z, z), both(-1.44269504f)), w0, w1);
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(w0));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(w1));
+    const uint64_t q = ptx::f32x2_mul(ptx::f32x2_mul(both(0.5f), ptx::f32x2_pack(e0, e1)), ptx::f32x2_mul(s, p));
+    ptx::f32x2_unpack(ptx::f32x2_fma(nt, q, ptx::f32x2_pack(__uint_as_float(pos << 16), __uint_as_float(pos & 0xFFFF0000u))), y0, y1);
     return ptx::pack_bf16x2(y0, y1);
 }
 

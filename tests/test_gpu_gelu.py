@@ -6,6 +6,8 @@ Contract (the GPU's GELU is an approximation of its own design, so it is not bit
   qvggt_gelu_rotate_smooth_quantize_c8: bit for bit the result of qvggt_gelu followed by
   qvggt_rotate_smooth_quantize_c8, and therefore the oracle's quantizer applied to the GPU's own bf16 GELU output.
 """
+import hashlib
+
 import numpy as np
 import pytest
 import torch
@@ -55,6 +57,22 @@ def test_gelu_every_finite_bf16_input(K):
     got = host_bits(q.gelu(dev_bf16(X)))
     exact = assert_gelu_within_one_ulp(got, oracle.gelu(X))
     assert exact > 0.99                                        # almost everywhere it IS the correctly rounded value
+
+
+def test_gelu_results_are_fixed_bit_for_bit():
+    """The quantized codes behind the GELU follow from its every bit, so its results are fixed over all 65536 inputs: the correctly rounded
+    value except at 18 normal inputs, one ulp off; the far tail flushes to a zero of x's sign; NaN and infinities give NaN."""
+    bits = np.arange(65536, dtype=np.uint32).astype(np.uint16)
+    got = host_bits(q.gelu(dev_bf16(bits.reshape(64, 1024)))).reshape(-1)
+    finite = ((bits >> 7) & 0xFF) != 0xFF
+    assert np.all(got[~finite] == 0x7FFF)
+    assert np.all(got[finite & (bits > 0xC153)] == 0x8000)                          # x <= -13.25
+    assert got[0] == 0 and got[0x8000] == 0
+    want = oracle.gelu(bits.reshape(64, 1024)).reshape(-1)
+    off = np.flatnonzero(finite & (got != want) & (np.abs(bf16_value(want).astype(np.float64)) >= 2.0 ** -120))
+    assert [int(b) for b in off] == [0x3B49, 0x3B4A, 0x3B8F, 0x3BF8, 0x3D18, 0x3DCE, 0xBB49, 0xBB4A, 0xBB8F, 0xBBF8, 0xBD18, 0xBDCE, 0xBEA0, 0xBEAC,
+                                     0xC049, 0xC0CB, 0xC0F4, 0xC11D]
+    assert hashlib.sha256(got.tobytes()).hexdigest() == "6eeba686042080e2e6fd7f87c00f9ec00db7374a1f362a9a961506d650ccd114"
 
 
 @pytest.mark.parametrize("K,M", [(4096, 1374), (1024, 257), (4096, 5), (1024, 1)])
