@@ -288,7 +288,10 @@ constexpr int TMEM_COLS = GACC * GN;                              // 512
 static_assert(DYN_SMEM <= 232448, "exceeds the 227 KB of shared memory a CTA may use");
 static_assert(GSTAGE % 1024 == 0, "operand tiles must stay 1024-byte aligned");
 
-template <bool DUMP>
+// WIDE: the scales are read 16 bytes at a time (a row of them is 32 or 128 bytes).  The caller's pointer need only be aligned to 4
+// bytes; off a 16-byte boundary the other instantiation runs (chosen inside one kernel, the second form of the loads cost the
+// aligned call 1.1 %: 817.5 -> 826.3 us for an MLP of 43 968 rows).
+template <bool DUMP, bool WIDE>
 __global__ void __launch_bounds__(GTHREADS, 1)
 gemm_c8_grouped_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
                        const __grid_constant__ CUtensorMap map_y, const float *__restrict__ a_scale,
@@ -360,9 +363,13 @@ gemm_c8_grouped_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
 #pragma unroll
             for (int j = 0; j < 16; ++j) sum2[j] = 0;
             // The row's scales come from L2, four groups per load, one load ahead (fetched one by one they set the pace: the latency
-            // of one load per K-block).
-            const float4 *as_row = reinterpret_cast<const float4 *>(a_scale + (long long)(row_ok ? gm : 0) * KB);
-            float4 as_next = __ldg(as_row);
+            // of one load per K-block).  Without WIDE the four groups are four loads, still one step ahead.
+            const float *as_row = a_scale + (long long)(row_ok ? gm : 0) * KB;
+            auto four_scales = [&](int kb) {
+                const float *p = as_row + kb;
+                return WIDE ? __ldg(reinterpret_cast<const float4 *>(p)) : make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
+            };
+            float4 as_next = four_scales(0);
             auto wait_full = [&](int p) {      // every warp polls for itself: no warp waits for a slower one between K-blocks
                 const bool ok = alive && ptx::mbar_wait(bar_tfull + 8 * (p % GPAIRS), (p / GPAIRS) & 1, s_abort, status, QVGGT_DEV_TIMEOUT_ACCUM, 20);
                 alive = __all_sync(0xFFFFFFFFu, ok);
@@ -384,7 +391,7 @@ gemm_c8_grouped_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
 #pragma unroll 1
             for (int kb = 0; kb < KB; kb += 4) {
                 const float as4[4] = {as_next.x, as_next.y, as_next.z, as_next.w};
-                if (kb + 4 < KB) as_next = __ldg(as_row + kb / 4 + 1);
+                if (kb + 4 < KB) as_next = four_scales(kb + 4);
 #pragma unroll
                 for (int g = 0; g < 4; ++g) {
                     if (!alive) continue;
@@ -490,13 +497,13 @@ gemm_c8_grouped_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_c
     }
 }
 
-template <bool DUMP>
+template <bool DUMP, bool WIDE>
 cudaError_t launch(const qvggt_weights *w, const signed char *Xq8, const float *a_scale, int M, void *Y, long long ldy,
                    int *acc_debug, cudaStream_t st)
 {
     static QvggtPerDevice cache;
     int max_workers = 0;
-    cudaError_t e = qvggt_configure_kernel(gemm_c8_grouped_kernel<DUMP>, GTHREADS, DYN_SMEM, 2, cache, &max_workers);
+    cudaError_t e = qvggt_configure_kernel(gemm_c8_grouped_kernel<DUMP, WIDE>, GTHREADS, DYN_SMEM, 2, cache, &max_workers);
     if (e != cudaSuccess) return e;
     const int K = w->K, N = w->N;
     CUtensorMap map_x, map_w, map_y;
@@ -518,7 +525,7 @@ cudaError_t launch(const qvggt_weights *w, const signed char *Xq8, const float *
     cfg.stream = st;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, gemm_c8_grouped_kernel<DUMP>, map_x, map_w, map_y, a_scale, (const float *)w->w_scale,
+    return cudaLaunchKernelEx(&cfg, gemm_c8_grouped_kernel<DUMP, WIDE>, map_x, map_w, map_y, a_scale, (const float *)w->w_scale,
                               (const uint16_t *)w->bias, acc_debug, M, N, K, w->status);
 }
 
@@ -652,5 +659,7 @@ cudaError_t qvggt_launch_gemm_c8_grouped(const qvggt_weights *w, const signed ch
     if (M == 0) return cudaSuccess;
     if (!w->Wq8 || w->bits != 4) return cudaErrorNotSupported;
     if (!acc_debug && qvggt_gemm_small_wins(w, M, false, true)) return qvggt_launch_gemm_small(w, Xq8, w->Wq8, false, a_scale, true, M, Y, ldy, st);
-    return acc_debug ? grp::launch<true>(w, Xq8, a_scale, M, Y, ldy, acc_debug, st) : grp::launch<false>(w, Xq8, a_scale, M, Y, ldy, acc_debug, st);
+    if (acc_debug) return grp::launch<true, false>(w, Xq8, a_scale, M, Y, ldy, acc_debug, st);
+    return (reinterpret_cast<uintptr_t>(a_scale) & 15u) == 0 ? grp::launch<false, true>(w, Xq8, a_scale, M, Y, ldy, acc_debug, st)
+                                                            : grp::launch<false, false>(w, Xq8, a_scale, M, Y, ldy, acc_debug, st);
 }

@@ -94,3 +94,28 @@ def test_weights_prepared_just_before():
         for (h, y), w in zip(got, want):
             assert torch.equal(y.view(torch.int16), w.view(torch.int16))
             h.free()
+
+
+# M on both sides of the few-rows line; an offset of 4 floats is a 16-byte boundary again
+@pytest.mark.parametrize("off", [1, 2, 3, 4])
+@pytest.mark.parametrize("K,N,M", [(1024, 1024, 384), (1024, 1024, 385), (4096, 1024, 192), (4096, 1024, 193)])
+def test_group_scales_on_any_float_boundary(K, N, M, off):
+    """Scales that are a contiguous view into a larger buffer need only be aligned to 4 bytes, whatever M: quantizing into such a view
+    and multiplying from it gives the bits of aligned scales, and nothing beside the view is written."""
+    g = torch.Generator(device="cuda").manual_seed(K + M)
+    W, x = (torch.randn(N, K, generator=g, device="cuda") * 0.02).bfloat16(), torch.randn(M, K, generator=g, device="cuda").bfloat16()
+    h = q.prepare_weights(W, None, torch.rand(K, generator=g, device="cuda") + 0.5, None, c8=True)
+    G = K // 128
+    buf = torch.full((M * G + 8,), 7.0, device="cuda")
+    a = buf[off:off + M * G].view(M, G)
+    assert a.is_contiguous() and a.data_ptr() % 16 == 4 * off % 16
+    xq, aligned = q.rotate_smooth_quantize_c8_grouped(h, x)
+    xq2, a2 = q.rotate_smooth_quantize_c8_grouped(h, x, None, a)
+    assert a2 is a and torch.equal(xq, xq2) and torch.equal(a, aligned)
+    assert torch.all(buf[:off] == 7) and torch.all(buf[off + M * G:] == 7)
+    want = q.w4a4_linear_c8_grouped(h, xq, aligned)
+    assert torch.equal(q.w4a4_linear_c8_grouped(h, xq, a).view(torch.int16), want.view(torch.int16))
+    packed, _ = q.rotate_smooth_quantize(h, x, 128)
+    assert torch.equal(q.w4a4_linear(h, packed, a, 128).view(torch.int16), want.view(torch.int16))
+    assert h.device_status() == 0
+    h.free()
