@@ -18,12 +18,19 @@ int device_is_sm100()
     return major == 10;
 }
 
-// The handle's device work is complete and its device is current.
-void release(qvggt_weights *w)
+// The handle's device is current.  `idle`: no device work uses the handle's memory any more.  Where that is not known (a
+// synchronisation that failed, as under a stream capture), the memory is not kept for the next handle.
+void release(qvggt_weights *w, bool idle)
 {
     if (!w) return;
-    qvggt_block_release(w->device, w->codes, w->codes_bytes);
-    qvggt_block_release(w->device, w->small, w->small_bytes);
+    if (idle) {
+        qvggt_block_release(w->device, w->codes, w->codes_bytes);
+        qvggt_block_release(w->device, w->small, w->small_bytes);
+    } else {
+        cudaFree(w->codes);
+        cudaFree(w->small);
+        cudaGetLastError();
+    }
     delete w;
 }
 
@@ -70,7 +77,7 @@ int qvggt_prepare_weights(const void *W_bf16, const void *bias_bf16, const float
     if (qvggt_block_acquire(w->device, codes, &w->codes, &w->codes_bytes) != cudaSuccess ||
         qvggt_block_acquire(w->device, small, &w->small, &w->small_bytes) != cudaSuccess) {
         cudaGetLastError();
-        release(w);
+        release(w, true);                    // nothing was launched
         return QVGGT_ERR_NOMEM;
     }
     unsigned char *wide = static_cast<unsigned char *>(w->codes), *base = static_cast<unsigned char *>(w->small);
@@ -91,8 +98,7 @@ int qvggt_prepare_weights(const void *W_bf16, const void *bias_bf16, const float
         if (e == cudaSuccess) e = qvggt_launch_rsq_static_c8(W_bf16, K, N, K, wmul, w->bits, wmul + K, w->Wq8, w->w_scale, st);
     }
     if (e != cudaSuccess) {
-        cudaStreamSynchronize(st);
-        release(w);
+        release(w, cudaStreamSynchronize(st) == cudaSuccess);
         return QVGGT_ERR_CUDA;
     }
     *out = w;
@@ -367,8 +373,7 @@ void qvggt_free_weights(qvggt_weights_t *w)
     cudaGetDevice(&cur);
     const int owner = w->device;
     if (cur != owner) cudaSetDevice(owner);
-    cudaDeviceSynchronize();
-    release(w);
+    release(w, cudaDeviceSynchronize() == cudaSuccess);
     if (cur != owner) cudaSetDevice(cur);
 }
 

@@ -4,8 +4,8 @@
 // unmap memory and may synchronise the device): a handle of six separate allocations took 0.9 - 8 ms to prepare and 0.6 - 12 ms to
 // free, 20 to 100 times the work on the GPU.  A freed block is therefore kept for the next handle of a similar size: at most
 // kMaxBytes and kMaxBlocks per device, the rest goes back to the driver at once, and all of it does when an allocation fails.
-// A block comes here only after the device was synchronised (qvggt_free_weights), so whoever takes it next may use it on
-// any stream.  One mutex serves all threads; nothing is kept by the address or the contents of a caller's buffer.
+// A block comes here only after the device was synchronised without an error (qvggt_free_weights), so whoever takes it next may use
+// it on any stream.  One mutex serves all threads; nothing is kept by the address or the contents of a caller's buffer.
 #include <mutex>
 
 #include "qvggt_internal.cuh"

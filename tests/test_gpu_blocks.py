@@ -1,5 +1,6 @@
 """Device memory of the weight handles: a freed handle's blocks may serve the next one.  Contents never leak from one handle into the
 next, threads and streams do not disturb each other, and what is kept is bounded."""
+import ctypes
 import threading
 
 import numpy as np
@@ -79,3 +80,49 @@ def test_what_is_kept_is_bounded():
         h.free()
     # at most 64 MB of freed blocks stay with the library (and the allocator's own granules)
     assert free0 - torch.cuda.mem_get_info()[0] <= (64 << 20) + (4 << 20)
+
+
+class _Capture:
+    """A capture of a stream of its own, begun and ended through the runtime API (torch keeps no state about it)."""
+
+    def __init__(self, mode):
+        self.rt, self.mode, self.stream = ctypes.CDLL("libcudart.so.12"), mode, ctypes.c_void_p()
+
+    def __enter__(self):
+        assert self.rt.cudaStreamCreate(ctypes.byref(self.stream)) == 0
+        assert self.rt.cudaStreamBeginCapture(self.stream, self.mode) == 0
+        return self
+
+    def __exit__(self, *exc):
+        graph = ctypes.c_void_p()
+        self.ended = self.rt.cudaStreamEndCapture(self.stream, ctypes.byref(graph))
+        if graph.value:
+            self.rt.cudaGraphDestroy(graph)
+        self.rt.cudaStreamDestroy(self.stream)
+        self.rt.cudaGetLastError()
+
+
+def _addresses(h):
+    p, s = ctypes.c_void_p(), ctypes.c_void_p()
+    assert q.lib().qvggt_weights_view_c8(h.handle, ctypes.byref(p), None) == 0
+    assert q.lib().qvggt_weights_view(h.handle, None, ctypes.byref(s), None, None, None, None) == 0
+    return p.value, s.value
+
+
+def test_memory_freed_without_a_synchronisation_is_not_handed_on():
+    """While a stream is captured the device cannot be synchronised, so work that was queued before may still read a handle that is
+    freed then: its memory must not become the next handle's.  (Global capture mode refuses cudaFree as well: the address cannot
+    come back from the driver either.)"""
+    W, b, c, ref, bias = _layer(1024, 640, 90)
+    q.prepare_weights(W, b, c, None, c8="only").free()           # what is kept, freed in the ordinary way
+    h = q.prepare_weights(W, b, c, None, c8="only")
+    codes, scales = _addresses(h)
+    torch.cuda.synchronize()
+    with _Capture(0):
+        h.free()
+    others = [q.prepare_weights(W, b, c, None, c8="only") for _ in range(3)]
+    for o in others:
+        assert _addresses(o)[0] != codes and _addresses(o)[1] != scales
+        _check(o, ref, bias, "only")
+    for o in others:
+        o.free()
