@@ -1,3 +1,4 @@
+import gc
 import os
 import sys
 
@@ -24,3 +25,10 @@ def pytest_collection_modifyitems(config, items):
     for item in items:
         if "gpu" in item.keywords:
             item.add_marker(skip)
+
+
+def pytest_runtest_setup(item):
+    # the readings of allocated memory in this file must not move because garbage of earlier tests (tensors held by the traceback
+    # of an expected exception) happens to be collected between two of them
+    if item.path.name == "test_zz_no_alloc.py":
+        gc.collect()
