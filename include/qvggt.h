@@ -79,7 +79,8 @@ typedef enum {
  *             QVGGT_PREP_W8A8 for 8-bit codes (see the *_c8 entry points)
  *   out       receives a new handle (device memory is allocated here, on the current device);
  *             release it with qvggt_free_weights.  The handle is bound to that device.
- * Work is enqueued on the stream; the inputs may be released once the stream has passed this call.
+ * Work is enqueued on the stream; the inputs may be released once the stream has passed this call.  A stream that is being
+ * captured is refused with QVGGT_ERR_NOMEM: a handle owns memory, which a graph cannot.
  */
 int qvggt_prepare_weights(const void *W_bf16, const void *bias_bf16, const float *smooth_c,
                           const signed char *sign_v, int N, int K, int flags, void *cuda_stream,

@@ -55,6 +55,13 @@ int qvggt_prepare_weights(const void *W_bf16, const void *bias_bf16, const float
     if (!aligned16(W_bf16)) return QVGGT_ERR_ALIGN;
     if (!device_is_sm100()) return QVGGT_ERR_UNSUPPORTED;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+    // A capture can hold no allocation: refused here, and not only when no kept memory happens to fit (the recorded launches would
+    // write a handle whose memory may by then belong to another).
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &capture) != cudaSuccess || capture != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return QVGGT_ERR_NOMEM;
+    }
 
     qvggt_weights *w = new (std::nothrow) qvggt_weights();
     if (!w) return QVGGT_ERR_NOMEM;

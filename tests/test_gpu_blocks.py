@@ -126,3 +126,24 @@ def test_memory_freed_without_a_synchronisation_is_not_handed_on():
         _check(o, ref, bias, "only")
     for o in others:
         o.free()
+
+
+@pytest.mark.parametrize("mode", [0, 1, 2], ids=["global", "thread_local", "relaxed"])
+@pytest.mark.parametrize("kept", [True, False])
+def test_preparing_on_a_captured_stream_is_refused(mode, kept):
+    """Whether or not kept memory would fit."""
+    W, b, c, ref, bias = _layer(1024, 768, 91)
+    first = q.prepare_weights(W, b, c, None, c8=True)
+    if kept:
+        first.free()
+    torch.cuda.synchronize()
+    with _Capture(mode) as cap, torch.cuda.stream(torch.cuda.ExternalStream(cap.stream.value)):
+        with pytest.raises(q.QvggtError) as e:
+            q.prepare_weights(W, b, c, None, c8=True)
+        status = e.value.status
+        del e
+    assert status == -7 and cap.ended == 0
+    h = q.prepare_weights(W, b, c, None, c8=True)
+    _check(h, ref, bias, True)
+    h.free()
+    first.free()
