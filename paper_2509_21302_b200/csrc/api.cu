@@ -23,14 +23,8 @@ int device_is_sm100()
 void release(qvggt_weights *w, bool idle)
 {
     if (!w) return;
-    if (idle) {
-        qvggt_block_release(w->device, w->codes, w->codes_bytes);
-        qvggt_block_release(w->device, w->small, w->small_bytes);
-    } else {
-        cudaFree(w->codes);
-        cudaFree(w->small);
-        cudaGetLastError();
-    }
+    qvggt_block_release(w->device, w->codes, idle);
+    qvggt_block_release(w->device, w->small, idle);
     delete w;
 }
 
@@ -69,7 +63,6 @@ int qvggt_prepare_weights(const void *W_bf16, const void *bias_bf16, const float
     w->K = K;
     w->bits = w8 ? 8 : 4;
     w->device = qvggt_current_device();
-    w->codes = w->small = nullptr;
     // each array on a 256-byte boundary of its block
     auto place = [](size_t &total, size_t bytes) {
         const size_t at = total;
@@ -81,13 +74,12 @@ int qvggt_prepare_weights(const void *W_bf16, const void *bias_bf16, const float
     const size_t at_scale = place(small, sizeof(float) * N), at_amul = place(small, sizeof(float) * K),
                  at_bias = place(small, bias_bf16 ? sizeof(uint16_t) * N : 0), at_status = place(small, sizeof(int)),
                  at_wmul = place(small, sizeof(float) * (K + 4));    // scratch: [K] multipliers, then one float for the tensor-wise step size
-    if (qvggt_block_acquire(w->device, codes, &w->codes, &w->codes_bytes) != cudaSuccess ||
-        qvggt_block_acquire(w->device, small, &w->small, &w->small_bytes) != cudaSuccess) {
+    if (qvggt_block_acquire(w->device, codes, &w->codes) != cudaSuccess || qvggt_block_acquire(w->device, small, &w->small) != cudaSuccess) {
         cudaGetLastError();
         release(w, true);                    // nothing was launched
         return QVGGT_ERR_NOMEM;
     }
-    unsigned char *wide = static_cast<unsigned char *>(w->codes), *base = static_cast<unsigned char *>(w->small);
+    unsigned char *wide = static_cast<unsigned char *>(w->codes.p), *base = static_cast<unsigned char *>(w->small.p);
     w->Wq = packed ? wide + at_wq : nullptr;
     w->Wq8 = c8 ? reinterpret_cast<signed char *>(wide + at_wq8) : nullptr;
     w->w_scale = reinterpret_cast<float *>(base + at_scale);

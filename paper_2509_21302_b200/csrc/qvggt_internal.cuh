@@ -5,6 +5,13 @@
 
 #include "../../include/qvggt.h"
 
+// Device memory of a handle as device_blocks.cu gave it.
+struct QvggtBlock {
+    void *p = nullptr;
+    size_t bytes = 0;                  // as allocated
+    unsigned long long context = 0;    // the CUDA context that it was allocated in (a device reset makes a new one); 0: not known
+};
+
 struct qvggt_weights {
     int N, K;
     int device;
@@ -15,8 +22,7 @@ struct qvggt_weights {
     float *amul;         // [K]
     uint16_t *bias;      // [N] bf16 bits, or nullptr
     int *status;         // device status word (0 = ok)
-    void *codes, *small; // the two device blocks that these lie in: Wq and Wq8; the rest
-    size_t codes_bytes, small_bytes;   // their sizes as allocated
+    QvggtBlock codes, small;   // the two device blocks that these lie in: Wq and Wq8; the rest
 };
 
 // Device status codes written by kernels whose bounded waits expire.
@@ -30,10 +36,10 @@ enum : int {
     QVGGT_DEV_TIMEOUT_PACKED_FREE = 6 // TMA producer gave up waiting for a packed stage to be released
 };
 
-// device_blocks.cu: device memory of the handles, kept for the next handle within a bound.  A block that is released must have
-// no work in flight that uses it.
-cudaError_t qvggt_block_acquire(int device, size_t bytes, void **block, size_t *block_bytes);
-void qvggt_block_release(int device, void *block, size_t block_bytes);
+// device_blocks.cu: device memory of the handles, kept for the next handle within a bound; the device is the current one.  A block
+// of which it is not known that no work in flight uses it (`idle` false) is given back to the driver.
+cudaError_t qvggt_block_acquire(int device, size_t bytes, QvggtBlock *block);
+void qvggt_block_release(int device, const QvggtBlock &block, bool idle);
 
 // rsq.cu
 // multipliers; also copies the bias and clears the status word, if given

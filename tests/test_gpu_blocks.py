@@ -1,6 +1,9 @@
 """Device memory of the weight handles: a freed handle's blocks may serve the next one.  Contents never leak from one handle into the
 next, threads and streams do not disturb each other, and what is kept is bounded."""
 import ctypes
+import os
+import subprocess
+import sys
 import threading
 
 import numpy as np
@@ -147,3 +150,44 @@ def test_preparing_on_a_captured_stream_is_refused(mode, kept):
     _check(h, ref, bias, True)
     h.free()
     first.free()
+
+
+_RESET = r"""
+import ctypes, sys
+import numpy as np
+L, rt = ctypes.CDLL(sys.argv[1]), ctypes.CDLL("libcudart.so.12")
+vp = ctypes.c_void_p
+L.qvggt_prepare_weights.argtypes = [vp, vp, vp, vp, ctypes.c_int, ctypes.c_int, ctypes.c_int, vp, ctypes.POINTER(vp)]
+L.qvggt_free_weights.argtypes = [vp]
+L.qvggt_free_weights.restype = None
+N, K = 128, 1024
+
+def device(a):
+    p = vp()
+    assert rt.cudaMalloc(ctypes.byref(p), ctypes.c_size_t(a.nbytes)) == 0
+    assert rt.cudaMemcpy(p, a.ctypes.data_as(vp), ctypes.c_size_t(a.nbytes), 1) == 0
+    return p
+
+def prepare():
+    W, c = device(np.full((N, K), 0x3F80, np.uint16)), device(np.ones(K, np.float32))
+    h = vp()
+    st = L.qvggt_prepare_weights(W, None, c, None, N, K, 1, None, ctypes.byref(h))
+    print(st, rt.cudaDeviceSynchronize())
+    return h
+
+a, b = prepare(), prepare()
+L.qvggt_free_weights(a)                  # its memory is kept
+assert rt.cudaDeviceReset() == 0
+c = prepare()                            # must not get that memory
+L.qvggt_free_weights(b)                  # of the context that is gone
+d = prepare()
+"""
+
+
+def test_kept_memory_is_not_used_after_a_device_reset():
+    """In a process of its own.  Whatever the runtime answers to launches after a reset, no launch touches memory of the old context."""
+    from paper_2509_21302_b200 import buildlib
+    r = subprocess.run([sys.executable, "-c", _RESET, buildlib.LIB], capture_output=True, text=True, timeout=120, cwd=os.path.dirname(buildlib.LIB))
+    assert r.returncode == 0, r.stdout + r.stderr
+    lines = [tuple(int(v) for v in x.split()) for x in r.stdout.split("\n") if x]
+    assert lines[:2] == [(0, 0)] * 2 and len(lines) == 4 and all(st in (0, -5) and sync == 0 for st, sync in lines[2:]), lines
