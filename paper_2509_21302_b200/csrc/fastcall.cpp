@@ -287,7 +287,7 @@ PyObject *linear_c8(PyObject *, PyObject *const *args, Py_ssize_t n)
     const int64_t N = in.integer(), K = in.integer();
     const Tensor &xq = in.at_least(at::kChar, 0);
     if (!in.ok || xq.dim() != 2 || xq.size(1) != K) Py_RETURN_NONE;
-    const Tensor &as = in.at_least(at::kFloat, xq.size(0) * (GROUPED ? K / 128 : 1));
+    const Tensor &as = GROUPED ? in.exact(at::kFloat, xq.size(0), K / 128) : in.at_least(at::kFloat, xq.size(0));
     return linear(in, xq, as, N, [&](const void *q, const float *a, int M, void *y, int64_t ldy, void *st) {
         return FN(h, static_cast<const S8 *>(q), a, M, y, ldy, nullptr, st);
     });

@@ -123,3 +123,16 @@ def test_preparation_calls_give_the_same_and_refuse_the_same(monkeypatch):
     with pytest.raises(q.QvggtError) as e:
         q.prepare_weights(W[:100], None, fast[0])
     assert e.value.status == -2
+
+
+def test_group_scales_of_another_shape_are_refused():
+    """[M, K/128] and nothing else that holds as many values: transposed scales or those of a larger batch give no result."""
+    K, N, M = 1024, 128, 5
+    h, hp, g = _handles(K, N)
+    x = torch.randn(M, K, generator=g, device="cuda").bfloat16()
+    xq, a = q.rotate_smooth_quantize_c8_grouped(h, x)
+    for bad in (a.t().contiguous(), a.reshape(-1), a.reshape(1, M, K // 128), torch.cat([a, a]), torch.cat([a, a], 1)):
+        with pytest.raises(AssertionError):
+            q.w4a4_linear_c8_grouped(h, xq, bad)
+    for keep in (a, a.clone()):
+        q.w4a4_linear_c8_grouped(h, xq, keep)
