@@ -13,6 +13,7 @@
 #include <ATen/ops/empty.h>
 #include <ATen/ops/from_blob.h>
 #include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 
 #include "../../include/qvggt.h"
@@ -356,19 +357,30 @@ PyObject *prepare_weights(PyObject *, PyObject *const *args, Py_ssize_t n)
     QVGGT_GUARD_END
 }
 
-// Copy of a device array as a new tensor on the current device (d1 < 0: one dimension), None for a null pointer.
-PyObject *copy_array(const void *p, ScalarType type, int64_t d0, int64_t d1)
+// Copy of a device array as a new tensor on the current device (d1 < 0: one dimension), undefined for a null pointer.  The array lies
+// on the device of its handle, which need not be the current one.
+Tensor copy_array(const void *p, ScalarType type, int64_t d0, int64_t d1)
 {
-    if (!p) Py_RETURN_NONE;
-    const auto options = at::TensorOptions().dtype(type).device(at::kCUDA, c10::cuda::getCurrentCUDAStream().device_index());
+    if (!p) return Tensor();
+    const auto options = at::TensorOptions().dtype(type).device(at::kCUDA);
     void *q = const_cast<void *>(p);
-    return THPVariable_Wrap((d1 < 0 ? at::from_blob(q, {d0}, options) : at::from_blob(q, {d0, d1}, options)).clone());
+    const Tensor t = d1 < 0 ? at::from_blob(q, {d0}, options) : at::from_blob(q, {d0, d1}, options);
+    const at::Device here(at::kCUDA, c10::cuda::getCurrentCUDAStream().device_index());
+    return t.device() == here ? t.clone() : t.to(here);
 }
+
+PyObject *wrap_or_none(const Tensor &t)
+{
+    if (!t.defined()) Py_RETURN_NONE;
+    return THPVariable_Wrap(t);
+}
+
+// The two views have no other route: what goes wrong in them (out of memory, say) is raised as it is.
 
 // (handle) -> copies (wq, w_scale, amul, bias), None where the handle has no such array
 PyObject *weights_view(PyObject *, PyObject *const *args, Py_ssize_t n)
 {
-    QVGGT_GUARD_BEGIN
+    HANDLE_TH_ERRORS
     Args in{args, n};
     auto *h = in.handle();
     const U8 *wq = nullptr;
@@ -376,23 +388,25 @@ PyObject *weights_view(PyObject *, PyObject *const *args, Py_ssize_t n)
     const void *bias = nullptr;
     int N = 0, K = 0;
     if (!in.done() || qvggt_weights_view(h, &wq, &ws, &am, &bias, &N, &K) != QVGGT_OK) Py_RETURN_NONE;
-    return release_items(PyTuple_Pack(4, copy_array(wq, at::kByte, N, K / 2), copy_array(ws, at::kFloat, N, -1), copy_array(am, at::kFloat, K, -1),
-                                      copy_array(bias, at::kBFloat16, N, -1)));
-    QVGGT_GUARD_END
+    const Tensor a = copy_array(wq, at::kByte, N, K / 2), b = copy_array(ws, at::kFloat, N, -1), c = copy_array(am, at::kFloat, K, -1),
+                 d = copy_array(bias, at::kBFloat16, N, -1);
+    return release_items(PyTuple_Pack(4, wrap_or_none(a), wrap_or_none(b), wrap_or_none(c), wrap_or_none(d)));
+    END_HANDLE_TH_ERRORS
 }
 
 // (handle, N, K) -> (copy of the codes one per byte or None, code width)
 PyObject *weights_view_c8(PyObject *, PyObject *const *args, Py_ssize_t n)
 {
-    QVGGT_GUARD_BEGIN
+    HANDLE_TH_ERRORS
     Args in{args, n};
     auto *h = in.handle();
     const int64_t N = in.integer(), K = in.integer();
     const S8 *wq8 = nullptr;
     int bits = 0;
     if (!in.done() || qvggt_weights_view_c8(h, &wq8, &bits) != QVGGT_OK) Py_RETURN_NONE;
-    return release_items(PyTuple_Pack(2, copy_array(wq8, at::kChar, N, K), PyLong_FromLong(bits)));
-    QVGGT_GUARD_END
+    const Tensor codes = copy_array(wq8, at::kChar, N, K);
+    return release_items(PyTuple_Pack(2, wrap_or_none(codes), PyLong_FromLong(bits)));
+    END_HANDLE_TH_ERRORS
 }
 
 #define FAST(name, fn) {name, reinterpret_cast<PyCFunction>(reinterpret_cast<void (*)()>(static_cast<PyObject *(*)(PyObject *, PyObject *const *, Py_ssize_t)>(fn))), METH_FASTCALL, nullptr}

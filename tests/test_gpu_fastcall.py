@@ -136,3 +136,30 @@ def test_group_scales_of_another_shape_are_refused():
             q.w4a4_linear_c8_grouped(h, xq, bad)
     for keep in (a, a.clone()):
         q.w4a4_linear_c8_grouped(h, xq, keep)
+
+
+def test_a_view_that_cannot_be_copied_says_why():
+    """Out of memory is out of memory, not a status of the library."""
+    h, hp, g = _handles(1024, 4096)
+    torch.cuda.empty_cache()
+    total, used = torch.cuda.get_device_properties(0).total_memory, torch.cuda.memory_reserved()
+    torch.cuda.set_per_process_memory_fraction(used / total)
+    try:
+        for view in (h.view, h.view_c8):
+            with pytest.raises(torch.cuda.OutOfMemoryError):
+                view()
+    finally:
+        torch.cuda.set_per_process_memory_fraction(1.0)
+    assert h.view()["wq"].shape == (4096, 512) and h.view_c8().shape == (4096, 1024)
+
+
+@pytest.mark.skipif(torch.cuda.device_count() < 2, reason="needs two devices")
+def test_a_handle_of_another_device_can_be_viewed():
+    h, hp, g = _handles(1024, 128)
+    want, codes = h.view(), h.view_c8()
+    torch.cuda.synchronize()
+    with torch.cuda.device(1):
+        got, other = h.view(), h.view_c8()
+        for k, v in got.items():
+            assert v.device.index == 1 and torch.equal(v.cpu(), want[k].cpu())
+        assert other.device.index == 1 and torch.equal(other.cpu(), codes.cpu())
