@@ -94,13 +94,15 @@ int64_t pitch(const Tensor &t) { return t.size(0) > 1 ? t.stride(0) : t.size(1);
 
 void *stream() { return c10::cuda::getCurrentCUDAStream().stream(); }
 
+// f() touches no tensor and no Python object: a tensor's data_ptr() may throw, or call back into Python.
 template <class F>
 int without_gil(F f)
 {
-    PyThreadState *s = PyEval_SaveThread();
-    const int st = f();
-    PyEval_RestoreThread(s);
-    return st;
+    struct Released {
+        PyThreadState *s = PyEval_SaveThread();
+        ~Released() { PyEval_RestoreThread(s); }
+    } released;
+    return f();
 }
 
 PyObject *wrap(const Tensor &given, const Tensor &made, PyObject *obj)
@@ -130,7 +132,8 @@ PyObject *quantize(Args &in, const Tensor &X, ScalarType code, int64_t row_codes
     void *q = (xq.defined() ? xq : made_q).data_ptr();
     float *a = static_cast<float *>((as.defined() ? as : made_a).data_ptr());
     void *st = stream();
-    if (without_gil([&] { return f(x, pitch(X), (int)M, q, a, st); }) != QVGGT_OK) Py_RETURN_NONE;
+    const int64_t ldx = pitch(X);
+    if (without_gil([&] { return f(x, ldx, (int)M, q, a, st); }) != QVGGT_OK) Py_RETURN_NONE;
     return PyTuple_Pack(2, wrap(xq, made_q, oq), wrap(as, made_a, oa));
 }
 
@@ -158,7 +161,8 @@ PyObject *linear(Args &in, const Tensor &xq, const Tensor &as, int64_t N, F f)
     const void *q = xq.data_ptr();
     const float *a = static_cast<const float *>(as.data_ptr());
     void *out = Y.data_ptr(), *st = stream();
-    if (without_gil([&] { return f(q, a, (int)M, out, pitch(Y), st); }) != QVGGT_OK) Py_RETURN_NONE;
+    const int64_t ldy = pitch(Y);
+    if (without_gil([&] { return f(q, a, (int)M, out, ldy, st); }) != QVGGT_OK) Py_RETURN_NONE;
     return wrap(y, made, oy);
 }
 
@@ -221,9 +225,10 @@ PyObject *rotate_smooth_quantize_static_c8(PyObject *, PyObject *const *args, Py
     const int64_t K = in.integer();
     const Tensor &X = in.rows(K);
     const Tensor &delta = in.at_least(at::kFloat, 1);
-    if (in.ok && delta.numel() != 1) in.ok = false;
+    if (!in.ok || delta.numel() != 1) Py_RETURN_NONE;
+    const auto *d = static_cast<const float *>(delta.data_ptr());
     return release_items(quantize(in, X, at::kChar, K, -1, [&](const void *x, int64_t ldx, int M, void *q, float *a, void *st) {
-        return qvggt_rotate_smooth_quantize_static_c8(h, x, ldx, M, static_cast<const float *>(delta.data_ptr()), static_cast<S8 *>(q), a, st);
+        return qvggt_rotate_smooth_quantize_static_c8(h, x, ldx, M, d, static_cast<S8 *>(q), a, st);
     }));
     QVGGT_GUARD_END
 }
@@ -238,9 +243,10 @@ PyObject *layernorm_rotate_smooth_quantize_c8(PyObject *, PyObject *const *args,
     const Tensor &X = in.rows(K);
     const Tensor &gamma = in.exact(at::kFloat, K, -1), &beta = in.exact(at::kFloat, K, -1);
     const float eps = (float)in.real();
+    if (!in.ok) Py_RETURN_NONE;
+    const auto *gp = static_cast<const float *>(gamma.data_ptr()), *bp = static_cast<const float *>(beta.data_ptr());
     return release_items(quantize(in, X, at::kChar, K, -1, [&](const void *x, int64_t ldx, int M, void *q, float *a, void *st) {
-        return qvggt_layernorm_rotate_smooth_quantize_c8(h, x, ldx, M, static_cast<const float *>(gamma.data_ptr()), static_cast<const float *>(beta.data_ptr()),
-                                                         eps, static_cast<S8 *>(q), a, st);
+        return qvggt_layernorm_rotate_smooth_quantize_c8(h, x, ldx, M, gp, bp, eps, static_cast<S8 *>(q), a, st);
     }));
     QVGGT_GUARD_END
 }
@@ -254,8 +260,10 @@ PyObject *rotate_smooth_quantize_c8_expand(PyObject *, PyObject *const *args, Py
     const int64_t N = in.integer(), K = in.integer();
     const Tensor &X = in.rows(K);
     const Tensor &scratch = in.at_least(at::kChar, N * K);
+    if (!in.ok) Py_RETURN_NONE;
+    S8 *w = static_cast<S8 *>(scratch.data_ptr());
     return release_items(quantize(in, X, at::kChar, K, -1, [&](const void *x, int64_t ldx, int M, void *q, float *a, void *st) {
-        return qvggt_rotate_smooth_quantize_c8_expand(h, x, ldx, M, static_cast<S8 *>(q), a, static_cast<S8 *>(scratch.data_ptr()), st);
+        return qvggt_rotate_smooth_quantize_c8_expand(h, x, ldx, M, static_cast<S8 *>(q), a, w, st);
     }));
     QVGGT_GUARD_END
 }
@@ -307,8 +315,9 @@ PyObject *linear_scratch(PyObject *, PyObject *const *args, Py_ssize_t n)
     if (!in.ok || xq.dim() != 2 || xq.size(1) != K) Py_RETURN_NONE;
     const Tensor &as = in.at_least(at::kFloat, xq.size(0));
     const Tensor &scratch = in.at_least(at::kChar, N * K);
+    if (!in.ok) Py_RETURN_NONE;
+    S8 *w = static_cast<S8 *>(scratch.data_ptr());
     return linear(in, xq, as, N, [&](const void *q, const float *a, int M, void *y, int64_t ldy, void *st) {
-        S8 *w = static_cast<S8 *>(scratch.data_ptr());
         return EXPANDED ? qvggt_w4a4_linear_c8_expanded(h, static_cast<const S8 *>(q), a, M, y, ldy, w, nullptr, st)
                         : qvggt_w4a4_linear_c8_packed_weights(h, static_cast<const S8 *>(q), a, M, y, ldy, w, nullptr, st);
     });
@@ -330,7 +339,8 @@ PyObject *calibrate_smooth(PyObject *, PyObject *const *args, Py_ssize_t n)
     const void *x = X.data_ptr(), *w = W.data_ptr();
     float *s = static_cast<float *>(scratch.data_ptr()), *out = static_cast<float *>(c.data_ptr());
     void *st = stream();
-    if (without_gil([&] { return qvggt_calibrate_smooth(x, (int)X.size(0), w, (int)W.size(0), (int)K, alpha, lo, hi, s, out, st); }) != QVGGT_OK) Py_RETURN_NONE;
+    const int Mc = (int)X.size(0), N = (int)W.size(0);
+    if (without_gil([&] { return qvggt_calibrate_smooth(x, Mc, w, N, (int)K, alpha, lo, hi, s, out, st); }) != QVGGT_OK) Py_RETURN_NONE;
     return THPVariable_Wrap(c);
     QVGGT_GUARD_END
 }

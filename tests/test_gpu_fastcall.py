@@ -163,3 +163,24 @@ def test_a_handle_of_another_device_can_be_viewed():
         for k, v in got.items():
             assert v.device.index == 1 and torch.equal(v.cpu(), want[k].cpu())
         assert other.device.index == 1 and torch.equal(other.cpu(), codes.cpu())
+
+
+def test_a_tensor_without_memory_of_its_own_is_refused():
+    """A tensor whose address cannot be asked for (one inside vmap) among real ones, in every place: an exception, and no harm to the
+    interpreter."""
+    K, N, M = 1024, 128, 3
+    h, hp, g = _handles(K, N)
+    x = torch.randn(M, K, generator=g, device="cuda").bfloat16()
+    gamma, beta = torch.rand(K, generator=g, device="cuda"), torch.rand(K, generator=g, device="cuda")
+    xq, a = q.rotate_smooth_quantize_c8(h, x)
+    scratch, delta = torch.empty(N * K, dtype=torch.int8, device="cuda"), torch.tensor([0.2], device="cuda")
+    for f, t in ((lambda v: q.rotate_smooth_quantize_c8(h, v), x), (lambda v: q.layernorm_rotate_smooth_quantize_c8(h, x, v, beta), gamma),
+                 (lambda v: q.layernorm_rotate_smooth_quantize_c8(h, x, gamma, v), beta), (lambda v: q.rotate_smooth_quantize_static_c8(h, x, v), delta),
+                 (lambda v: q.rotate_smooth_quantize_c8_expand(hp, x, v), scratch), (lambda v: q.w4a4_linear_c8(h, v, a), xq),
+                 (lambda v: q.w4a4_linear_c8(h, xq, v), a), (lambda v: q.w4a4_linear_c8_packed_weights(hp, xq, a, v), scratch),
+                 (lambda v: q.w4a4_linear_c8_expanded(hp, xq, a, v), scratch), (lambda v: q.calibrate_smooth(x, v), x),
+                 (lambda v: q.prepare_weights(x.repeat(128, 1)[:128], None, v), gamma)):
+        with pytest.raises(Exception):
+            torch.func.vmap(f)(torch.stack([t, t]))
+    want = q.w4a4_linear_c8(h, xq, a)
+    assert torch.equal(want, q.w4a4_linear_c8(h, xq, a)) and h.device_status() == 0
