@@ -6,11 +6,21 @@ import os
 import subprocess
 import sysconfig
 
+import torch
+
 _HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(_HERE, "csrc")
 LIB = os.path.join(_HERE, "libqvggt.so")
-FASTCALL = os.path.join(_HERE, "_qvggt_fastcall.so")
+
 INCLUDE = os.path.join(os.path.dirname(_HERE), "include")
+
+
+def fastcall_path(torch_version: str = torch.__version__) -> str:
+    """The extension module is bound to one Python and one torch: both are in its name, so that another one builds its own."""
+    return os.path.join(_HERE, f"_qvggt_fastcall.{sysconfig.get_config_var('SOABI')}.torch-{torch_version}.so")
+
+
+FASTCALL = fastcall_path()
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -50,8 +60,6 @@ def build(force: bool = False, verbose: bool = False) -> str:
         os.replace(tmp, LIB)
     src = os.path.join(CSRC, "fastcall.cpp")
     if force or _stale(FASTCALL, [src] + _headers()):
-        import torch
-
         root = os.path.dirname(torch.__file__)
         tmp = FASTCALL + f".tmp{os.getpid()}"
         subprocess.check_call(

@@ -58,3 +58,15 @@ def test_no_oracle_or_cpu_fallback_in_the_product_path():
             if f.endswith((".py", ".cu", ".cuh", ".h")):
                 text = open(os.path.join(dirpath, f)).read()
                 assert "oracle" not in text.lower().replace("no cpu fallback", ""), f
+
+
+def test_the_extension_module_is_bound_to_this_python_and_torch(monkeypatch):
+    """A module built for another torch is not taken for this one's, however new its file is."""
+    import sysconfig
+    import torch
+    from paper_2509_21302_b200 import buildlib
+    q.build()
+    assert torch.__version__ in buildlib.FASTCALL and sysconfig.get_config_var("SOABI") in buildlib.FASTCALL
+    assert not buildlib.is_stale()
+    monkeypatch.setattr(buildlib, "FASTCALL", buildlib.fastcall_path("0.0.0"))
+    assert buildlib.is_stale()
