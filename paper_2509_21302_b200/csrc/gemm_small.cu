@@ -179,19 +179,23 @@ cudaError_t dispatch(const qvggt_weights *w, const void *Xq, const void *Wq, con
 }  // namespace
 
 // Where the lines lie: this kernel's time grows with M N K (its rate is that of mma.sync), the persistent kernels' hardly moves
-// below one round of tiles.  Measured (us, this kernel / the other one):
-//   one code per byte   K = 1024: N = 3072, M = 64 4.9 / 4.6, M = 128 6.3 / 4.7; N = 1024, M = 192 4.1 / 4.6; N = 4096, M = 32 4.3 / 4.9
-//                       K = 4096: N = 1024, M = 128 7.3 / 8.2, M = 192 10.2 / 8.2
-//   packed              K = 1024: N = 3072, M = 256 7.1 / 8.2; N = 4096, M = 192 7.2 / 8.2, M = 256 9.3 / 8.2
-//                       K = 4096: N = 1024, M = 256 8.9 / 16.7, M = 512 15.9 / 16.7
-//   group scales        K = 1024: N = 3072, M = 128 6.6 / 6.6, M = 192 8.1 / 6.6; N = 4096, M = 96 6.6 / 6.8; N = 1024, M = 256 4.3 / 6.5
-//                       K = 4096: N = 1024, M = 192 13.3 / 15.1, M = 256 17.3 / 15.1
-// and at 5 rows           K = 1024, N = 3072 2.3 / 4.5, packed 2.0 / 7.8, groups 2.4 / 6.3; K = 4096 2.5 / 8.0, 2.2 / 16.4, 3.1 / 14.8
+// below one round of tiles.  What decides is the layer, the quantize launch and the GEMM behind it: the persistent kernels hide more of
+// their start behind the quantize launch, so alone and back to back this kernel would win for longer than it does in a layer.
+// Layers in a replayed graph (us, this kernel / the other one), each line between the first and the second M:
+//   one code per byte   K = 1024: N = 128, M = 1536 6.8 / 7.1, M = 3072 9.9 / 7.7; N = 1024, M = 192 6.1 / 5.9, M = 257 6.8 / 5.9;
+//                                 N = 3072, M = 64 5.6 / 5.9, M = 85 6.8 / 5.9; N = 4096, M = 48 5.7 / 5.9, M = 96 7.8 / 6.3
+//                       K = 4096: N = 128, M = 512 10.0 / 12.0, M = 1024 16.7 / 12.9; N = 640, M = 153 10.4 / 10.4, M = 204 13.2 / 10.4;
+//                                 N = 1024, M = 96 9.7 / 10.6, M = 128 11.7 / 11.0; N = 4096, M = 24 9.4 / 11.4, M = 32 11.0 / 10.3
+//   packed              K = 1024: N = 128, M = 6144 12.6 / 13.5, M = 8232 15.6 / 15.1; N = 3072, M = 256 9.1 / 9.3, M = 343 11.2 / 9.6
+//                       K = 4096: N = 1024, M = 384 17.8 / 19.5, M = 514 21.4 / 21.6; N = 4096, M = 96 16.2 / 19.9, M = 128 20.3 / 18.8
+//   group scales        K = 1024: N = 1024, M = 384 8.5 / 9.0, M = 514 9.6 / 8.9; N = 4096, M = 96 8.2 / 8.2, M = 128 9.1 / 8.3
+//                       K = 4096: N = 128, M = 1152 19.4 / 21.5, M = 1536 24.2 / 22.8; N = 1024, M = 144 15.6 / 17.7, M = 192 19.4 / 17.5
+// and the GEMM alone at 5 rows   K = 1024, N = 3072 2.3 / 4.5, packed 2.0 / 7.8, groups 2.4 / 6.3; K = 4096 2.5 / 8.0, 2.2 / 16.4, 3.1 / 14.8
 bool qvggt_gemm_small_wins(const qvggt_weights *w, int M, bool packed, bool grouped)
 {
     const long long outputs = (long long)M * w->N;
     if (w->K == 1024) return outputs <= (packed ? 3LL << 18 : grouped ? 3LL << 17 : 3LL << 16);
-    return outputs <= (packed ? 3LL << 17 : grouped ? 3LL << 16 : 1LL << 17);
+    return outputs <= (packed ? 3LL << 17 : grouped ? 9LL << 14 : 3LL << 15);
 }
 
 cudaError_t qvggt_launch_gemm_small(const qvggt_weights *w, const void *Xq, const void *Wq, bool packed, const float *a_scale, bool grouped, int M,

@@ -58,7 +58,8 @@ def test_row_tiles(K, N, M):
 
 
 # M on the last size of the kernel and the first of the other one, for each of the rule's lines
-@pytest.mark.parametrize("K,N,lines", [(1024, 1024, (192, 384, 768)), (1024, 3072, (64, 128, 256)), (4096, 1024, (128, 192, 384))])
+@pytest.mark.parametrize("K,N,lines", [(1024, 1024, (192, 384, 768)), (1024, 3072, (64, 128, 256)), (4096, 1024, (96, 128, 144, 192, 384)),
+                                         (4096, 512, (192, 288, 768))])
 def test_both_sides_of_the_rule(K, N, lines):
     for line in lines:
         for M in (line, line + 1):
@@ -98,7 +99,7 @@ def test_weights_prepared_just_before():
 
 # M on both sides of the few-rows line; an offset of 4 floats is a 16-byte boundary again
 @pytest.mark.parametrize("off", [1, 2, 3, 4])
-@pytest.mark.parametrize("K,N,M", [(1024, 1024, 384), (1024, 1024, 385), (4096, 1024, 192), (4096, 1024, 193)])
+@pytest.mark.parametrize("K,N,M", [(1024, 1024, 384), (1024, 1024, 385), (4096, 1024, 144), (4096, 1024, 145), (4096, 1024, 193)])
 def test_group_scales_on_any_float_boundary(K, N, M, off):
     """Scales that are a contiguous view into a larger buffer need only be aligned to 4 bytes, whatever M: quantizing into such a view
     and multiplying from it gives the bits of aligned scales, and nothing beside the view is written."""
