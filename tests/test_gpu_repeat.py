@@ -107,3 +107,33 @@ def test_two_streams_share_a_handle(q):
             assert torch.equal(y4.view(torch.int16), want[i][0].view(torch.int16))
     assert h.device_status() == 0
     h.free()
+
+
+# 3 and 4 tiles per pair of CTAs on 74 pairs: 96 and 128 K-blocks per worker, on either side of the limit of 100 up to which the packed
+# GEMM starts under the tail of the kernel in front of it
+@pytest.mark.parametrize("M", [74 * 3 * 256, 74 * 3 * 256 + 1])
+def test_packed_gemm_on_both_sides_of_its_launch_rule(q, M):
+    """Quantize and multiply in turn, each launch writing what the next one reads, without a wait in between: the packed route gives the
+    bits of the one-code-per-byte route."""
+    K, N = 4096, 128
+    g = torch.Generator(device="cuda").manual_seed(M)
+    W = (torch.randn(N, K, generator=g, device="cuda") * 0.02).bfloat16()
+    h = q.prepare_weights(W, None, torch.rand(K, generator=g, device="cuda") + 0.5, None, c8=True)
+    x = torch.randn(M, K, generator=g, device="cuda").bfloat16()
+    xq, a, y = torch.empty(M, K // 2, dtype=torch.uint8, device="cuda"), torch.empty(M, device="cuda"), torch.empty(M, N, dtype=torch.bfloat16, device="cuda")
+    want, got = [], []
+    for i in range(3):
+        xi = x.roll(i, 0)
+        want.append(q.w4a4_linear_c8(h, *q.rotate_smooth_quantize_c8(h, xi)))
+        torch.cuda.synchronize()
+    for i in range(3):
+        xi = x.roll(i, 0)
+        q.rotate_smooth_quantize(h, xi, 0, xq, a)
+        q.w4a4_linear(h, xq, a, 0, y)
+        got.append(y.clone())
+    for u, v in zip(got, want):
+        assert torch.equal(u.view(torch.int16), v.view(torch.int16))
+    assert h.device_status() == 0
+    h.free()
+    del x, want, got
+    torch.cuda.empty_cache()
