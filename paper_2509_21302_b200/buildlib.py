@@ -11,7 +11,6 @@ import torch
 _HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(_HERE, "csrc")
 LIB = os.path.join(_HERE, "libqvggt.so")
-
 INCLUDE = os.path.join(os.path.dirname(_HERE), "include")
 
 

@@ -5,8 +5,8 @@
 // from the tensors to the C entry points directly (2.7 us a call in all).
 //
 // A function returns what its namesake in binding.py returns, or None when an argument is not plainly what the call expects or
-// the library returned a status: binding.py then takes its own path, which checks, converts and reports.  Nothing
-// here keeps state.
+// the library returned a status: binding.py then takes its own path, which checks, converts and reports.  (The two views of a handle
+// have no other path and raise.)  Nothing here keeps state.
 #include <Python.h>
 
 #include <ATen/core/Tensor.h>
@@ -52,7 +52,7 @@ struct Args {
         if (PyErr_Occurred()) { PyErr_Clear(); ok = false; }
         return v;
     }
-    // A tensor on the current device, or an undefined one for None where `optional`.
+    // A CUDA tensor (which device it is on is the caller's affair, as on the other route), or an undefined one for None where `optional`.
     const Tensor &tensor(bool optional = false)
     {
         static const Tensor none;

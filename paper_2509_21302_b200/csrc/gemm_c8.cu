@@ -282,8 +282,7 @@ constexpr int OFF_BAR = OFF_CH + GEPI * 64 * 4;                 // full[GSTAGES]
 constexpr int NBARS = 2 * GSTAGES + 2 * GPAIRS;
 constexpr int OFF_TMEM = OFF_BAR + NBARS * 8;
 constexpr int OFF_ABORT = OFF_TMEM + 4;
-constexpr int OFF_FLAGS = OFF_ABORT + 4;
-constexpr int DYN_SMEM = OFF_FLAGS + 8 + 1024;
+constexpr int DYN_SMEM = OFF_ABORT + 4 + 1024;                    // slack to align the base to 1024 bytes
 constexpr int TMEM_COLS = GACC * GN;                              // 512
 static_assert(DYN_SMEM <= 232448, "exceeds the 227 KB of shared memory a CTA may use");
 static_assert(GSTAGE % 1024 == 0, "operand tiles must stay 1024-byte aligned");

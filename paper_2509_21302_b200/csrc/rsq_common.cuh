@@ -34,14 +34,6 @@ __device__ __forceinline__ float tree_sum(const float (&a)[N])
     }
 }
 
-// The same tree over the squares of N of the T registers, starting at O.
-template <int N, int O = 0, int T>
-__device__ __forceinline__ float tree_sum_squares(const float (&a)[T])
-{
-    if constexpr (N == 1) return __fmul_rn(a[O], a[O]);
-    else return __fadd_rn(tree_sum_squares<N / 2, O>(a), tree_sum_squares<N / 2, O + N / 2>(a));
-}
-
 // GELU x Phi(x) (the activation between the two linears of the MLP: the producer of fc2's input) of two bf16 values, rounded to
 // bf16, evaluated so that the negative tail keeps its RELATIVE accuracy.  With t = |x|, z = t / sqrt(2):
 //   Q(t) = 1 - Phi(t) = exp(-z^2) E(z) / 2,   E(z) = exp(z^2) erfc(z)  (smooth, from 1 down to ~1 / (z sqrt(pi))),
@@ -50,7 +42,10 @@ __device__ __forceinline__ float tree_sum_squares(const float (&a)[T])
 // At most one bf16 ulp wherever the result is a normal number above 2^-120; below that (x < -12.9) the exponential flushes to
 // zero, with the sign of x.  NaN stays NaN, and an infinite x gives NaN (the product of infinity and a flushed tail).
 // Everything but the two special-function operations of an element (reciprocal, exp2) runs on two elements per instruction; each of
-// these operations rounds exactly like its scalar form, and no product feeds an addition that is not written as a fused one.
+// these operations rounds exactly like its scalar form, and no product feeds an addition that is not written as a fused one.  The fused
+// kernel is bound by instruction issue and, through the four special-function operations of a pair, by that unit; scalar / paired, us back
+// to back: K = 1024 15.9 / 15.3 at 10 992 rows, 158 / 154 at 137 400; K = 4096 62.2 / 59.9, 714 / 678.  (A polynomial for log2 Q, with the
+// exponential alone on the special-function unit, took 14.4, 145, 54.1, 624, but gave other bits.)
 __device__ __forceinline__ uint32_t gelu_bf16x2(uint32_t x)
 {
     const uint32_t a = x | 0x80008000u;                    // -t
