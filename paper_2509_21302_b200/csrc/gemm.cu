@@ -288,13 +288,13 @@ cudaError_t launch(const qvggt_weights *w, const unsigned char *Xq, const float 
         return cudaErrorInvalidValue;
     const int total_tiles = ((M + BM * CG - 1) / (BM * CG)) * ((N + BN - 1) / BN);
     const int workers = total_tiles < max_workers ? total_tiles : max_workers;
-    // Launched programmatically (its start-up under the tail of the kernel in front) up to 100 K-blocks per worker.  A quantize +
-    // GEMM pair called from Python, us, programmatic / plain: K = 1024, N = 1024: 10.6 / 12.5 at 512 rows (8 K-blocks per
-    // worker), 26.1 / 28.8 at 10 992 (24), N = 3072: 67.2 / 67.7 at 16 488 (88), K = 4096, N = 1024: 84.5 / 84.5 at 10 992 (96); beyond,
-    // K = 1024, N = 4096: 84.7 / 84.2 at 16 488 (120), 112.2 / 110.7 at 21 984 (152), 219.8 / 215.1 at 43 968 (304).  The GEMM
-    // back to back with itself gains 1 - 2 us from it up to those sizes too, so the cost must fall on the quantize launch that it
-    // overlaps (not traced further).
-    const bool programmatic = (long long)((total_tiles + workers - 1) / workers) * (K / BK) <= 100;
+    // Launched programmatically (its start-up under the tail of the kernel in front) up to 64 K-blocks per worker.  A layer as a program
+    // calls it, quantize + GEMM on inputs beyond L2, us, programmatic / plain: K = 1024, N = 1024: 12.1 / 14.4 at 2731 rows (8 K-blocks
+    // per worker), N = 4096: 34.9 / 35.9 at 5496 (40), 50.9 / 51.1 at 8244 (64); K = 4096, N = 1024: 62.5 / 63.6 at 8244 (64), N = 4096:
+    // 42.0 / 43.0 at 1374 (64).  Beyond: K = 1024, N = 4096: 63.9 / 63.6 at 10 992 (80), K = 4096, N = 1024: 84.4 / 84.4 at 10 992 (96),
+    // N = 4096: 62.9 / 61.7 at 3300 (96), 79.3 / 78.0 at 4122 (128).  The GEMM back to back with itself gains 1 - 2 us from it at every
+    // size, so what it costs must fall on the quantize launch that it overlaps (not traced further).
+    const bool programmatic = (long long)((total_tiles + workers - 1) / workers) * (K / BK) <= 64;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(workers * CG);
     cfg.blockDim = dim3(THREADS);

@@ -109,9 +109,9 @@ def test_two_streams_share_a_handle(q):
     h.free()
 
 
-# 3 and 4 tiles per pair of CTAs on 74 pairs: 96 and 128 K-blocks per worker, on either side of the limit of 100 up to which the packed
-# GEMM starts under the tail of the kernel in front of it
-@pytest.mark.parametrize("M", [74 * 3 * 256, 74 * 3 * 256 + 1])
+# 2 and 3 tiles per pair of CTAs on 74 pairs: 64 and 96 K-blocks per worker, the last size at which the packed GEMM starts under the tail of
+# the kernel in front of it and the first at which it does not
+@pytest.mark.parametrize("M", [74 * 2 * 256, 74 * 2 * 256 + 1])
 def test_packed_gemm_on_both_sides_of_its_launch_rule(q, M):
     """Quantize and multiply in turn, each launch writing what the next one reads, without a wait in between: the packed route gives the
     bits of the one-code-per-byte route."""
