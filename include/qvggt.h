@@ -266,7 +266,8 @@ int qvggt_gelu_rotate_smooth_quantize_c8(const qvggt_weights_t *w, const void *X
                                          signed char *Xq8, float *a_scale, void *cuda_stream);
 int qvggt_gelu(const void *X_bf16, long long ldx, int M, int K, void *Y_bf16, void *cuda_stream);
 
-/* Frees the handle and its device memory (synchronises the device first).  NULL is allowed. */
+/* Frees the handle and its device memory (synchronises the device first).  At most 64 MB per device stay with the library for
+ * the next handle; they go back to the driver when an allocation of the library fails.  NULL is allowed. */
 void qvggt_free_weights(qvggt_weights_t *w);
 
 /*
