@@ -7,18 +7,29 @@
 // stages by TMA and nothing in this kernel touches an operand byte with an ordinary instruction.  Per K-block
 // a CTA's shared memory sees one TMA write and one tensor-core read of its 32 KB of operands, the minimum.
 //
-// Persistent and warp-specialised; a worker is a pair of CTAs on neighbouring SMs (tile 256 tokens x BN = 256 or 128
-// channels, each CTA stages 128 token rows and BN / 2 weight rows; one thread of the leader CTA issues
-// tcgen05.mma.cta_group::2.kind::i8 for both; accumulators int32 in tensor memory, two buffers of BN columns).
-//   warps 0..7   epilogue: TMEM -> registers -> scale, bias, bf16 -> swizzled staging -> whole-line stores; no warp waits for another
+// Persistent and warp-specialised; a worker is a pair of CTAs on neighbouring SMs (tile 256 tokens x up to 256 channels, each CTA stages
+// 128 token rows and half of the tile's weight rows; one thread of the leader CTA issues tcgen05.mma.cta_group::2.kind::i8 for both;
+// accumulators int32 in tensor memory, two buffers of 256 columns).
+//   warps 0..7   epilogue: TMEM -> registers -> scale, bias, bf16 -> swizzled staging -> TMA stores; no warp waits for another
 //   warp  8      one elected thread issues tcgen05.mma and the commits that release stages / publish accumulators
 //   warp  9      one thread per CTA issues the TMA loads of its half of every operand stage; both CTAs signal
 //                the leader's "full" barrier (cta_group::2 form of the load)
-// The tiles are dealt round-robin to the workers.
+// What bounds it, and what follows from it (us back to back; the earlier form took A and B of every tile from L2, read the channel
+// parameters from shared memory for every 16 rows and wrote 128-byte lines with ordinary stores):
+//  - At 256 channels the MMAs of a K-block take 512 cycles and its 32 KB per CTA take as long from L2 (64 bytes per cycle and SM), so with
+//    K = 1024, where a tile's outputs are another 8 KB per K-block, the traffic of the SM was the limit.  With K = 1024 the eight
+//    K-blocks of the token rows (128 KB) stay in shared memory for RUN consecutive tiles and only weights stream.
+//  - The epilogue shares the shared-memory pipe with the operands: parameters in registers, outputs through the TMA engine.
+//  - The outputs are marked first to leave L2 (default policy: 35.1 instead of 31.9 at N = 4096).
+//  - Tiles that do not fill a round of workers are cut into narrower ones (make_plan()).
+//   K = 1024, N = 3072 / 1024 / 4096 and K = 4096, N = 1024 at 10 992 rows: 27.4 / 13.0 / 36.8 / 32.8 -> 24.8 / 11.3 / 31.9 / 29.9;
+//   at 137 400 rows K = 1024, N = 4096: 432 -> 394 (at the power limit).
 // Every wait is bounded; on expiry the kernel records a code in *status and all roles fall through to the
 // common exit, where tensor memory is released.
 #include <cuda.h>
 #include <cuda_bf16.h>
+
+#include <type_traits>
 
 #include "gemm_common.cuh"
 #include "qvggt_internal.cuh"
@@ -33,110 +44,181 @@ using gemmc::STG_BYTES;
 
 constexpr int BM = 128;            // token rows per CTA (TMEM lanes)
 constexpr int BK = 128;            // codes along K per stage = one 128-byte swizzled row
+constexpr int UNIT = 64;           // channels per unit of work; a tile is 256 token rows x 1 .. 4 units
+constexpr int MAX_UNITS = 4;
 constexpr int ACC_BUFS = 2;        // TMEM accumulators: the epilogue of tile i overlaps the MMAs of tile i+1
-constexpr int EPI_WARPS = 8;       // warp w: TMEM lane quarter w % 4, column part w / 4
+constexpr int ACC_COLS = MAX_UNITS * UNIT;
+constexpr int EPI_WARPS = 8;       // warp w: TMEM lane quarter w % 4, part w / 4 of the tile
 constexpr int MMA_WARP = EPI_WARPS;
 constexpr int TMA_WARP = EPI_WARPS + 1;
 constexpr int THREADS = (EPI_WARPS + 2) * 32;
+constexpr int TMEM_COLS = ACC_BUFS * ACC_COLS;
 
-// BN = output channels per tile: 256, or 128 where that keeps more of the chip busy (see wide_tiles()).
-template <int BN>
-struct Lay {
-    static constexpr int B_ROWS = BN / 2;                         // weight rows staged by one CTA
-    static constexpr int STAGE = (BM + B_ROWS) * BK;              // 32 / 24 KB
-    static constexpr int STAGES = BN == 256 ? 6 : 8;
-    static constexpr int OFF_STG = STAGES * STAGE;                // operand stages first: they need 1024-byte alignment
-    static constexpr int OFF_CH = OFF_STG + EPI_WARPS * STG_BYTES;          // per warp: scales and biases of its BN / 2 channels, fp32
-    static constexpr int OFF_BAR = OFF_CH + EPI_WARPS * BN * 4;             // full[STAGES] empty[STAGES] tfull[2] tempty[2]
-    static constexpr int NBARS = 2 * STAGES + 2 * ACC_BUFS;
-    static constexpr int OFF_TMEM = OFF_BAR + NBARS * 8;
-    static constexpr int OFF_ABORT = OFF_TMEM + 4;
-    static constexpr int SMEM_BYTES = OFF_ABORT + 4;
-    static constexpr int DYN_SMEM = SMEM_BYTES + 1024;            // slack to align the base to 1024 bytes
-    static constexpr int TMEM_COLS = ACC_BUFS * BN;               // 512 / 256
-    static_assert(DYN_SMEM <= 232448, "exceeds the 227 KB of shared memory a CTA may use");
-    static_assert(2 * STAGE < (1 << 20), "transaction count of a stage must fit the barrier");
-    static_assert(STAGE % 1024 == 0, "operand tiles must stay 1024-byte aligned");
+constexpr int A_BYTES = BM * BK;                       // one K-block of a CTA's token rows: 16 KB
+constexpr int UNIT_BYTES = UNIT / 2 * BK;              // one K-block of a CTA's half of a unit's weight rows: 4 KB
+constexpr int RES_KB = 8;                              // K-blocks of the token rows that stay resident (K = 1024)
+constexpr int RUN = 4;                                 // consecutive tiles of a worker that share them, see make_plan()
+constexpr int STG_WARP = 16 * 2 * UNIT;                // staging of one epilogue warp: 16 rows x 64 bf16, 128-byte swizzled
+constexpr int OFF_OPS = EPI_WARPS * STG_WARP;          // operands: [resident token rows,] ring of stages (1024-byte aligned)
+constexpr int OPS_BYTES = 208 * 1024;
+constexpr int MAX_STAGES = 12;
+constexpr int OFF_BAR = OFF_OPS + OPS_BYTES;           // full[MAX_STAGES] empty[MAX_STAGES] tfull[2] tempty[2]
+constexpr int NBARS = 2 * MAX_STAGES + 2 * ACC_BUFS;
+constexpr int OFF_TMEM = OFF_BAR + NBARS * 8;
+constexpr int OFF_ABORT = OFF_TMEM + 4;
+constexpr int DYN_SMEM = OFF_ABORT + 4 + 1024;         // slack to align the base to 1024 bytes
+static_assert(DYN_SMEM <= 232448, "exceeds the 227 KB of shared memory a CTA may use");
+static_assert(2 * (A_BYTES + MAX_UNITS * UNIT_BYTES) < (1 << 20), "transaction count of a stage must fit the barrier");
+
+// How the tiles are dealt to the workers; filled in by make_plan(), so that no thread of the kernel divides.  Work is counted in units of 256
+// token rows x 64 channels; whole tiles are numbered along the channels, row tile by row tile.
+struct Plan {
+    int NU, NT;                  // units and whole tiles of a row tile: NT tiles of `narrow` units, the first `wider` of them one unit more
+    int narrow, wider, wide;     // wide: most units of a whole tile
+    int runs, run;               // each worker first takes `runs` times `run` consecutive tiles,
+    int rounds;                  // then so many single tiles,
+    int cut;                     // then at most one piece of `cut` units
+    int workers, row_tiles;
+    int behind_row, behind_unit, behind_first, behind_pieces;   // where the pieces begin, how many the begun row tile has, how many a row tile has
+    unsigned long long div_nt, div_pieces;                      // see div()
+    int stages, stage_bytes;
+    // x / d for x d < 2^40, with m = ceil(2^40 / d)
+    static __host__ __device__ unsigned long long reciprocal(int d) { return ((1ull << 40) + d - 1) / d; }
+    static __host__ __device__ __forceinline__ int div(int x, unsigned long long m) { return (int)((x * m) >> 40); }
 };
 
+// The tiles of one worker, in order.
+struct Tiles {
+    int row, unit, units;                                 // the current tile: row tile, first unit, how many units
+    int count;                                            // of tiles
+    __device__ __forceinline__ Tiles(const Plan &plan, int worker_) : row(0), unit(0), units(0), worker(worker_), t(0), p(plan)
+    {
+        // behind the whole tiles: what is left of a row tile, then whole row tiles
+        const int i = worker - p.behind_first, full = i < 0 ? 0 : Plan::div(i, p.div_pieces);
+        behind_row = p.behind_row + (i < 0 ? 0 : 1 + full);
+        behind_unit = i < 0 ? p.behind_unit + worker * p.cut : (i - full * p.behind_pieces) * p.cut;
+        count = p.runs * p.run + p.rounds + (behind_row < p.row_tiles ? 1 : 0);
+        at = worker * p.run;
+        in_run = 0;
+        next();
+    }
+    __device__ __forceinline__ void next()     // (one beyond the last is never used)
+    {
+        const int in_runs = p.runs * p.run;
+        if (t < in_runs + p.rounds) {
+            if (t >= in_runs) at = in_runs * p.workers + (t - in_runs) * p.workers + worker;
+            row = Plan::div(at, p.div_nt);
+            const int j = at - row * p.NT;
+            unit = j * p.narrow + min(j, p.wider);
+            units = p.narrow + (j < p.wider ? 1 : 0);
+            ++at;
+            if (++in_run == p.run) { in_run = 0; at += (p.workers - 1) * p.run; }
+        } else {
+            row = behind_row;
+            unit = behind_unit;
+            units = min(p.cut, p.NU - unit);
+        }
+        ++t;
+    }
+
+private:
+    int worker, t, at, in_run, behind_row, behind_unit;
+    const Plan &p;
+};
+
+// A position in the ring of operand stages together with the parity of the phase it is in.
+struct StageRing {
+    int s = 0;
+    uint32_t ph = 0, stage;
+    __device__ __forceinline__ explicit StageRing(uint32_t ring) : stage(ring) {}
+    __device__ __forceinline__ void advance(const Plan &plan, uint32_t ring)
+    {
+        stage += plan.stage_bytes;
+        if (++s == plan.stages) { s = 0; ph ^= 1; stage = ring; }
+    }
+};
+
+// RESIDENT (K = 1024): all eight K-blocks of a tile's token rows stay in shared memory for as long as the worker's tiles share
+// them, and only weight rows stream.
 // DUMP: also write the int32 sums to acc_debug (its own instantiation keeps that code out of the production kernel).
 // wait_limit: bound of every device-side wait, in cycles.  skip_loads: the TMA producers issue nothing, so that the
 // first wait for operands runs out (used only to exercise the timeout path; no asynchronous operation is in flight).
-template <int BN, bool DUMP>
+template <bool RESIDENT, bool DUMP>
 __global__ void __launch_bounds__(THREADS, 1)
-gemm_c8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w,
-               uint16_t *__restrict__ Y, long long ldy,
-               const float *__restrict__ a_scale, const float *__restrict__ w_scale, const uint16_t *__restrict__ bias,
+gemm_c8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant__ CUtensorMap map_w, const __grid_constant__ CUtensorMap map_wu,
+               const __grid_constant__ CUtensorMap map_y, const __grid_constant__ Plan plan, const float *__restrict__ a_scale, const float *__restrict__ w_scale, const uint16_t *__restrict__ bias,
                int *__restrict__ acc_debug, int M, int N, int K, int *status, long long wait_limit, int skip_loads)
 {
-    using L = Lay<BN>;
-    constexpr int STAGES = L::STAGES, STAGE = L::STAGE, B_ROWS = L::B_ROWS, TMEM_COLS = L::TMEM_COLS;
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const uint32_t sbase = ptx::smem_addr(smem);
-    const uint32_t bar_full = sbase + L::OFF_BAR;
-    const uint32_t bar_empty = bar_full + STAGES * 8;
-    const uint32_t bar_tfull = bar_empty + STAGES * 8;
+    const uint32_t bar_full = sbase + OFF_BAR;
+    const uint32_t bar_empty = bar_full + MAX_STAGES * 8;
+    const uint32_t bar_tfull = bar_empty + MAX_STAGES * 8;
     const uint32_t bar_tempty = bar_tfull + ACC_BUFS * 8;
-    uint32_t *s_tmem = reinterpret_cast<uint32_t *>(smem + L::OFF_TMEM);
-    volatile int *s_abort = reinterpret_cast<volatile int *>(smem + L::OFF_ABORT);
+    const uint32_t ops = sbase + OFF_OPS, ring = ops + (RESIDENT ? RES_KB * A_BYTES : 0);
+    uint32_t *s_tmem = reinterpret_cast<uint32_t *>(smem + OFF_TMEM);
+    volatile int *s_abort = reinterpret_cast<volatile int *>(smem + OFF_ABORT);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t rank = ptx::cluster_ctarank();                       // 0 = leader of the pair
-    const int worker = blockIdx.x / 2, workers = gridDim.x / 2;
-    const int KB = K / BK;
-    const int n_tiles = (N + BN - 1) / BN;
-    const int total_tiles = ((M + 2 * BM - 1) / (2 * BM)) * n_tiles;
-    const int my_tiles = (total_tiles > worker) ? (total_tiles - 1 - worker) / workers + 1 : 0;
+    const int KB = RESIDENT ? RES_KB : K / BK;
 
-    if (threadIdx.x == 0) {
-        gemmc::init_barriers(bar_full, STAGES, 1);                     // the leader's arrive.expect_tx (bytes of both CTAs)
-        gemmc::init_barriers(bar_empty, STAGES, 1);                    // tcgen05.commit
-        gemmc::init_barriers(bar_tfull, ACC_BUFS, 1);                  // tcgen05.commit
-        gemmc::init_barriers(bar_tempty, ACC_BUFS, EPI_WARPS * 2);     // the epilogue warps of both CTAs
-        *s_abort = 0;
+    // full: the leader's arrive.expect_tx (bytes of both CTAs); empty, tfull: tcgen05.commit; tempty: the epilogue warps of both CTAs
+    if (threadIdx.x < NBARS) {
+        ptx::mbar_init(bar_full + 8 * threadIdx.x, threadIdx.x < NBARS - ACC_BUFS ? 1 : EPI_WARPS * 2);
         ptx::fence_mbar_init();
+        if (threadIdx.x == 0) *s_abort = 0;
     }
     if (warp == MMA_WARP) { ptx::tmem_alloc_pair(ptx::smem_addr(s_tmem), TMEM_COLS); ptx::tmem_relinquish_pair(); }
     if (warp == TMA_WARP && lane == 0) {
         ptx::prefetch_tensormap(&map_x);
         ptx::prefetch_tensormap(&map_w);
+        ptx::prefetch_tensormap(&map_wu);
+        ptx::prefetch_tensormap(&map_y);
     }
+    // Both CTAs meet: the leader's barriers exist before the peer's loads signal them.  The first tile is worked out on the way.
+    __syncwarp();
     ptx::tc_fence_before_sync();
-    __syncthreads();
-    ptx::cluster_sync();                     // the leader's barriers exist before the peer's loads signal them
+    ptx::cluster_arrive();
+    Tiles tile(plan, blockIdx.x / 2);
+    const int my_tiles = tile.count;
+    ptx::cluster_wait();
     ptx::tc_fence_after_sync();
     const uint32_t tmem_base = *s_tmem;
-    // everything above touched only kernel parameters and on-chip state: it may overlap the tail of the previous
-    // kernel in the stream; the operands (and the output buffer) may not be touched before that kernel is done
+    // Everything up to grid_dependency_wait() touches only kernel parameters and on-chip state: it may overlap the tail of the previous
+    // kernel in the stream; the operands and the output buffer may not be touched before that kernel is done.  (The MMA thread touches
+    // neither: it waits for what the producers load.)
     ptx::grid_launch_dependents();
-    ptx::grid_dependency_wait();
 
     if (warp < EPI_WARPS) {
         // ------------------------------------------------------------ epilogue
-        const int quarter = warp & 3, cpart = warp >> 2;   // TMEM lane quarter, column part
-        unsigned char *stg = smem + L::OFF_STG + warp * STG_BYTES;
-        const uint32_t stg_addr = sbase + L::OFF_STG + warp * STG_BYTES;
-        float *wsb = reinterpret_cast<float *>(smem + L::OFF_CH) + warp * BN, *bsb = wsb + BN / 2;     // the warp's channel scales, biases
+        const int quarter = warp & 3, part = warp >> 2;    // TMEM lane quarter; of the units, part 0 takes the first half
+        const uint32_t stg_addr = sbase + warp * STG_WARP;
         const uint32_t leader_tempty = ptx::map_to_cta(bar_tempty, 0);
         const uint64_t one2 = ptx::f32x2_one(N & 127);                       // N is a multiple of 128
+        const uint64_t policy = ptx::policy_evict_first();
         bool alive = true;
-        constexpr int CW = BN / 2, NCH = CW / 64;              // columns and 64-column chunks of one warp's part
-        for (int t = 0; t < my_tiles; ++t) {
-            const int tile = worker + t * workers;
-            const int m0 = (tile / n_tiles) * (2 * BM) + (int)rank * BM + quarter * 32;
-            const int n0 = (tile % n_tiles) * BN + cpart * CW; // first channel of this warp's part
+        ptx::grid_dependency_wait();
+        for (int t = 0; t < my_tiles; ++t, tile.next()) {
+            const int m0 = tile.row * (2 * BM) + (int)rank * BM + quarter * 32;
             const int b = t & 1;
-            const bool cols_ok = n0 < N;                       // N is a multiple of 128: a part is all in or all out
-            // The scales and biases of the warp's channels: each warp keeps its own copy in shared memory, so that no warp ever
-            // waits for another.
-            float my_ws[CW / 32], my_bs[CW / 32];
+            // A tile of one unit is shared by rows: 16 of a warp's 32 each.
+            const bool by_rows = tile.units == 1;
+            const int first = by_rows ? 0 : part * ((tile.units + 1) / 2), units = by_rows ? 1 : part ? tile.units / 2 : (tile.units + 1) / 2;
+            const int n0 = (tile.unit + first) * UNIT;         // first channel of this warp
+            // Scales and biases of channels 8 e + 2 (lane mod 4) and + 1 of each unit, in the layout of the accumulator fragments and
+            // straight into registers: read from shared memory for every 16 rows they took as much of its bandwidth as the outputs.
+            uint64_t w2[2][8];
+            uint32_t c2[2][8];
 #pragma unroll
-            for (int e = 0; e < CW / 32; ++e) {
-                const int n = n0 + 32 * e + lane;
-                my_ws[e] = cols_ok ? __ldg(w_scale + n) : 0.0f;
-                my_bs[e] = (cols_ok && bias) ? __uint_as_float(static_cast<uint32_t>(__ldg(bias + n)) << 16) : 0.0f;
-            }
+            for (int k = 0; k < 2; ++k)
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const int n = n0 + (k < units ? k * UNIT : 0) + 8 * e + 2 * (lane & 3);
+                    w2[k][e] = __ldg(reinterpret_cast<const unsigned long long *>(w_scale + n));
+                    c2[k][e] = bias ? __ldg(reinterpret_cast<const uint32_t *>(bias + n)) : 0u;
+                }
             uint64_t as2[2][2];                                // rows lane / 4 + 8 h of the warp's 16 u .. 16 u + 15
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
@@ -144,72 +226,72 @@ gemm_c8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
                 const float as = gm < M ? __ldg(a_scale + gm) : 0.0f;
                 as2[u >> 1][u & 1] = ptx::f32x2_pack(as, as);
             }
-            __syncwarp();                                      // the previous tile's last reads
-#pragma unroll
-            for (int e = 0; e < CW / 32; ++e) {
-                wsb[32 * e + lane] = my_ws[e];
-                bsb[32 * e + lane] = my_bs[e];
-            }
-            __syncwarp();
             {
                 int ok = 1;
-                if (lane == 0) ok = (alive && ptx::mbar_wait(bar_tfull + 8 * b, (t >> 1) & 1, s_abort, status, QVGGT_DEV_TIMEOUT_ACCUM, 32, wait_limit)) ? 1 : 0;
+                if (lane == 0) ok = (alive && ptx::mbar_wait(bar_tfull + 8 * b, (t >> 1) & 1, s_abort, status, QVGGT_DEV_TIMEOUT_ACCUM, 0, wait_limit)) ? 1 : 0;
                 alive = __shfl_sync(0xFFFFFFFFu, ok, 0) != 0;
             }
             ptx::tc_fence_after_sync();
             if (alive) {
 #pragma unroll
-                for (int c = 0; c < NCH; ++c) {
-                    uint32_t raw[2][32];
+                for (int k = 0; k < 2; ++k) {
+                    if (k < units) {
+                        uint32_t raw[2][32];
 #pragma unroll
-                    for (int u = 0; u < 2; ++u)
-                        ptx::tmem_ld_16x256b_x8(tmem_base + (static_cast<uint32_t>(quarter * 32 + 16 * u) << 16) + b * BN + cpart * CW + c * 64, raw[u]);
-                    ptx::tmem_ld_wait();
-                    if (c == NCH - 1) {                        // tensor memory goes back to the MMA thread
-                        ptx::tc_fence_before_sync();
-                        __syncwarp();
-                        // (nobody waits for the last tiles' arrivals: none may be on its way when the leader CTA exits)
-                        if (lane == 0 && t + ACC_BUFS < my_tiles) ptx::mbar_arrive_cluster(leader_tempty + 8 * b);
-                    }
-                    if (cols_ok) {
+                        for (int u = 0; u < 2; ++u)
+                            ptx::tmem_ld_16x256b_x8(tmem_base + (static_cast<uint32_t>(quarter * 32 + 16 * u) << 16) + b * ACC_COLS + (first + k) * UNIT, raw[u]);
+                        ptx::tmem_ld_wait();
+                        if (k == units - 1) {                  // tensor memory goes back to the MMA thread
+                            ptx::tc_fence_before_sync();
+                            __syncwarp();
+                            // (nobody waits for the last tiles' arrivals: none may be on its way when the leader CTA exits)
+                            if (lane == 0 && t + ACC_BUFS < my_tiles) ptx::mbar_arrive_cluster(leader_tempty + 8 * b);
+                        }
 #pragma unroll
                         for (int u = 0; u < 2; ++u) {
-                            const int m = m0 + 16 * u, n = n0 + 64 * c;
-                            gemmc::finish_16x64(raw[u], as2[u], wsb + 64 * c, bsb + 64 * c, stg, stg_addr, Y + (long long)m * ldy + n, ldy, M - m, lane, one2);
+                            const int m = m0 + 16 * u, n = n0 + k * UNIT;
+                            if (by_rows && u != part) continue;
+                            gemmc::finish_16x64_tma(raw[u], as2[u], w2[k], c2[k], stg_addr, &map_y, n, m, m < M, lane, one2, policy);
                             if (DUMP && acc_debug) gemmc::dump_16x64<0>(acc_debug + (long long)m * N + n, N, raw[u], M - m, lane);
                         }
                     }
                 }
             }
         }
+        if (lane == 0) ptx::tma_store_wait_read<0>();
     } else if (warp == MMA_WARP) {
         // ------------------------------------------------------------ MMA issuer (one thread of the leader CTA)
         // The thread is chosen by elect.sync, not by its lane number: the assembler then knows that one thread is active and keeps
         // the descriptors in uniform registers, where tcgen05 wants them (behind `lane == 0` every one is moved there anew, which
         // made this loop, at 545 cycles per K-block, the bound of the kernel).
         if (rank == 0 && ptx::elect_one()) {
-            constexpr uint32_t idesc = ptx::idesc_i8(2 * BM, BN);
             bool alive = true;
-            Ring r;
-            int left = my_tiles * KB;                                      // K-blocks to come, this one included
-            for (int t = 0; t < my_tiles && alive; ++t) {
+            StageRing r(ring);
+            int left = my_tiles * KB - plan.stages;                        // K-blocks for whose stage a load will wait
+            for (int t = 0; t < my_tiles && alive; ++t, tile.next()) {
                 const int b = t & 1;
                 if (t >= ACC_BUFS) {
                     alive = ptx::mbar_wait_cluster(bar_tempty + 8 * b, ((t >> 1) - 1) & 1, s_abort, status, QVGGT_DEV_TIMEOUT_TMEM_FREE, wait_limit);
                     if (!alive) break;
                     ptx::tc_fence_after_sync();
                 }
-                const uint32_t d_tmem = tmem_base + b * BN;
-                for (int kb = 0; kb < KB; ++kb) {
-                    alive = ptx::mbar_wait_cluster(bar_full + 8 * r.s, r.ph, s_abort, status, QVGGT_DEV_TIMEOUT_FULL, wait_limit);
-                    if (!alive) break;
-                    ptx::tc_fence_after_sync();
-                    const uint32_t a_addr = sbase + r.s * STAGE;
-                    gemmc::mma_kblock_i8<true>(d_tmem, a_addr, a_addr + BM * BK, idesc, kb == 0);
-                    if (left-- > STAGES) ptx::mma_commit_pair(bar_empty + 8 * r.s, 3);   // frees the stage in both CTAs, if a load waits for it
-                    if (kb == KB - 1) ptx::mma_commit_pair(bar_tfull + 8 * b, 3);
-                    r.advance(STAGES);
-                }
+                const uint32_t d_tmem = tmem_base + b * ACC_COLS;
+                auto k_blocks = [&](auto units) {                          // the width is a constant of the instruction descriptor
+                    constexpr uint32_t idesc = ptx::idesc_i8(2 * BM, decltype(units)::value * UNIT);
+                    for (int kb = 0; kb < KB; ++kb) {
+                        alive = ptx::mbar_wait_cluster(bar_full + 8 * r.s, r.ph, s_abort, status, QVGGT_DEV_TIMEOUT_FULL, wait_limit);
+                        if (!alive) break;
+                        ptx::tc_fence_after_sync();
+                        gemmc::mma_kblock_i8<true>(d_tmem, RESIDENT ? ops + kb * A_BYTES : r.stage, RESIDENT ? r.stage : r.stage + A_BYTES, idesc, kb == 0);
+                        if (left-- > 0) ptx::mma_commit_pair(bar_empty + 8 * r.s, 3);   // frees the stage in both CTAs
+                        if (kb == KB - 1) ptx::mma_commit_pair(bar_tfull + 8 * b, 3);
+                        r.advance(plan, ring);
+                    }
+                };
+                if (tile.units == 4) k_blocks(std::integral_constant<int, 4>());
+                else if (tile.units == 3) k_blocks(std::integral_constant<int, 3>());
+                else if (tile.units == 2) k_blocks(std::integral_constant<int, 2>());
+                else k_blocks(std::integral_constant<int, 1>());
             }
         }
         __syncwarp();
@@ -217,25 +299,43 @@ gemm_c8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
         // ------------------------------------------------------------ TMA producer (one thread per CTA)
         if (!skip_loads && ptx::elect_one()) {
             const uint32_t leader_full = ptx::map_to_cta(bar_full, 0);
+            ptx::grid_dependency_wait();
             bool alive = true;
-            Ring r;
-            int it = 0;
-            for (int t = 0; t < my_tiles && alive; ++t) {
-                const int tile = worker + t * workers;
-                const int m0 = (tile / n_tiles) * (2 * BM) + (int)rank * BM;
-                const int n0 = (tile % n_tiles) * BN + (int)rank * B_ROWS;
-                for (int kb = 0; kb < KB; ++kb, ++it) {
-                    if (it >= STAGES) {
-                        alive = ptx::mbar_wait(bar_empty + 8 * r.s, r.ph ^ 1, s_abort, status, QVGGT_DEV_TIMEOUT_EMPTY, 20, wait_limit);
-                        if (!alive) break;
+            StageRing r(ring);
+            int ahead = plan.stages, resident = -1;                        // K-blocks that need not wait for their stage; resident row tile
+            for (int t = 0; t < my_tiles && alive; ++t, tile.next()) {
+                const int m0 = tile.row * (2 * BM) + (int)rank * BM;
+                const int n0 = tile.unit * UNIT + (int)rank * (tile.units * (UNIT / 2));
+                // the box of weight rows may reach beyond a narrower tile: rows that nothing reads
+                auto k_blocks = [&](const CUtensorMap *map, auto rows, int box_units) {
+                    constexpr bool ROWS = decltype(rows)::value;
+                    const uint32_t bytes = 2 * ((ROWS ? A_BYTES : 0) + box_units * UNIT_BYTES);
+                    for (int kb = 0; kb < KB; ++kb) {
+                        if (--ahead < 0) {
+                            alive = ptx::mbar_wait(bar_empty + 8 * r.s, r.ph ^ 1, s_abort, status, QVGGT_DEV_TIMEOUT_EMPTY, 0, wait_limit);
+                            if (!alive) break;
+                        }
+                        const uint32_t full = leader_full + 8 * r.s;
+                        // the leader's barrier expects the bytes of both CTAs; the peer's completions may arrive first
+                        // (the count goes negative for a while), the phase cannot end before the leader has arrived
+                        if (rank == 0) ptx::mbar_arrive_expect_tx(bar_full + 8 * r.s, bytes);
+                        // The K-block of the resident rows that this overwrites was last read RES_KB K-blocks ago, and the MMAs up to
+                        // plan.stages <= RES_KB K-blocks ago are known to be done.
+                        if (ROWS) ptx::tma_load_2d_pair(&map_x, full, RESIDENT ? ops + kb * A_BYTES : r.stage, kb * BK, m0);
+                        ptx::tma_load_2d_pair(map, full, RESIDENT ? r.stage : r.stage + A_BYTES, kb * BK, n0);
+                        r.advance(plan, ring);
                     }
-                    const uint32_t dst = sbase + r.s * STAGE;
-                    // the leader's barrier expects the bytes of both CTAs; the peer's completions may arrive first
-                    // (the count goes negative for a while), the phase cannot end before the leader has arrived
-                    if (rank == 0) ptx::mbar_arrive_expect_tx(bar_full + 8 * r.s, 2 * STAGE);
-                    ptx::tma_load_2d_pair(&map_x, leader_full + 8 * r.s, dst, kb * BK, m0);
-                    ptx::tma_load_2d_pair(&map_w, leader_full + 8 * r.s, dst + BM * BK, kb * BK, n0);
-                    r.advance(STAGES);
+                };
+                const std::true_type yes;
+                const std::false_type no;
+                const bool load_rows = !RESIDENT || tile.row != resident, whole = t < plan.runs * plan.run + plan.rounds;
+                resident = tile.row;
+                if (load_rows) {
+                    if (whole) k_blocks(&map_w, yes, plan.wide);
+                    else k_blocks(&map_wu, yes, plan.cut);
+                } else {
+                    if (whole) k_blocks(&map_w, no, plan.wide);
+                    else k_blocks(&map_wu, no, plan.cut);
                 }
             }
         }
@@ -542,22 +642,63 @@ __global__ void __launch_bounds__(256) unpack_w4_kernel(const uint4 *__restrict_
     qvggt_unpack_w4_item(packed, out, i);
 }
 
-template <int BN, bool DUMP>
-cudaError_t launch_tiles(const qvggt_weights *w, const signed char *wq8, const signed char *Xq8, const float *a_scale, int M, void *Y, long long ldy,
-                   int *acc_debug, cudaStream_t st, long long wait_limit, int skip_loads)
+// Whole tiles first, as many as every worker gets alike, and what remains (less than a round of them) cut into pieces as narrow as one more
+// round allows: a K-block costs about 0.27 us at 256 channels, 0.2 at 128 (K = 4096, N = 1024: 32.8 -> 29.9 us at 10 992 rows, 14.6 -> 11.8
+// at 2748; cut in halves only, or not at all, before).
+// With resident token rows the whole tiles are dealt in runs of four.  Longer runs save more loads, but the chip's stores then
+// scatter over more rows of the result, which costs DRAM more than the loads do; N = 4096, us at 10 992 / 43 968 / 137 400 rows, runs of
+// 1: 37.9 / 135.7 / 412, 2: 37.6 / 138.5 / 418, 4: 35.1 / 129.5 / 397, 8: 36.5 / 140 / 437, 16: 38.0 / 142 / 439 (without the L2 policy
+// of the stores).
+Plan make_plan(int M, int N, int K, int max_workers, int *workers)
 {
-    using L = Lay<BN>;
+    const bool resident = K == RES_KB * BK;
+    Plan p = {};
+    p.row_tiles = (M - 1) / (2 * BM) + 1;
+    p.NU = N / UNIT;
+    p.NT = (p.NU + MAX_UNITS - 1) / MAX_UNITS;
+    p.narrow = p.NU / p.NT;
+    p.wider = p.NU % p.NT;
+    p.wide = p.narrow + (p.wider ? 1 : 0);
+    p.div_nt = Plan::reciprocal(p.NT);
+    const int tiles = p.row_tiles * p.NT;
+    p.run = resident ? RUN : 1;
+    p.runs = tiles / (p.run * max_workers);
+    const int each = tiles / max_workers, first = each * max_workers, j = first % p.NT;
+    p.rounds = each - p.runs * p.run;
+    p.behind_row = first / p.NT;
+    p.behind_unit = j * p.narrow + (j < p.wider ? j : p.wider);
+    int pieces = 0;
+    for (p.cut = 1;; ++p.cut) {
+        p.behind_first = (p.NU - p.behind_unit + p.cut - 1) / p.cut;
+        p.behind_pieces = (p.NU + p.cut - 1) / p.cut;
+        pieces = p.behind_first + (p.row_tiles - 1 - p.behind_row) * p.behind_pieces;
+        if (pieces <= max_workers || p.cut == p.wide) break;
+    }
+    p.div_pieces = Plan::reciprocal(p.behind_pieces);
+    *workers = p.workers = each == 0 ? pieces : max_workers;
+    const int widest = each == 0 ? p.cut : p.wide;
+    p.stage_bytes = (resident ? 0 : A_BYTES) + widest * UNIT_BYTES;
+    const int fit = (OPS_BYTES - (resident ? RES_KB * A_BYTES : 0)) / p.stage_bytes, most = resident ? RES_KB : MAX_STAGES;
+    p.stages = fit < most ? fit : most;
+    return p;
+}
+
+template <bool RESIDENT, bool DUMP>
+cudaError_t launch_plan(const qvggt_weights *w, const signed char *wq8, const signed char *Xq8, const float *a_scale, int M, void *Y, long long ldy,
+                        int *acc_debug, cudaStream_t st, long long wait_limit, int skip_loads)
+{
     static QvggtPerDevice cache;
-    int max_workers = 0;
-    cudaError_t e = qvggt_configure_kernel(gemm_c8_kernel<BN, DUMP>, THREADS, L::DYN_SMEM, 2, cache, &max_workers);
+    int workers = 0;
+    cudaError_t e = qvggt_configure_kernel(gemm_c8_kernel<RESIDENT, DUMP>, THREADS, DYN_SMEM, 2, cache, &workers);
     if (e != cudaSuccess) return e;
     const int K = w->K, N = w->N;
-    CUtensorMap map_x, map_w;
+    const Plan plan = make_plan(M, N, K, workers, &workers);
+    CUtensorMap map_x, map_w, map_wu, map_y;
     if (!qvggt_make_map(&map_x, CU_TENSOR_MAP_DATA_TYPE_UINT8, Xq8, K, M, K, BK, BM, CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !qvggt_make_map(&map_w, CU_TENSOR_MAP_DATA_TYPE_UINT8, wq8, K, N, K, BK, L::B_ROWS, CU_TENSOR_MAP_SWIZZLE_128B))
+        !qvggt_make_map(&map_w, CU_TENSOR_MAP_DATA_TYPE_UINT8, wq8, K, N, K, BK, plan.wide * (UNIT / 2), CU_TENSOR_MAP_SWIZZLE_128B) ||
+        !qvggt_make_map(&map_wu, CU_TENSOR_MAP_DATA_TYPE_UINT8, wq8, K, N, K, BK, plan.cut * (UNIT / 2), CU_TENSOR_MAP_SWIZZLE_128B) ||
+        !qvggt_make_map(&map_y, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, Y, N, M, (uint64_t)ldy * 2, UNIT, 16, CU_TENSOR_MAP_SWIZZLE_128B))
         return cudaErrorInvalidValue;
-    const int total_tiles = ((M + 2 * BM - 1) / (2 * BM)) * ((N + BN - 1) / BN);
-    const int workers = total_tiles < max_workers ? total_tiles : max_workers;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
@@ -566,34 +707,20 @@ cudaError_t launch_tiles(const qvggt_weights *w, const signed char *wq8, const s
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(workers * 2);
     cfg.blockDim = dim3(THREADS);
-    cfg.dynamicSmemBytes = L::DYN_SMEM;
+    cfg.dynamicSmemBytes = DYN_SMEM;
     cfg.stream = st;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, gemm_c8_kernel<BN, DUMP>, map_x, map_w, static_cast<uint16_t *>(Y), ldy, a_scale, (const float *)w->w_scale,
-                              (const uint16_t *)w->bias, acc_debug, M, N, K, w->status, wait_limit, skip_loads);
-}
-
-// Whether tiles of 256 channels are the faster ones for this shape.  A narrow tile takes 0.55 of a wide one's time per K-block
-// (0.15 against 0.27 us) and half its epilogue, so the number of rounds decides: narrow tiles win while they need at most 1.5
-// times as many (wide / narrow, us: K = 4096, N = 1024: 13.4 / 9.4 at 1374 rows, 22.9 / 20.1 at 5496, but 24.0 / 26.1 at 8244,
-// 32.9 / 33.8 at 10 992), and with K = 1024, where the epilogue behind the last K-block weighs as much as the K-blocks, also when
-// they turn a single round into two (N = 1024: 7.0 / 5.4 at 1374 rows, 7.5 / 7.0 at 2748; two rounds into four: N = 3072
-// 10.7 / 11.5 at 2748 rows).
-bool wide_tiles(int M, int N, int K, int workers)
-{
-    const long long row_tiles = (M + 2 * BM - 1) / (2 * BM);
-    const long long wide = (row_tiles * ((N + 255) / 256) + workers - 1) / workers;
-    const long long narrow = (row_tiles * ((N + 127) / 128) + workers - 1) / workers;
-    return !(2 * narrow <= 3 * wide || (K == 1024 && wide == 1));
+    return cudaLaunchKernelEx(&cfg, gemm_c8_kernel<RESIDENT, DUMP>, map_x, map_w, map_wu, map_y, plan, a_scale,
+                              (const float *)w->w_scale, (const uint16_t *)w->bias, acc_debug, M, N, K, w->status, wait_limit, skip_loads);
 }
 
 template <bool DUMP>
 cudaError_t launch(const qvggt_weights *w, const signed char *wq8, const signed char *Xq8, const float *a_scale, int M, void *Y, long long ldy,
                    int *acc_debug, cudaStream_t st, long long wait_limit, int skip_loads)
 {
-    if (wide_tiles(M, w->N, w->K, qvggt_sm_count() / 2)) return launch_tiles<256, DUMP>(w, wq8, Xq8, a_scale, M, Y, ldy, acc_debug, st, wait_limit, skip_loads);
-    return launch_tiles<128, DUMP>(w, wq8, Xq8, a_scale, M, Y, ldy, acc_debug, st, wait_limit, skip_loads);
+    if (w->K == RES_KB * BK) return launch_plan<true, DUMP>(w, wq8, Xq8, a_scale, M, Y, ldy, acc_debug, st, wait_limit, skip_loads);
+    return launch_plan<false, DUMP>(w, wq8, Xq8, a_scale, M, Y, ldy, acc_debug, st, wait_limit, skip_loads);
 }
 
 }  // namespace

@@ -310,6 +310,10 @@ __device__ __forceinline__ void cluster_sync()   // every thread of every CTA in
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+// The same in two halves, with room for work between them.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+
 // The same meeting without any ordering of memory: for the way out, where it only keeps a CTA's shared memory alive until its peer
 // is done.  (The release form waits for the outstanding global stores of the whole epilogue first, about 0.5 us.)
 __device__ __forceinline__ void cluster_sync_relaxed()
@@ -408,6 +412,21 @@ __device__ __forceinline__ void tma_store_2d(const void *tmap, uint32_t smem_src
 {
     asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group [%0, {%1, %2}], [%3];" ::"l"(tmap), "r"(x), "r"(y),
                  "r"(smem_src)
+                 : "memory");
+}
+
+// The same for results that no kernel near will read again: first to leave L2.
+__device__ __forceinline__ uint64_t policy_evict_first()
+{
+    uint64_t policy;
+    asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+    return policy;
+}
+
+__device__ __forceinline__ void tma_store_2d(const void *tmap, uint32_t smem_src, int x, int y, uint64_t policy)
+{
+    asm volatile("cp.async.bulk.tensor.2d.global.shared::cta.bulk_group.L2::cache_hint [%0, {%1, %2}], [%3], %4;" ::"l"(tmap), "r"(x), "r"(y),
+                 "r"(smem_src), "l"(policy)
                  : "memory");
 }
 
