@@ -508,6 +508,7 @@ colmax_kernel(const uint16_t *__restrict__ A, int rows_a, int grid_a, const uint
 {
     using G = RowGeom<K>;
     extern __shared__ float smem[];                              // [ROWS][PADDED]
+    ptx::grid_launch_dependents();
     const int slot = threadIdx.x / G::T;
     const int t = threadIdx.x % G::T;
     const bool first = (int)blockIdx.x < grid_a;
@@ -541,6 +542,8 @@ __global__ void multipliers_kernel(const float *__restrict__ c, const signed cha
                                    float *__restrict__ wmul, const uint16_t *__restrict__ bias, int N, uint16_t *__restrict__ bias_out,
                                    int *__restrict__ status)
 {
+    ptx::grid_launch_dependents();
+    ptx::grid_dependency_wait();
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (status && k == 0) *status = 0;
     if (bias_out && k < N) bias_out[k] = bias[k];
@@ -572,6 +575,8 @@ __global__ void __launch_bounds__(1024) max_reduce_kernel(const float *__restric
 __global__ void smooth_finalize_kernel(const float *__restrict__ ax, const float *__restrict__ aw, int K, float alpha,
                                        float lo, float hi, float *__restrict__ c)
 {
+    ptx::grid_launch_dependents();
+    ptx::grid_dependency_wait();
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= K) return;
     float x = ax[k], w = aw[k], r;
@@ -593,12 +598,32 @@ int rsq_grid(int M, int rows_per_cta, int ctas_per_sm = 6)
 
 }  // namespace
 
+// The small kernels of a load (column maxima -> smoothing factors -> multipliers -> codes) are a chain of launches of 1 - 10 us: each may
+// become resident while the one in front drains, and waits for its memory before touching any.
+namespace {
+
+template <class... Args>
+cudaError_t launch_chained(void (*kernel)(Args...), int grid, int block, cudaStream_t st, Args... args)
+{
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+}  // namespace
+
 cudaError_t qvggt_launch_multipliers(const float *c, const signed char *v, int K, float *amul, float *wmul, cudaStream_t st,
                                      const uint16_t *bias, int N, uint16_t *bias_out, int *status)
 {
     const int n = (bias_out && N > K) ? N : K;
-    multipliers_kernel<<<(n + 255) / 256, 256, 0, st>>>(c, v, K, amul, wmul, bias, N, bias_out, status);
-    return cudaGetLastError();
+    return launch_chained(multipliers_kernel, (n + 255) / 256, 256, st, c, v, K, amul, wmul, bias, N, bias_out, status);
 }
 
 namespace {
@@ -771,6 +796,5 @@ cudaError_t qvggt_launch_colmax(const void *A, int rows_a, const void *B, int ro
 cudaError_t qvggt_launch_smooth_finalize(const float *ax, const float *aw, int K, float alpha, float lo, float hi,
                                          float *c, cudaStream_t st)
 {
-    smooth_finalize_kernel<<<(K + 255) / 256, 256, 0, st>>>(ax, aw, K, alpha, lo, hi, c);
-    return cudaGetLastError();
+    return launch_chained(smooth_finalize_kernel, (K + 255) / 256, 256, st, ax, aw, K, alpha, lo, hi, c);
 }
