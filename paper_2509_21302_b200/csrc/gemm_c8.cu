@@ -187,8 +187,7 @@ gemm_c8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
     ptx::tc_fence_after_sync();
     const uint32_t tmem_base = *s_tmem;
     // Everything up to grid_dependency_wait() touches only kernel parameters and on-chip state: it may overlap the tail of the previous
-    // kernel in the stream; the operands and the output buffer may not be touched before that kernel is done.  (The MMA thread touches
-    // neither: it waits for what the producers load.)
+    // kernel in the stream; the operands, the output buffer and the status word may not be touched before that kernel is done.
     ptx::grid_launch_dependents();
 
     if (warp < EPI_WARPS) {
@@ -265,6 +264,7 @@ gemm_c8_kernel(const __grid_constant__ CUtensorMap map_x, const __grid_constant_
         // the descriptors in uniform registers, where tcgen05 wants them (behind `lane == 0` every one is moved there anew, which
         // made this loop, at 545 cycles per K-block, the bound of the kernel).
         if (rank == 0 && ptx::elect_one()) {
+            ptx::grid_dependency_wait();                                   // the limit of its waits bounds this kernel's own work only
             bool alive = true;
             StageRing r(ring);
             int left = my_tiles * KB - plan.stages;                        // K-blocks for whose stage a load will wait

@@ -58,3 +58,39 @@ def test_starved_gemm_reports_a_timeout_and_leaves_the_context_usable(M, N):
     assert np.array_equal(acc.cpu().numpy(), ref["acc"])
     assert np.array_equal(host_bits(Y2), ref["y"])
     h2.free()
+
+
+def test_limits_do_not_run_while_the_previous_kernel_does():
+    """A launch becomes resident while the previous kernel of the stream still runs (here a starved one on four
+    pairs of SMs): its limited waits must only begin when that one is done.  Both launches load nothing."""
+    import time
+
+    import paper_2509_21302_b200 as q
+    q.build()
+    M = N = 256
+    for K in (1024, 4096):
+        spec = workload.LinearSpec("starved", K, N, workload.DIST_NORMAL, 78, 0)
+        W, b = spec.weight(), spec.bias()
+        c = torch.from_numpy(oracle.smooth_factors(spec.x_calib(64), W)).cuda()
+        first, second = (q.prepare_weights(dev_bf16(W), dev_bf16(b), c, None, c8="only") for _ in range(2))
+        X8 = torch.ones((M, K), dtype=torch.int8, device="cuda")
+        a = torch.ones((M,), dtype=torch.float32, device="cuda")
+        Y = torch.full((M, N), -3.0, dtype=torch.bfloat16, device="cuda")
+        code = ctypes.c_int(0)
+        assert first.device_status() == 0 and second.device_status() == 0
+        side, done = torch.cuda.Stream(), torch.cuda.Event()
+        side.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(side):
+            assert q.debug_starved_linear_c8(first, X8, a, Y, 400_000_000) == 0      # at least 0.2 s
+            assert q.debug_starved_linear_c8(second, X8, a, Y, 1_000_000) == 0       # about 0.5 ms, once it is its turn
+            done.record()
+        time.sleep(0.05)
+        status = q.lib().qvggt_device_status(second.handle, torch.cuda.current_stream().cuda_stream, ctypes.byref(code))
+        assert not done.query(), "the first launch was to be still running"
+        assert (status, code.value) == (0, 0), "a wait of the second launch ran out while the first one was running"
+        side.synchronize()
+        assert torch.all(Y == -3.0)
+        for h in (first, second):
+            assert q.lib().qvggt_device_status(h.handle, side.cuda_stream, ctypes.byref(code)) == ERR_DEVICE_TIMEOUT
+            assert code.value in (DEV_TIMEOUT_FULL, DEV_TIMEOUT_ACCUM)
+            h.free()
