@@ -96,9 +96,10 @@ __device__ __forceinline__ void finish_16x64(const uint32_t (&raw)[32], const ui
 
 // The same with the parameters of the thread's channels in registers (w2[b]: the scales of channels 8 b + 2 (lane mod 4) and + 1, cb[b]:
 // their bf16 biases), and a TMA store of the staging tile (128-byte swizzle, the same layout), which clips the rows beyond the tensor.
-// (x, y): channel and row of the 16 x 64; nothing is stored unless `issue`.
+// (x, y): channel and row of the 16 x 64; nothing is stored unless `issue`.  reused: an earlier store may still be reading the tile.
 __device__ __forceinline__ void finish_16x64_tma(const uint32_t (&raw)[32], const uint64_t (&as2)[2], const uint64_t (&w2)[8], const uint32_t (&cb)[8],
-                                                 uint32_t stg_addr, const void *map_y, int x, int y, bool issue, int lane, uint64_t one2, uint64_t policy)
+                                                 uint32_t stg_addr, bool reused, const void *map_y, int x, int y, bool issue, int lane, uint64_t one2,
+                                                 uint64_t policy)
 {
     uint32_t out[16];
 #pragma unroll
@@ -114,8 +115,10 @@ __device__ __forceinline__ void finish_16x64_tma(const uint32_t (&raw)[32], cons
         }
     }
     const uint32_t st_row = stg_addr + (lane & 15) * 128;
-    if (lane == 0) ptx::tma_store_wait_read<0>();
-    __syncwarp();                           // the previous 16 rows have left the staging tile
+    if (reused) {
+        if (lane == 0) ptx::tma_store_wait_read<0>();
+        __syncwarp();                       // the previous 16 rows have left the staging tile
+    }
 #pragma unroll
     for (int b = 0; b < 8; b += 2)          // matrices (rows 0-7, block b), (rows 8-15, b), (0-7, b + 1), (8-15, b + 1)
         ptx::stmatrix_x4(st_row + (((b + (lane >> 4)) ^ (lane & 7)) << 4), out[2 * b], out[2 * b + 1], out[2 * b + 2], out[2 * b + 3]);
