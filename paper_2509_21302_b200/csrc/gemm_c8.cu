@@ -655,8 +655,18 @@ __global__ void __launch_bounds__(256) unpack_w4_kernel(const uint4 *__restrict_
 }
 
 // Whole tiles first, as many as every worker gets alike, and what remains (less than a round of them) cut into pieces as narrow as one more
-// round allows: a K-block costs about 0.27 us at 256 channels, 0.2 at 128 (K = 4096, N = 1024: 32.8 -> 29.9 us at 10 992 rows, 14.6 -> 11.8
-// at 2748; cut in halves only, or not at all, before).
+// round allows: a launch of one round at K = 4096 takes 8.0 us with tiles of 64 channels, 8.2 - 8.7 with 128, 11.2 with 192 and 13.5 with 256
+// (K = 4096, N = 1024: 32.8 -> 29.9 us at 10 992 rows, 13.7 -> 11.2 at 2748; cut in halves only, or not at all, before).
+// A launch of nothing but pieces takes those of 64 channels only where they leave half of the chip free.  They gain 0.25 us over 128
+// channels at most, and the blocks of the quantize launch behind this one, let in while it runs, crowd on the SMs that it leaves.
+// Layers in a replayed graph, us with 64 / 128 channels (n: pieces of 64 on 74 pairs of SMs):
+//   K = 1024: N = 1024, 204 - 219 rows (n = 16) 5.5 / 5.8, 455 - 492 (32) 5.9 / 6.0 - 6.15, 666 - 759 (48) 7.0 / 6.4, 964 - 996 (64) 7.15 / 6.9;
+//             N = 3072 (48), 141 - 195 rows 5.65 / 5.8, 222 - 256 6.04 / 5.9; N = 4096 (64), 174 - 230 rows 6.55 / 5.95
+//   K = 4096: N = 1024, 192 - 209 rows (16) 10.26 / 10.52, 260 - 300 (32) 11.1 / 11.2, 369 - 458 (32) 11.95 / 11.4, 793 - 931 (64) 12.8 - 13.8 / 13.0 - 13.2;
+//             N = 3072 (48) 12.1 / 11.3; N = 4096 (64) 12.3 / 11.4
+// and the mean over 260 layers, 64 against 128 channels, K = 1024 / 4096: up to n = 24 0.972 / 0.986, 25 - 37 0.979 / 1.014, 38 - 49
+// 1.026 / 1.020, 50 - 74 1.04 / 1.07.  Behind whole tiles, where the chip is busy anyway, the narrowest win at any number (K = 4096, N = 1024, 7975
+// rows 50.8 / 52.4).
 // With resident token rows the whole tiles are dealt in runs of four.  Longer runs save more loads, but the chip's stores then
 // scatter over more rows of the result, which costs DRAM more than the loads do; N = 4096, us at 10 992 / 43 968 / 137 400 rows, runs of
 // 1: 37.9 / 135.7 / 412, 2: 37.6 / 138.5 / 418, 4: 35.1 / 129.5 / 397, 8: 36.5 / 140 / 437, 16: 38.0 / 142 / 439 (without the L2 policy
@@ -684,7 +694,8 @@ Plan make_plan(int M, int N, int K, int max_workers, int *workers)
         p.behind_first = (p.NU - p.behind_unit + p.cut - 1) / p.cut;
         p.behind_pieces = (p.NU + p.cut - 1) / p.cut;
         pieces = p.behind_first + (p.row_tiles - 1 - p.behind_row) * p.behind_pieces;
-        if (pieces <= max_workers || p.cut == p.wide) break;
+        const bool crowding = p.cut == 1 && each == 0 && 2 * pieces > max_workers;
+        if ((pieces <= max_workers && !crowding) || p.cut == p.wide) break;
     }
     p.div_pieces = Plan::reciprocal(p.behind_pieces);
     *workers = p.workers = each == 0 ? pieces : max_workers;
