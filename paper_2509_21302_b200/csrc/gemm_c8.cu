@@ -678,6 +678,10 @@ Plan make_plan(int M, int N, int K, int max_workers, int *workers)
     p.row_tiles = (M - 1) / (2 * BM) + 1;
     p.NU = N / UNIT;
     p.NT = (p.NU + MAX_UNITS - 1) / MAX_UNITS;
+    // Where N is no multiple of 256, tiles of 128 channels may fit two rounds although those of up to 256 are just more than one, and two such
+    // rounds cost less than one of 256 and one of 64 (layers, us, 256 + 64 / 128 + 128: K = 4096, N = 1152, 3867 rows 34.2 / 31.1, N = 640, 6500 rows
+    // 42.3 / 39.0; K = 1024 11.55 / 11.16 and 12.95 / 12.55; three or more rounds: K = 1024, N = 1152, 8100 rows 17.35 / 17.7).
+    if (p.row_tiles * p.NT > max_workers && p.row_tiles * (p.NU / 2) <= 2 * max_workers) p.NT = p.NU / 2;
     p.narrow = p.NU / p.NT;
     p.wider = p.NU % p.NT;
     p.wide = p.narrow + (p.wider ? 1 : 0);

@@ -23,6 +23,7 @@ pytestmark = pytest.mark.gpu
     (4096, 384, 20000),              # tiles of three units, then pieces of one
     (4096, 1024, 256 * 37 + 1),      # two full rounds and one row tile
     (4096, 1024, 2748), (4096, 896, 4700), (4096, 128, 256 * 74 + 9),
+    (4096, 640, 6500), (1024, 1152, 3867),     # two rounds of 128 channels where 256 are just more than one
     (1024, 1024, 513), (1024, 1024, 400),      # nothing but pieces: of 128 channels (48 of 64 would not leave half of the chip), of 64
 ])
 def test_tiles(K, N, M):
