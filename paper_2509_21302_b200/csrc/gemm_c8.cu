@@ -657,8 +657,8 @@ __global__ void __launch_bounds__(256) unpack_w4_kernel(const uint4 *__restrict_
 // Whole tiles first, as many as every worker gets alike, and what remains (less than a round of them) cut into pieces as narrow as one more
 // round allows: a launch of one round at K = 4096 takes 8.0 us with tiles of 64 channels, 8.2 - 8.7 with 128, 11.2 with 192 and 13.5 with 256
 // (K = 4096, N = 1024: 32.8 -> 29.9 us at 10 992 rows, 13.7 -> 11.2 at 2748; cut in halves only, or not at all, before).
-// A launch of nothing but pieces takes those of 64 channels only where they leave half of the chip free.  They gain 0.25 us over 128
-// channels at most, and the blocks of the quantize launch behind this one, let in while it runs, crowd on the SMs that it leaves.
+// A launch of nothing but pieces takes those of 64 channels only where they leave half of the chip free, at K = 4096 two thirds.  They gain
+// 0.25 us over 128 channels at most, and the blocks of the quantize launch behind this one, let in while it runs, crowd on the SMs that it leaves.
 // Layers in a replayed graph, us with 64 / 128 channels (n: pieces of 64 on 74 pairs of SMs):
 //   K = 1024: N = 1024, 204 - 219 rows (n = 16) 5.5 / 5.8, 455 - 492 (32) 5.9 / 6.0 - 6.15, 666 - 759 (48) 7.0 / 6.4, 964 - 996 (64) 7.15 / 6.9;
 //             N = 3072 (48), 141 - 195 rows 5.65 / 5.8, 222 - 256 6.04 / 5.9; N = 4096 (64), 174 - 230 rows 6.55 / 5.95
@@ -698,7 +698,7 @@ Plan make_plan(int M, int N, int K, int max_workers, int *workers)
         p.behind_first = (p.NU - p.behind_unit + p.cut - 1) / p.cut;
         p.behind_pieces = (p.NU + p.cut - 1) / p.cut;
         pieces = p.behind_first + (p.row_tiles - 1 - p.behind_row) * p.behind_pieces;
-        const bool crowding = p.cut == 1 && each == 0 && 2 * pieces > max_workers;
+        const bool crowding = p.cut == 1 && each == 0 && (resident ? 2 : 3) * pieces > max_workers;
         if ((pieces <= max_workers && !crowding) || p.cut == p.wide) break;
     }
     p.div_pieces = Plan::reciprocal(p.behind_pieces);
