@@ -182,10 +182,13 @@ cudaError_t dispatch(const qvggt_weights *w, const void *Xq, const void *Wq, con
 // below one round of tiles.  What decides is the layer, the quantize launch and the GEMM behind it: the persistent kernels hide more of
 // their start behind the quantize launch, so alone and back to back this kernel would win for longer than it does in a layer.
 // Layers in a replayed graph (us, this kernel / the other one), each line between the first and the second M:
-//   one code per byte   K = 1024: N = 128, M = 1536 6.8 / 7.1, M = 3072 9.9 / 7.7; N = 1024, M = 192 6.1 / 5.9, M = 257 6.8 / 5.9;
-//                                 N = 3072, M = 64 5.6 / 5.9, M = 85 6.8 / 5.9; N = 4096, M = 48 5.7 / 5.9, M = 96 7.8 / 6.3
-//                       K = 4096: N = 128, M = 512 10.0 / 12.0, M = 1024 16.7 / 12.9; N = 640, M = 153 10.4 / 10.4, M = 204 13.2 / 10.4;
-//                                 N = 1024, M = 96 9.7 / 10.6, M = 128 11.7 / 11.0; N = 4096, M = 24 9.4 / 11.4, M = 32 11.0 / 10.3
+//   one code per byte   K = 1024: N = 256, M = 384 5.4 / 5.5, M = 576 6.4 / 5.9; N = 640, M = 128 5.0 / 5.4, M = 153 5.8 / 5.4;
+//                                 N = 1024, M = 96 5.4 / 5.4, M = 192 6.0 / 5.5; N = 2048, M = 80 5.5 / 5.8, M = 96 5.7 / 5.6, M = 160 7.1 / 5.8;
+//                                 N = 3072, M = 58 5.5 / 6.05, M = 69 6.4 / 5.8; N = 4096, M = 48 5.5 / 5.9, M = 56 6.4 / 5.9; N = 128 within
+//                                 10 % either way from M = 512 to 2048.  Up to 96 rows the outputs decide at 3 * 2^16, beyond at half of that
+//                       K = 4096: N = 128, M = 576 10.1 / 11.8, M = 640 11.9 / 11.8, M = 768 13.3 / 11.9; N = 384, M = 213 10.2 / 10.2, M = 256 11.1 / 10.2;
+//                                 N = 640, M = 153 10.1 / 10.1, M = 166 10.8 / 10.1; N = 1024, M = 96 9.6 / 10.1, M = 112 10.3 / 10.15;
+//                                 N = 4096, M = 24 9.3 / 11.1, M = 32 10.75 / 10.4
 //   packed              K = 1024: N = 128, M = 6144 12.6 / 13.5, M = 8232 15.6 / 15.1; N = 3072, M = 256 9.1 / 9.3, M = 343 11.2 / 9.6
 //                       K = 4096: N = 1024, M = 384 17.8 / 19.5, M = 514 21.4 / 21.6; N = 4096, M = 96 16.2 / 19.9, M = 128 20.3 / 18.8
 //   group scales        K = 1024: N = 1024, M = 384 8.5 / 9.0, M = 514 9.6 / 8.9; N = 4096, M = 96 8.2 / 8.2, M = 128 9.1 / 8.3
@@ -194,8 +197,8 @@ cudaError_t dispatch(const qvggt_weights *w, const void *Xq, const void *Wq, con
 bool qvggt_gemm_small_wins(const qvggt_weights *w, int M, bool packed, bool grouped)
 {
     const long long outputs = (long long)M * w->N;
-    if (w->K == 1024) return outputs <= (packed ? 3LL << 18 : grouped ? 3LL << 17 : 3LL << 16);
-    return outputs <= (packed ? 3LL << 17 : grouped ? 9LL << 14 : 3LL << 15);
+    if (w->K == 1024) return outputs <= (packed ? 3LL << 18 : grouped ? 3LL << 17 : M <= 96 ? 3LL << 16 : 3LL << 15);
+    return outputs <= (packed ? 3LL << 17 : grouped ? 9LL << 14 : w->N < 640 ? 5LL << 14 : 3LL << 15);
 }
 
 cudaError_t qvggt_launch_gemm_small(const qvggt_weights *w, const void *Xq, const void *Wq, bool packed, const float *a_scale, bool grouped, int M,

@@ -59,7 +59,7 @@ def test_row_tiles(K, N, M):
 
 # M on the last size of the kernel and the first of the other one, for each of the rule's lines
 @pytest.mark.parametrize("K,N,lines", [(1024, 1024, (192, 384, 768)), (1024, 3072, (64, 128, 256)), (4096, 1024, (96, 128, 144, 192, 384)),
-                                         (4096, 512, (192, 288, 768))])
+                                         (4096, 512, (192, 288, 768)), (1024, 1024, (96,)), (1024, 512, (192,)), (4096, 512, (160,)), (4096, 640, (153,))])
 def test_both_sides_of_the_rule(K, N, lines):
     for line in lines:
         for M in (line, line + 1):
