@@ -4,8 +4,7 @@
 // tcgen05 has no 4-bit integer kind: whatever the storage format, the tensor core multiplies int8.  Here the
 // producers already emit one code per byte (the quantize kernel for the activations, the offline weight
 // preparation for the weights), so the tiles go from global memory straight into the 128-byte-swizzled operand
-// stages by TMA and nothing in this kernel touches an operand byte with an ordinary instruction.  Per K-block
-// a CTA's shared memory sees one TMA write and one tensor-core read of its 32 KB of operands, the minimum.
+// stages by TMA and nothing in this kernel touches an operand byte with an ordinary instruction.
 //
 // Persistent and warp-specialised; a worker is a pair of CTAs on neighbouring SMs (tile 256 tokens x up to 256 channels, each CTA stages
 // 128 token rows and half of the tile's weight rows; one thread of the leader CTA issues tcgen05.mma.cta_group::2.kind::i8 for both;
@@ -18,9 +17,10 @@
 // parameters from shared memory for every 16 rows and wrote 128-byte lines with ordinary stores):
 //  - At 256 channels the MMAs of a K-block take 512 cycles and its 32 KB per CTA take as long from L2 (64 bytes per cycle and SM), so with
 //    K = 1024, where a tile's outputs are another 8 KB per K-block, the traffic of the SM was the limit.  With K = 1024 the eight
-//    K-blocks of the token rows (128 KB) stay in shared memory for RUN consecutive tiles and only weights stream.
+//    K-blocks of the token rows (128 KB) stay in shared memory for as long as a worker's tiles share them, and only weights stream: in runs of
+//    four tiles where every worker gets at least four (make_plan()).  Calls with fewer share nothing; what they gained is due to the next points.
 //  - The epilogue shares the shared-memory pipe with the operands: parameters in registers, outputs through the TMA engine.
-//  - The outputs are marked first to leave L2 (default policy: 35.1 instead of 31.9 at N = 4096).
+//  - The outputs are marked first to leave L2, see ptx::policy_evict_first().
 //  - Tiles that do not fill a round of workers are cut into narrower ones (make_plan()).
 //   K = 1024, N = 3072 / 1024 / 4096 and K = 4096, N = 1024 at 10 992 rows: 27.4 / 13.0 / 36.8 / 32.8 -> 24.8 / 11.3 / 31.9 / 29.9;
 //   at 137 400 rows K = 1024, N = 4096: 432 -> 394 (at the power limit).
@@ -31,6 +31,7 @@
 
 #include <type_traits>
 
+#include "gemm_c8_plan.cuh"
 #include "gemm_common.cuh"
 #include "qvggt_internal.cuh"
 #include "sm100_ptx.cuh"
@@ -39,13 +40,10 @@
 
 namespace {
 
+using namespace gemm_c8;
 using gemmc::Ring;
 using gemmc::STG_BYTES;
 
-constexpr int BM = 128;            // token rows per CTA (TMEM lanes)
-constexpr int BK = 128;            // codes along K per stage = one 128-byte swizzled row
-constexpr int UNIT = 64;           // channels per unit of work; a tile is 256 token rows x 1 .. 4 units
-constexpr int MAX_UNITS = 4;
 constexpr int ACC_BUFS = 2;        // TMEM accumulators: the epilogue of tile i overlaps the MMAs of tile i+1
 constexpr int ACC_COLS = MAX_UNITS * UNIT;
 constexpr int EPI_WARPS = 8;       // warp w: TMEM lane quarter w % 4, part w / 4 of the tile
@@ -54,15 +52,9 @@ constexpr int TMA_WARP = EPI_WARPS + 1;
 constexpr int THREADS = (EPI_WARPS + 2) * 32;
 constexpr int TMEM_COLS = ACC_BUFS * ACC_COLS;
 
-constexpr int A_BYTES = BM * BK;                       // one K-block of a CTA's token rows: 16 KB
-constexpr int UNIT_BYTES = UNIT / 2 * BK;              // one K-block of a CTA's half of a unit's weight rows: 4 KB
-constexpr int RES_KB = 8;                              // K-blocks of the token rows that stay resident (K = 1024)
-constexpr int RUN = 4;                                 // consecutive tiles of a worker that share them, see make_plan()
 constexpr int STG_WARP = 16 * 2 * UNIT;                // staging of one epilogue warp: 16 rows x 64 bf16, 128-byte swizzled
 constexpr int OFF_OPS = EPI_WARPS * STG_WARP;          // operands: [resident token rows,] ring of stages (1024-byte aligned)
-constexpr int OPS_BYTES = 208 * 1024;
 static_assert(EPI_WARPS * 4 * STG_WARP <= OPS_BYTES, "the last tile is staged where the operands were");
-constexpr int MAX_STAGES = 12;
 constexpr int OFF_BAR = OFF_OPS + OPS_BYTES;           // full[MAX_STAGES] empty[MAX_STAGES] tfull[2] tempty[2]
 constexpr int NBARS = 2 * MAX_STAGES + 2 * ACC_BUFS;
 constexpr int OFF_TMEM = OFF_BAR + NBARS * 8;
@@ -70,62 +62,6 @@ constexpr int OFF_ABORT = OFF_TMEM + 4;
 constexpr int DYN_SMEM = OFF_ABORT + 4 + 1024;         // slack to align the base to 1024 bytes
 static_assert(DYN_SMEM <= 232448, "exceeds the 227 KB of shared memory a CTA may use");
 static_assert(2 * (A_BYTES + MAX_UNITS * UNIT_BYTES) < (1 << 20), "transaction count of a stage must fit the barrier");
-
-// How the tiles are dealt to the workers; filled in by make_plan(), so that no thread of the kernel divides.  Work is counted in units of 256
-// token rows x 64 channels; whole tiles are numbered along the channels, row tile by row tile.
-struct Plan {
-    int NU, NT;                  // units and whole tiles of a row tile: NT tiles of `narrow` units, the first `wider` of them one unit more
-    int narrow, wider, wide;     // wide: most units of a whole tile
-    int runs, run;               // each worker first takes `runs` times `run` consecutive tiles,
-    int rounds;                  // then so many single tiles,
-    int cut;                     // then at most one piece of `cut` units
-    int workers, row_tiles;
-    int behind_row, behind_unit, behind_first, behind_pieces;   // where the pieces begin, how many the begun row tile has, how many a row tile has
-    unsigned long long div_nt, div_pieces;                      // see div()
-    int stages, stage_bytes;
-    // x / d for x d < 2^40, with m = ceil(2^40 / d)
-    static __host__ __device__ unsigned long long reciprocal(int d) { return ((1ull << 40) + d - 1) / d; }
-    static __host__ __device__ __forceinline__ int div(int x, unsigned long long m) { return (int)((x * m) >> 40); }
-};
-
-// The tiles of one worker, in order.
-struct Tiles {
-    int row, unit, units;                                 // the current tile: row tile, first unit, how many units
-    int count;                                            // of tiles
-    __device__ __forceinline__ Tiles(const Plan &plan, int worker_) : row(0), unit(0), units(0), worker(worker_), t(0), p(plan)
-    {
-        // behind the whole tiles: what is left of a row tile, then whole row tiles
-        const int i = worker - p.behind_first, full = i < 0 ? 0 : Plan::div(i, p.div_pieces);
-        behind_row = p.behind_row + (i < 0 ? 0 : 1 + full);
-        behind_unit = i < 0 ? p.behind_unit + worker * p.cut : (i - full * p.behind_pieces) * p.cut;
-        count = p.runs * p.run + p.rounds + (behind_row < p.row_tiles ? 1 : 0);
-        at = worker * p.run;
-        in_run = 0;
-        next();
-    }
-    __device__ __forceinline__ void next()     // (one beyond the last is never used)
-    {
-        const int in_runs = p.runs * p.run;
-        if (t < in_runs + p.rounds) {
-            if (t >= in_runs) at = in_runs * p.workers + (t - in_runs) * p.workers + worker;
-            row = Plan::div(at, p.div_nt);
-            const int j = at - row * p.NT;
-            unit = j * p.narrow + min(j, p.wider);
-            units = p.narrow + (j < p.wider ? 1 : 0);
-            ++at;
-            if (++in_run == p.run) { in_run = 0; at += (p.workers - 1) * p.run; }
-        } else {
-            row = behind_row;
-            unit = behind_unit;
-            units = min(p.cut, p.NU - unit);
-        }
-        ++t;
-    }
-
-private:
-    int worker, t, at, in_run, behind_row, behind_unit;
-    const Plan &p;
-};
 
 // A position in the ring of operand stages together with the parity of the phase it is in.
 struct StageRing {
@@ -652,62 +588,6 @@ __global__ void __launch_bounds__(256) unpack_w4_kernel(const uint4 *__restrict_
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n16) return;
     qvggt_unpack_w4_item(packed, out, i);
-}
-
-// Whole tiles first, as many as every worker gets alike, and what remains (less than a round of them) cut into pieces as narrow as one more
-// round allows: a launch of one round at K = 4096 takes 8.0 us with tiles of 64 channels, 8.2 - 8.7 with 128, 11.2 with 192 and 13.5 with 256
-// (K = 4096, N = 1024: 32.8 -> 29.9 us at 10 992 rows, 13.7 -> 11.2 at 2748; cut in halves only, or not at all, before).
-// A launch of nothing but pieces takes those of 64 channels only where they leave half of the chip free, at K = 4096 two thirds.  They gain
-// 0.25 us over 128 channels at most, and the blocks of the quantize launch behind this one, let in while it runs, crowd on the SMs that it leaves.
-// Layers in a replayed graph, us with 64 / 128 channels (n: pieces of 64 on 74 pairs of SMs):
-//   K = 1024: N = 1024, 204 - 219 rows (n = 16) 5.5 / 5.8, 455 - 492 (32) 5.9 / 6.0 - 6.15, 666 - 759 (48) 7.0 / 6.4, 964 - 996 (64) 7.15 / 6.9;
-//             N = 3072 (48), 141 - 195 rows 5.65 / 5.8, 222 - 256 6.04 / 5.9; N = 4096 (64), 174 - 230 rows 6.55 / 5.95
-//   K = 4096: N = 1024, 192 - 209 rows (16) 10.26 / 10.52, 260 - 300 (32) 11.1 / 11.2, 369 - 458 (32) 11.95 / 11.4, 793 - 931 (64) 12.8 - 13.8 / 13.0 - 13.2;
-//             N = 3072 (48) 12.1 / 11.3; N = 4096 (64) 12.3 / 11.4
-// and the mean over 260 layers, 64 against 128 channels, K = 1024 / 4096: up to n = 24 0.972 / 0.986, 25 - 37 0.979 / 1.014, 38 - 49
-// 1.026 / 1.020, 50 - 74 1.04 / 1.07.  Behind whole tiles, where the chip is busy anyway, the narrowest win at any number (K = 4096, N = 1024, 7975
-// rows 50.8 / 52.4).
-// With resident token rows the whole tiles are dealt in runs of four.  Longer runs save more loads, but the chip's stores then
-// scatter over more rows of the result, which costs DRAM more than the loads do; N = 4096, us at 10 992 / 43 968 / 137 400 rows, runs of
-// 1: 37.9 / 135.7 / 412, 2: 37.6 / 138.5 / 418, 4: 35.1 / 129.5 / 397, 8: 36.5 / 140 / 437, 16: 38.0 / 142 / 439 (without the L2 policy
-// of the stores).
-Plan make_plan(int M, int N, int K, int max_workers, int *workers)
-{
-    const bool resident = K == RES_KB * BK;
-    Plan p = {};
-    p.row_tiles = (M - 1) / (2 * BM) + 1;
-    p.NU = N / UNIT;
-    p.NT = (p.NU + MAX_UNITS - 1) / MAX_UNITS;
-    // Where N is no multiple of 256, tiles of 128 channels may fit two rounds although those of up to 256 are just more than one, and two such
-    // rounds cost less than one of 256 and one of 64 (layers, us, 256 + 64 / 128 + 128: K = 4096, N = 1152, 3867 rows 34.2 / 31.1, N = 640, 6500 rows
-    // 42.3 / 39.0; K = 1024 11.55 / 11.16 and 12.95 / 12.55; three or more rounds: K = 1024, N = 1152, 8100 rows 17.35 / 17.7).
-    if (p.row_tiles * p.NT > max_workers && p.row_tiles * (p.NU / 2) <= 2 * max_workers) p.NT = p.NU / 2;
-    p.narrow = p.NU / p.NT;
-    p.wider = p.NU % p.NT;
-    p.wide = p.narrow + (p.wider ? 1 : 0);
-    p.div_nt = Plan::reciprocal(p.NT);
-    const int tiles = p.row_tiles * p.NT;
-    p.run = resident ? RUN : 1;
-    p.runs = tiles / (p.run * max_workers);
-    const int each = tiles / max_workers, first = each * max_workers, j = first % p.NT;
-    p.rounds = each - p.runs * p.run;
-    p.behind_row = first / p.NT;
-    p.behind_unit = j * p.narrow + (j < p.wider ? j : p.wider);
-    int pieces = 0;
-    for (p.cut = 1;; ++p.cut) {
-        p.behind_first = (p.NU - p.behind_unit + p.cut - 1) / p.cut;
-        p.behind_pieces = (p.NU + p.cut - 1) / p.cut;
-        pieces = p.behind_first + (p.row_tiles - 1 - p.behind_row) * p.behind_pieces;
-        const bool crowding = p.cut == 1 && each == 0 && (resident ? 2 : 3) * pieces > max_workers;
-        if ((pieces <= max_workers && !crowding) || p.cut == p.wide) break;
-    }
-    p.div_pieces = Plan::reciprocal(p.behind_pieces);
-    *workers = p.workers = each == 0 ? pieces : max_workers;
-    const int widest = each == 0 ? p.cut : p.wide;
-    p.stage_bytes = (resident ? 0 : A_BYTES) + widest * UNIT_BYTES;
-    const int fit = (OPS_BYTES - (resident ? RES_KB * A_BYTES : 0)) / p.stage_bytes, most = resident ? RES_KB : MAX_STAGES;
-    p.stages = fit < most ? fit : most;
-    return p;
 }
 
 template <bool RESIDENT, bool DUMP>
