@@ -56,9 +56,8 @@ __device__ __forceinline__ void load_channel_params(float *s_ws, float *s_bs, co
 // fl(fl(float(acc) * fl(a_scale * w_scale)) + bias), every operation rounded to nearest, then bf16 (round to nearest even).
 // as2[h] holds a_scale of the thread's row lane / 4 + 8 h in both halves; ws / bs point at the 64 channel scales / biases.
 // The rows then go through 2 KB of the warp's shared memory (16-byte chunk q of a row at q XOR (row mod 8), free of bank
-// conflicts both ways) and from there to global memory as whole 128-byte lines.  Against one row per thread and a TMA store per
-// 32 x 32 tile this reads the channel parameters from shared memory a quarter as often and leaves the TMA engine, which
-// also feeds the operands, alone: 39.0 -> 36.6 us at M = 10 992, K = 1024, N = 4096, 14.0 -> 13.1 us at N = 1024.
+// conflicts both ways) and from there to global memory as whole 128-byte lines.  This is the packed kernel's form: its 18 warps have
+// 96 registers each, too few for the channel parameters of finish_16x64_tma(), which is the faster one where they fit.
 // Y points at row 0, channel 0 of the 16 x 64; only the first `rows` rows are stored.  one2: see ptx::f32x2_add_uncontracted.
 __device__ __forceinline__ void finish_16x64(const uint32_t (&raw)[32], const uint64_t (&as2)[2], const float *ws, const float *bs, unsigned char *stg,
                                              uint32_t stg_addr, uint16_t *__restrict__ Y, long long ldy, int rows, int lane,

@@ -415,7 +415,11 @@ __device__ __forceinline__ void tma_store_2d(const void *tmap, uint32_t smem_src
                  : "memory");
 }
 
-// The same for results that no kernel near will read again: first to leave L2.
+// The same with an L2 policy.  The GEMM on byte codes marks its results first to leave L2, so that they don't displace the operands of tiles
+// still to come, also where the next kernel reads them.  K = 1024, N = 4096, us with / without the policy: alone 33.2 / 40.5 at 10 992 rows,
+// 75.3 / 81.1 at 21 984, 442 / 485 at 137 400, equal up to 8244; together with a GELU + quantize launch on its result 19.05 / 19.0 at 1374 rows,
+// 39.2 / 39.0 at 4122, 78.0 / 77.1 at 8244, 98.4 / 98.4 at 10 992, 412 / 416 at 43 968, 1163 / 1179 at 137 400; a whole MLP 58.5 / 58.9 at 4122,
+// 109.1 / 109.3 at 8244, 140.3 / 142.4 at 10 992, 1630 / 1656 at 137 400.
 __device__ __forceinline__ uint64_t policy_evict_first()
 {
     uint64_t policy;

@@ -18,7 +18,10 @@ pytestmark = pytest.mark.gpu
     (1024, 128, 256 * 80 + 1),       # one tile of two units per row tile
     (1024, 384, 256 * 37),           # a whole number of rounds: no piece behind them
     (1024, 4096, 2600),              # two rounds, then pieces
-    (1024, 3072, 256 * 5 + 3),       # less than a round: one unit less than a tile each
+    (1024, 3072, 256 * 5 + 3),       # less than a round: 72 tiles of four units
+    (1024, 1024, 2748),              # less than a round: 66 pieces of three units
+    (1024, 4096, 4122),              # three tiles per worker, none of which share token rows, then pieces of three units
+    (1024, 1152, 256 * 120 + 5),     # two runs of four tiles, the second begins inside a row tile; no single tile behind them
     (1024, 640, 700), (4096, 640, 700),
     (4096, 384, 20000),              # tiles of three units, then pieces of one
     (4096, 1024, 256 * 37 + 1),      # two full rounds and one row tile
